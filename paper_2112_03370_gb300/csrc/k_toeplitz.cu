@@ -312,7 +312,7 @@ __device__ __forceinline__ void pair_meta(const TileArgs& a, int64_t g, int64_t 
 template <typename T, int MODE, int NB>
 __device__ __forceinline__ void gather_pairs(const TileArgs& a, int rhs, const TileDesc& td,
                                              const int64_t (&g)[NB], T (&v)[NB][2]) {
-  if constexpr (MODE == MODE_APPLY_T || MODE == MODE_NINV_T) {   // coalesced read of t, zero outside the block
+  if constexpr (MODE == MODE_APPLY_T) {   // coalesced read of t, zero outside the block
     const float* t = reinterpret_cast<const float*>(a.x) + rhs * a.x_stride;
 #pragma unroll
     for (int u = 0; u < NB; u++) {
@@ -387,12 +387,6 @@ __device__ __forceinline__ void scatter_pairs(const TileArgs& a, int rhs, const 
       if (p[u][1] >= 0) Map4<T>::add(a.y, rhs * a.y_stride, p[u][1], y1, c1 * y1, s1 * y1);
     }
   }
-}
-
-// Bulk prefetch of [p, p + bytes) into L2 (p and bytes multiples of 16; a hint, no completion to wait for).
-__device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "r"(bytes)
-               : "memory");
 }
 
 // ---- fused stride-1 passes and pair update (FP32 tiles) ----------------------------------------
@@ -573,17 +567,6 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile(const TileArgs a_in) {
         }
       }
       __syncthreads();
-      if constexpr (MODE == MODE_NINV_T && std::is_same<T, float>::value) {
-        // the next tile's new input samples [in0 + L, in0 + L + vstep) start on their way to L2 now,
-        // so its gather finds them there instead of waiting on DRAM
-        if (threadIdx.x == 0 && step + 1 < n_steps) {
-          int64_t lo = max(td.in0 + LT, td.blk_lo), hi = min(td.in0 + LT + (int64_t)seg.vstep, td.blk_hi);
-          lo = (lo + 3) & ~(int64_t)3;   // 16-byte aligned and inside the block
-          hi &= ~(int64_t)3;
-          if (hi > lo)
-            prefetch_l2_bulk(reinterpret_cast<const float*>(a.x) + rhs * a.x_stride + lo, (uint32_t)((hi - lo) * 4));
-        }
-      }
       if (step + 1 < n_steps) {   // keep input samples [vstep, L) for the next tile
         const int n0 = seg.vstep / 2;
         for (int n = threadIdx.x; n < 2 * halo_q; n += NT) {
@@ -707,21 +690,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile(const TileArgs a_in) {
       cl.sync();
       other = cl.map_shared_rank(sm, rank ^ 1);
     }
-    if constexpr (MODE == MODE_NINV_T && CL == 1) {
-      // y of the tile's output range, float pairs (g even, so 8-byte aligned inside the range)
-      float* yo = reinterpret_cast<float*>(a.y) + rhs * a.y_stride;
-      const int n_lo = r_lo >> 1, n_hi = (r_hi + 1) >> 1;
-      for (int n = n_lo + threadIdx.x; n < n_hi; n += NT) {
-        const C z = sm[smem_pad(n)];
-        const int64_t g = td.in0 + 2 * (int64_t)n;
-        if (g >= td.out_lo && g + 2 <= td.out_hi) {
-          __stcs(reinterpret_cast<float2*>(yo + g), make_float2(z.x, z.y));
-        } else {
-          if (g >= td.out_lo && g < td.out_hi) yo[g] = z.x;
-          if (g + 1 >= td.out_lo && g + 1 < td.out_hi) yo[g + 1] = z.y;
-        }
-      }
-    } else if constexpr (CL == 1) {
+    if constexpr (CL == 1) {
       constexpr int NB = 8;
       const int n_lo = r_lo >> 1, n_hi = (r_hi + 1) >> 1;
       for (int n0 = n_lo + threadIdx.x; n0 < n_hi; n0 += NB * NT) {
@@ -833,15 +802,15 @@ int tile_kernels_init() {
   static int status = MM_OK;
   if (done) return status;
   done = 1;
+  status = ninv32_init();
+  if (status != MM_OK) return status;
   cudaError_t e = cudaSuccess;
 #define MM_SET(K, B)                                                                       \
   if (e == cudaSuccess) e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(B));
   MM_SET((k_tile<float, 1, MODE_APPLY>), kSmemMax);
   MM_SET((k_tile<float, 1, MODE_RHS>), kSmemMax);
   MM_SET((k_tile<float, 1, MODE_APPLY, true>), kSmemMax);
-  MM_SET((k_tile<float, 1, MODE_NINV_T, true>), kSmemMax);
   MM_SET((k_tile<float, 1, MODE_APPLY_T>), kSmemMax);
-  MM_SET((k_tile<float, 1, MODE_NINV_T>), kSmemMax);
   MM_SET((k_tile<double, 2, MODE_APPLY>), kSmemBytes64);
   MM_SET((k_tile<double, 2, MODE_RHS>), kSmemBytes64);
   MM_SET((k_tile<double, 2, MODE_NINV>), kSmemBytes64);
@@ -895,7 +864,6 @@ cudaError_t launch_tiles_fp32(int mode, const TileArgs& a, int halo_samples, cud
   if (smem > kSmemMax) return cudaErrorInvalidValue;
   if (mode == MODE_APPLY) return launch_tiles<float, 1, MODE_APPLY>(a, smem, s);
   if (mode == MODE_APPLY_T) return launch_tiles<float, 1, MODE_APPLY_T>(a, smem, s);
-  if (mode == MODE_NINV_T) return launch_tiles<float, 1, MODE_NINV_T>(a, smem, s);
   if (mode == MODE_RHS) return launch_tiles<float, 1, MODE_RHS>(a, smem, s);
   return cudaErrorInvalidValue;
 }
@@ -947,12 +915,6 @@ cudaError_t launch_tiles_fp32_multi(const TileArgs& a, int halo_samples, cudaStr
   const size_t smem = kSmemBytes32 + (size_t)halo_samples * sizeof(float);
   if (smem > kSmemMax || a.nrhs != 1 || a.probs == nullptr) return cudaErrorInvalidValue;
   return launch_tiles<float, 1, MODE_APPLY, true>(a, smem, s);
-}
-
-cudaError_t launch_ninv32_multi(const TileArgs& a, int halo_samples, cudaStream_t s) {
-  const size_t smem = kSmemBytes32 + (size_t)halo_samples * sizeof(float);
-  if (smem > kSmemMax || a.nrhs != 1 || a.probs == nullptr) return cudaErrorInvalidValue;
-  return launch_tiles<float, 1, MODE_NINV_T, true>(a, smem, s);
 }
 
 int fp32_max_halo_samples() { return (int)((kSmemMax - kSmemBytes32) / sizeof(float)); }

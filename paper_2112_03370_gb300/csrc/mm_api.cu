@@ -200,7 +200,7 @@ void free_plan(Plan* P) {
   if (P->stream) cudaStreamSynchronize(P->stream);
   dfree(P->lpix); dfree(P->psi); dfree(P->w32); dfree(P->w64); dfree(P->obs_to_global); dfree(P->minv);
   dfree(P->band); dfree(P->block_off_dev); dfree(P->c0_blk); dfree(P->tab32); dfree(P->tab64);
-  dfree(P->tw32); dfree(P->tw64); dfree(P->tiles); dfree(P->segs); dfree(P->map32_in); dfree(P->map32_out);
+  dfree(P->tw32); dfree(P->tw64); dfree(P->tiles); dfree(P->segs); dfree(P->nsegs); dfree(P->ntab32); dfree(P->ntw32); dfree(P->map32_in); dfree(P->map32_out);
   dfree(P->map64_in); dfree(P->map64_out); dfree(P->td_a); dfree(P->td_b); dfree(P->t32);
   dfree(P->wdf); dfree(P->tabdf); dfree(P->twdf); dfree(P->tdf); dfree(P->mapdf);
   dfree(P->ang2); dfree(P->groups); dfree(P->slot); dfree(P->slot_pix); dfree(P->u32);
@@ -393,8 +393,36 @@ struct Scratch {
   }
 };
 
+// Tile size of k_ninv32 for these blocks: the least estimated time over 8192-, 16384- and 32768-sample
+// tiles.  A CTA's tile takes about 10.6, 11.5 and 13.5 us with 4, 2 and 1 CTAs per SM, whether or not
+// the SM is full (measured on GB300; 32768-sample tiles for lambda 8192, N 268M: 1.45 ms against 2.18
+// ms of the earlier shared-memory passes; 16384 for lambda 2048, N 16.8M: 64 us, 8192: 80, 32768: 81;
+// 8192 for lambda 1024, N 262144: 10 us, 32768: 18), so few tiles ask for small ones (one wave) and
+// many for the ones that keep the most outputs per unit of work.  shared: the tiles run in launches
+// together with other plans' (server), so the waves are not counted, only the work.
+int choose_ninv_logm(const std::vector<int64_t>& off, int lam, bool shared) {
+  int best = kNinvLogMax;
+  double best_t = 1e300;
+  const double us[3] = {10.6, 11.5, 13.5};
+  for (int logm = kNinvLogMax; logm >= kNinvLogMin; logm--) {
+    const int64_t vmax = ((int64_t)2 << logm) - 2 * (int64_t)lam - 4;
+    if (vmax <= 0) break;
+    int64_t n = 0;
+    for (size_t b = 0; b + 1 < off.size(); b++) n += (off[b + 1] - off[b] + vmax - 1) / vmax;
+    const int64_t slots = (int64_t)sm_count() << (kNinvLogMax - logm);
+    const double waves = shared ? (double)n / (double)slots : (double)((n + slots - 1) / slots);
+    const double t = waves * us[logm - kNinvLogMin];
+    if (t < best_t) {
+      best_t = t;
+      best = logm;
+    }
+  }
+  return best;
+}
+
 // FP32 segments of up to `steps` consecutive tiles (replacing previous ones: captured graphs
-// must be captured again)
+// must be captured again): of the fused tiles, and of k_ninv32 when it is built (at most 4 tiles there,
+// where walking only spares the twiddle tables)
 int build_segments(Plan* P, int steps, cudaStream_t s) {
   BandTables bt;
   bt.blk_tab = P->blk_tab;
@@ -410,6 +438,21 @@ int build_segments(Plan* P, int steps, cudaStream_t s) {
   P->tile_steps = std::max(1, steps);
   MM_TRY(dalloc(P, &P->segs, segs.size()));
   MM_CUDA(cudaMemcpyAsync(P->segs, segs.data(), segs.size() * sizeof(TileDesc), cudaMemcpyHostToDevice, s));
+  if (P->ninv_logm > 0) {
+    const int64_t len = (int64_t)2 << P->ninv_logm;
+    const int64_t slots = (int64_t)sm_count() << (kNinvLogMax - P->ninv_logm);
+    const int64_t n1 = (int64_t)make_tiles(P->block_off, bt, P->lambda, 1, 0, nullptr, len).size();
+    const int walk = P->steps_given ? std::max(1, steps) : (int)std::max<int64_t>(1, std::min<int64_t>(4, n1 / (8 * slots)));
+    P->nsegs_host = make_tiles(P->block_off, bt, P->lambda, walk, kL, nullptr, len);
+    if (P->nsegs) {
+      P->bytes -= (size_t)P->n_nsegs * sizeof(TileDesc);
+      dfree(P->nsegs);
+    }
+    P->n_nsegs = (int64_t)P->nsegs_host.size();
+    MM_TRY(dalloc(P, &P->nsegs, P->nsegs_host.size()));
+    MM_CUDA(cudaMemcpyAsync(P->nsegs, P->nsegs_host.data(), P->nsegs_host.size() * sizeof(TileDesc),
+                            cudaMemcpyHostToDevice, s));
+  }
   return MM_OK;
 }
 
@@ -741,6 +784,14 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
   MM_CUDA(cudaMemcpyAsync(P->tiles, tiles.data(), tiles.size() * sizeof(TileDesc), cudaMemcpyHostToDevice, s));
   P->blk_tab = bt.blk_tab;
   P->blk_scale = bt.blk_scale;
+  if (P->precision == MM_FP32 && windows && P->groups && !P->tc) {
+    P->ninv_logm = choose_ninv_logm(P->block_off, lam, P->no_big);
+    MM_TRY(dalloc(P, &P->ntab32, pair_table_reg_floats(P->ninv_logm, P->n_tab)));
+    MM_TRY(dalloc(P, &P->ntw32, twiddle_image_len(P->ninv_logm)));
+    MM_CUDA(launch_pair_table_reg(P->ninv_logm, H, P->n_tab, costab_d, P->ntab32, s));
+    MM_CUDA(launch_twiddle_image(P->ninv_logm, P->tw32, P->ntw32, s));
+  }
+  P->steps_given = d->tile_steps > 0;
   // FP32 segments: enough of them to keep every SM busy (about 8 per SM), at most 16 tiles each
   const int64_t steps = d->tile_steps > 0 ? d->tile_steps
                                            : std::max<int64_t>(1, std::min<int64_t>(16, P->n_tiles / (8 * sm_count())));
@@ -994,8 +1045,10 @@ int ninv32(Plan* P, const float* t, float* u, int64_t ts, int g, const int32_t* 
     MM_CUDA(launch_ninv32_big(a, s));
     return MM_OK;
   }
-  a.tiles = P->segs;
-  a.n_tiles = P->n_segs;
+  a.tiles = P->nsegs;
+  a.n_tiles = P->n_nsegs;
+  a.tab = P->ntab32;
+  a.tw = P->ntw32;
   a.nrhs = g;
   a.x = t;
   a.x_stride = ts;
@@ -1003,7 +1056,7 @@ int ninv32(Plan* P, const float* t, float* u, int64_t ts, int g, const int32_t* 
   a.y_stride = ts;
   a.done = done;
   a.done_stride = done_stride;
-  MM_CUDA(launch_tiles_fp32(MODE_NINV_T, a, P->seg_halo, s));
+  MM_CUDA(launch_ninv32(P->ninv_logm, a, s));
   return MM_OK;
 }
 
@@ -1392,12 +1445,12 @@ struct Server {
   int64_t n_wgroups = 0;
   WinProb* wprobs_dev = nullptr;
   size_t wprobs_cap = 0;
-  TileDesc* ntiles_dev = nullptr;
-  size_t ntiles_cap = 0;
-  int64_t n_ntiles = 0;
+  TileDesc* ntiles_dev[kNinvSizes] = {};   // one list (and launch) per tile size
+  size_t ntiles_cap[kNinvSizes] = {};
+  int64_t n_ntiles[kNinvSizes] = {};
+  const float2* ntw32[kNinvSizes] = {};    // twiddle image of a running plan with that tile size
   ProbPtrs* nprobs_dev = nullptr;
   size_t nprobs_cap = 0;
-  int nhalo = 0;
   const float2* tw32 = nullptr;    // twiddles of a running request's plan (the same in every plan)
   bool dirty = true;
 };
@@ -1523,12 +1576,13 @@ static int upload_list(const std::vector<T>& v, T*& dev, size_t& cap, cudaStream
 
 // combined launch lists and per-problem pointers of the running FP32 requests
 int rebuild_launch(Server* S) {
-  std::vector<TileDesc> tiles, ntiles;
+  std::vector<TileDesc> tiles, ntiles[kNinvSizes];
   std::vector<ProbPtrs> probs, nprobs;
   std::vector<PGroup> wgroups;
   std::vector<WinProb> wprobs;
-  int halo = 0, nhalo = 0;
+  int halo = 0;
   S->tw32 = nullptr;
+  for (const float2*& tw : S->ntw32) tw = nullptr;
   for (size_t i = 0; i < S->running.size(); i++) {
     Request* r = S->running[i];
     if (!r->fp32) continue;   // FP64-class requests run their own iterations
@@ -1550,11 +1604,13 @@ int rebuild_launch(Server* S) {
       }
       wprobs.push_back(WinProb{P->block_off_dev, P->slot, P->slot_pix, P->ang2, r->cg->p32, P->t32, P->u32,
                                r->cg->q32, halt});
-      for (TileDesc td : P->segs_host) {
+      const int sz = P->ninv_logm - kNinvLogMin;
+      S->ntw32[sz] = P->ntw32;
+      for (TileDesc td : P->nsegs_host) {
         td.prob = (int32_t)nprobs.size();
-        ntiles.push_back(td);
+        ntiles[sz].push_back(td);
       }
-      nhalo = std::max(nhalo, (int)P->seg_halo);
+      pp.tab = P->ntab32;
       pp.x = P->t32;
       pp.y = P->u32;
       nprobs.push_back(pp);
@@ -1571,15 +1627,16 @@ int rebuild_launch(Server* S) {
   }
   MM_TRY(upload_list(tiles, S->tiles_dev, S->tiles_cap, S->stream));
   MM_TRY(upload_list(probs, S->probs_dev, S->probs_cap, S->stream));
-  MM_TRY(upload_list(ntiles, S->ntiles_dev, S->ntiles_cap, S->stream));
+  for (int k = 0; k < kNinvSizes; k++) {
+    MM_TRY(upload_list(ntiles[k], S->ntiles_dev[k], S->ntiles_cap[k], S->stream));
+    S->n_ntiles[k] = (int64_t)ntiles[k].size();
+  }
   MM_TRY(upload_list(nprobs, S->nprobs_dev, S->nprobs_cap, S->stream));
   MM_TRY(upload_list(wgroups, S->wgroups_dev, S->wgroups_cap, S->stream));
   MM_TRY(upload_list(wprobs, S->wprobs_dev, S->wprobs_cap, S->stream));
   MM_CUDA(cudaStreamSynchronize(S->stream));   // host vectors go out of scope
   S->n_tiles = (int64_t)tiles.size();
   S->halo = halo;
-  S->n_ntiles = (int64_t)ntiles.size();
-  S->nhalo = nhalo;
   S->n_wgroups = (int64_t)wgroups.size();
   S->dirty = false;
   return MM_OK;
@@ -1589,13 +1646,15 @@ int rebuild_launch(Server* S) {
 int enqueue_multi_apply(Server* S, cudaStream_t s) {
   if (S->n_wgroups > 0) {
     MM_CUDA(launch_unpoint_win32_multi(S->wgroups_dev, S->n_wgroups, S->wprobs_dev, s));
-    TileArgs a{};
-    a.tiles = S->ntiles_dev;
-    a.n_tiles = S->n_ntiles;
-    a.nrhs = 1;
-    a.tw = S->tw32;
-    a.probs = S->nprobs_dev;
-    MM_CUDA(launch_ninv32_multi(a, S->nhalo, s));
+    for (int k = 0; k < kNinvSizes; k++) {
+      TileArgs a{};
+      a.tiles = S->ntiles_dev[k];
+      a.n_tiles = S->n_ntiles[k];
+      a.nrhs = 1;
+      a.tw = S->ntw32[k];
+      a.probs = S->nprobs_dev;
+      MM_CUDA(launch_ninv32(kNinvLogMin + k, a, s));
+    }
     MM_CUDA(launch_point_win32_multi(S->wgroups_dev, S->n_wgroups, S->wprobs_dev, s));
   }
   if (S->n_tiles > 0) {
@@ -2311,6 +2370,7 @@ int mm_autotune(mm_plan_t plan, int max_width, mm_tune_info* out, void* stream) 
   const int steps_c[] = {1, 2, 4, 8, 16, 32};
   double best = 1e300;
   int best_steps = P->tile_steps;
+  P->steps_given = true;
   for (int v : steps_c) {
     if (v > 1 && P->n_tiles / v < sm_count()) continue;   // fewer segments than SMs
     MM_TRY(build_segments(P, v, P->stream));
@@ -3247,7 +3307,8 @@ void mm_server_destroy(mm_server_t server) {
   for (auto& kv : S->all) delete kv.second;
   if (S->tiles_dev) cudaFree(S->tiles_dev);
   if (S->probs_dev) cudaFree(S->probs_dev);
-  if (S->ntiles_dev) cudaFree(S->ntiles_dev);
+  for (TileDesc* t : S->ntiles_dev)
+    if (t) cudaFree(t);
   if (S->nprobs_dev) cudaFree(S->nprobs_dev);
   if (S->wgroups_dev) cudaFree(S->wgroups_dev);
   if (S->wprobs_dev) cudaFree(S->wprobs_dev);

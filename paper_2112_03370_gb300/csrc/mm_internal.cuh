@@ -56,8 +56,8 @@ struct ProbPtrs {
 
 // MODE_APPLY_T: A-application whose un-pointed input t = P x was written beforehand (FP32
 // tiles: float t; df64 tiles: (hi, lo) float pairs, also used for the masked TOD of the RHS)
-// MODE_NINV_T: FP32 y = N^-1 t on the segments, float t in and float y out (the pointing is
-// applied by the window kernels around it)
+// MODE_NINV_T: y = N^-1 t alone (the pointing is applied by the window kernels around it), of the
+// df64 tiles and the FP32 65536-sample tiles; the other FP32 tiles are k_ninv32
 enum Mode { MODE_APPLY = 0, MODE_RHS = 1, MODE_NINV = 2, MODE_APPLY_T = 3, MODE_NINV_T = 4 };
 
 // ---------------------------------------------------------------------------------------------
@@ -205,6 +205,14 @@ struct Plan {
   std::vector<TileDesc> segs_host;     // host copy (multi-problem launches)
   std::vector<int32_t> blk_tab;        // host: spectrum table of each block
   std::vector<double> blk_scale;       // host: band scale of each block against its table
+  // FP32 N^-1 between the window kernels (k_ninv32): tiles of 2^(ninv_logm + 1) samples
+  int ninv_logm = 0;                   // 0: not built
+  TileDesc* nsegs = nullptr;
+  int64_t n_nsegs = 0;
+  std::vector<TileDesc> nsegs_host;    // host copy (multi-problem launches)
+  float* ntab32 = nullptr;             // pair tables of every band table
+  float2* ntw32 = nullptr;             // twiddle image
+  bool steps_given = false;            // the caller or the autotuner chose tile_steps
   int32_t tile_steps = 0;              // FP32 tiles walked per segment
   int32_t win_samples = 32768;         // target samples per pixel-window group
   int32_t tuned_width = 0;             // block width chosen by mm_autotune (0: not tuned)
@@ -350,9 +358,18 @@ cudaError_t launch_ninv32_big(const TileArgs& a, cudaStream_t s);
 cudaError_t launch_tiles_fp32(int mode, const TileArgs& a, int halo_samples, cudaStream_t s);
 // FP32 A-application over the tiles of several plans at once (a.probs set, nrhs = 1)
 cudaError_t launch_tiles_fp32_multi(const TileArgs& a, int halo_samples, cudaStream_t s);
-// u = N^-1 t of several problems' segments in one launch (a.probs: x = t, y = u, tab, done of
-// each problem; nrhs 1)
-cudaError_t launch_ninv32_multi(const TileArgs& a, int halo_samples, cudaStream_t s);
+// FP32 u = N^-1 t on register-transform tiles of 2^(logm + 1) samples, logm 12, 13 or 14
+// (k_ninv32.cu): t and u [nrhs][stride], a.tab from launch_pair_table_reg, a.tw from
+// launch_twiddle_image; with a.probs the segments of several problems (x = t, y = u, tab, done of
+// each; nrhs 1)
+constexpr int kNinvLogMin = 12, kNinvLogMax = 14, kNinvSizes = kNinvLogMax - kNinvLogMin + 1;
+cudaError_t launch_ninv32(int logm, const TileArgs& a, cudaStream_t s);
+size_t twiddle_image_len(int logm);   // float2 values
+cudaError_t launch_twiddle_image(int logm, const float2* tw, float2* out, cudaStream_t s);
+size_t pair_table_reg_floats(int logm, int32_t n_tab);
+cudaError_t launch_pair_table_reg(int logm, const double* H, int32_t n_tab, const double* costab, float* out,
+                                  cudaStream_t s);
+int ninv32_init();
 // t [nrhs][t_stride] float32 = P x for every sample (0 at masked samples), x float4 maps
 // [nrhs][n_obs]
 cudaError_t launch_unpoint32(const int32_t* lpix, const float2* w32, int64_t N, const float* x4,
