@@ -93,10 +93,10 @@ enum { MM_PREC_BD = 0, MM_PREC_2LVL_POST = 1 };
  *   inputs_on_device  non-zero: pix, psi and band are device pointers; zero: host pointers.
  *   tile_steps     FP32 operators: overlap-save tiles walked by one CTA, which keeps the overlap
  *                  of consecutive tiles in shared memory (0 = chosen from the problem size).
- *   pt_sub         FP32 operators, the reduction of P^T: 0 = per-sample sums per pixel in shared
- *                  memory over the pixel windows; 4096, 8192 or 16384 = segment reduction over
- *                  pixel-sorted sub-windows of at most that many samples (runs of equal pixels
- *                  summed in registers; the plan stores the sorted order, 8 more bytes per sample).
+ *   pt_sub         FP32 operators, the reduction of P^T: 0 = run sums over the pixel-sorted window
+ *                  groups, added to the map run by run; 4096, 8192 or 16384 = segment reduction over
+ *                  pixel-sorted sub-windows of at most that many samples into per-group sums in
+ *                  shared memory (the plan stores another sorted order, 8 more bytes per sample).
  *                  Other values: MM_EINVAL.  mm_autotune times both forms.
  */
 typedef struct {
@@ -248,8 +248,8 @@ int mm_solve_tod(mm_plan_t plan, const void* d, int d_is_fp32, double* x, int nr
  *      consecutive tiles in shared memory, more segments keep more SMs busy); for lambda > 6144,
  *      also 65536-sample tiles split over 2-CTA clusters (more of each tile kept, but every CTA
  *      reads the whole tile);
- *   2. target samples per pixel-window group of P and P^T (8192 ... 65536);
- *   2b. the P^T reduction: per-sample shared-memory sums over the windows, or segment reduction
+ *   2. target samples per pixel-window group of P and P^T (2048 ... 16384);
+ *   2b. the P^T reduction: run sums over the sorted groups, or segment reduction
  *      over pixel-sorted sub-windows of at most 4096, 8192 or 16384 samples;
  *   3. block width for mm_block_cg_solve with block_width = 0: the widest of 1, 2, 4, ..., max_width
  *      whose device time per column of A X is within 2% of the best.

@@ -8,9 +8,9 @@
 // its pixel among the sorted distinct pixels of its group (a uint16 slot), so
 //   P:   a CTA loads the group's map entries once into shared memory and every sample reads its
 //        (I, Q, U) from there;
-//   P^T: a CTA sums the group's samples per slot in shared memory and then adds each pixel's sum
-//        to the global map with one vector atomic, instead of one global atomic per sample (the
-//        local reduction before the global one of Sect. 3.1).
+//   P^T: the group's samples, ordered by slot once at plan time, are summed run by run in registers
+//        and each run is added to the global map with one vector atomic (the local reduction before
+//        the global one of Sect. 3.1).
 // The weights (cos 2psi, sin 2psi) are evaluated in registers from the angle 2psi reduced to
 // [-pi, pi] once at plan time in FP64, so the kernels stream 6 bytes of pointing per sample
 // (slot + angle) instead of a pixel index and two precomputed weights.
@@ -43,6 +43,23 @@ __device__ __forceinline__ void group_chunk(const PGroup& G, const int64_t* __re
   len = n > 0 ? (int)n : 0;
 }
 
+// Units of work of a group: its chunks, cut into pieces of 2^log_u samples (at least 128) when there
+// are fewer chunks than the CTA has warps, so that a group of few detectors and a long window still
+// uses every warp.
+__device__ __forceinline__ int unit_log(const PGroup& G, int warps) {
+  int lu = G.log_w;
+  while (lu > 7 && (G.n_blk << (G.log_w - lu)) < warps) lu--;
+  return lu;
+}
+__device__ __forceinline__ void group_unit(const PGroup& G, const int64_t* __restrict__ block_off, int unit, int lu,
+                                           int64_t& lo, int& len) {
+  const int ls = G.log_w - lu;
+  group_chunk(G, block_off, unit >> ls, lo, len);
+  const int o = (unit & ((1 << ls) - 1)) << lu;
+  lo += o;
+  len = max(0, min(len - o, 1 << lu));
+}
+
 // Insert p into the set (bounded probing); returns the position, or -1 when the set is full.
 __device__ __forceinline__ int set_insert(int32_t* keys, int32_t p, int* count) {
   uint32_t h = hash_of(p);
@@ -67,6 +84,16 @@ __device__ __forceinline__ int set_find(const int32_t* keys, int32_t p) {
     h = (h + 1) & (kHash - 1);
   }
   return -1;
+}
+
+// Slot of the k-th smallest of a group's n pixels.  The lanes of a warp hold samples some pixels
+// apart, along a sky row or across rows, so the ranks that one warp-wide access touches are often a
+// multiple of 8 apart (a square focal plane scanned across its rows: 128); the low three bits of the
+// rank are mixed with the higher ones so that such strides spread over the eight 16-byte bank groups
+// (map windows read 19.6 shared wavefronts per 32 samples without it, 16 x 16 detectors, half of the
+// intervals scanning along y).  A bijection on [0, n): the last partial group of 8 stays.
+__device__ __forceinline__ int slot_of_rank(int k, int n) {
+  return k < (n & ~7) ? (k & ~7) | ((k ^ (k >> 3) ^ (k >> 6) ^ (k >> 9)) & 7) : k;
 }
 
 // (cos x, sin x) for x in [-pi, pi] (the plan's reduced 2 psi)
@@ -99,10 +126,11 @@ __global__ void __launch_bounds__(kWinThreads) k_win_build(const PGroup* __restr
   }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int c = warp; c < G.n_blk; c += kWarps) {
+  const int lu = unit_log(G, kWarps), n_units = G.n_blk << (G.log_w - lu);
+  for (int c = warp; c < n_units; c += kWarps) {
     int64_t lo;
     int len;
-    group_chunk(G, block_off, c, lo, len);
+    group_unit(G, block_off, c, lu, lo, len);
     for (int o = lane; o < len; o += 32) {
       const int32_t p = __ldg(lpix + lo + o);
       if (p < 0) continue;
@@ -146,15 +174,16 @@ __global__ void __launch_bounds__(kWinThreads) k_win_build(const PGroup* __restr
   }
   for (int k = threadIdx.x; k < n; k += kWinThreads) {
     const int32_t p = sorted[k];
-    slot_pix[G.slot_off + k] = p;
+    const int sl = slot_of_rank(k, n);
+    slot_pix[G.slot_off + sl] = p;
     const int h = set_find(keys, p);
-    if (h >= 0) rank_of[h] = (uint16_t)k;
+    if (h >= 0) rank_of[h] = (uint16_t)sl;
   }
   __syncthreads();
-  for (int c = warp; c < G.n_blk; c += kWarps) {
+  for (int c = warp; c < n_units; c += kWarps) {
     int64_t lo;
     int len;
-    group_chunk(G, block_off, c, lo, len);
+    group_unit(G, block_off, c, lu, lo, len);
     for (int o = lane; o < len; o += 32) {
       const int32_t p = __ldg(lpix + lo + o);
       uint16_t r = kNoSlot;
@@ -168,7 +197,6 @@ __global__ void __launch_bounds__(kWinThreads) k_win_build(const PGroup* __restr
 }
 
 constexpr size_t kBuildSmem = (size_t)kHash * 4 + (size_t)kWinCap * 4 + (size_t)kHash * 2;
-constexpr size_t kUnpointSmem = (size_t)(kWinCap + kWinCap / 8) * sizeof(float4);
 
 #define MM_TRY_CUDA(expr)             \
   do {                                \
@@ -199,6 +227,107 @@ cudaError_t launch_win_build(const PGroup* groups, int64_t n_groups, const int64
   return cudaGetLastError();
 }
 
+// ---- sorted entries of the groups (P^T by run sums) -------------------------------------------
+// One CTA per group: a counting sort of its kept samples by slot in shared memory, written out in
+// the interleaved blocks that k_point_sorted reads.
+__global__ void __launch_bounds__(kWinThreads) k_srt_build(const PGroup* __restrict__ groups,
+                                                           const int64_t* __restrict__ block_off,
+                                                           const uint16_t* __restrict__ slot,
+                                                           const float* __restrict__ ang2, uint16_t* __restrict__ ent,
+                                                           float* __restrict__ ent_ang,
+                                                           uint16_t* __restrict__ first_slot) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int32_t* off = reinterpret_cast<int32_t*>(smem_raw);                  // [kWinCap + 1] counts, then next positions
+  uint32_t* key = reinterpret_cast<uint32_t*>(off + kWinCap + 4);       // [kWinMaxSamples] slot << 16 | position
+  __shared__ int32_t warp_sum[kWarps];
+  const PGroup G = groups[blockIdx.x];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int row = srt_row(G.log_w), zero = G.n_blk * row;
+  const int lu = unit_log(G, kWarps), n_units = G.n_blk << (G.log_w - lu), ls = G.log_w - lu;
+  for (int i = tid; i <= kWinCap; i += kWinThreads) off[i] = 0;
+  __syncthreads();
+  for (int u = warp; u < n_units; u += kWarps) {
+    int64_t lo;
+    int len;
+    group_unit(G, block_off, u, lu, lo, len);
+    for (int o = lane; o < len; o += 32) {
+      const uint32_t s = slot[lo + o];
+      if (s != kNoSlot) atomicAdd(off + s, 1);
+    }
+  }
+  __syncthreads();
+  // exclusive scan of the counts: kWinCap / kWinThreads consecutive slots per thread
+  constexpr int kPer = kWinCap / kWinThreads;
+  int32_t c[kPer], sum = 0;
+#pragma unroll
+  for (int i = 0; i < kPer; i++) {
+    c[i] = off[tid * kPer + i];
+    sum += c[i];
+  }
+  int32_t inc = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  if (lane == 31) warp_sum[warp] = inc;
+  __syncthreads();
+  int32_t base = inc - sum, total = 0;
+  for (int w = 0; w < kWarps; w++) {
+    if (w < warp) base += warp_sum[w];
+    total += warp_sum[w];
+  }
+#pragma unroll
+  for (int i = 0; i < kPer; i++) {
+    off[tid * kPer + i] = base;
+    base += c[i];
+  }
+  __syncthreads();
+  for (int u = warp; u < n_units; u += kWarps) {
+    int64_t lo, lo0;
+    int len, len0;
+    group_unit(G, block_off, u, lu, lo, len);
+    group_chunk(G, block_off, u >> ls, lo0, len0);
+    const int pos0 = (u >> ls) * row + (int)(lo0 & 3) + (int)(lo - lo0);
+    for (int o = lane; o < len; o += 32) {
+      const uint32_t s = slot[lo + o];
+      if (s != kNoSlot) key[atomicAdd(off + s, 1)] = (s << 16) | (uint32_t)(pos0 + o);
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < G.n_srt * kSrtBlock; i += kWinThreads) {
+    const int b = i / kSrtBlock, l = (i / 32) % 32, e = i % 32;
+    uint32_t w = (uint32_t)zero;
+    float a = 0.f;
+    if (i < total) {
+      const uint32_t k = key[i], pos = k & 0xFFFFu;
+      w = pos | ((e > 0 && (key[i - 1] >> 16) != (k >> 16)) ? kSrtRun : 0u);
+      const int r = (int)pos / row;
+      int64_t lo;
+      int len;
+      group_chunk(G, block_off, r, lo, len);
+      a = __ldg(ang2 + lo + ((int)pos - r * row - (int)(lo & 3)));
+    }
+    const int64_t blk = (G.srt_off + b) * kSrtBlock;
+    ent[blk + (e / 8) * 256 + l * 8 + e % 8] = (uint16_t)w;
+    ent_ang[blk + (e / 4) * 128 + l * 4 + e % 4] = a;
+    if (e == 0) first_slot[(G.srt_off + b) * 32 + l] = i < total ? (uint16_t)(key[i] >> 16) : kNoSlot;
+  }
+}
+
+constexpr size_t kSrtBuildSmem = (size_t)(kWinCap + 4) * 4 + (size_t)kWinMaxSamples * 4;
+cudaError_t launch_srt_build(const PGroup* groups, int64_t n_groups, const int64_t* block_off, const uint16_t* slot,
+                             const float* ang2, uint16_t* ent, float* ent_ang, uint16_t* first_slot, cudaStream_t s) {
+  if (n_groups == 0) return cudaSuccess;
+  if (n_groups > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  static cudaError_t st = cudaSuccess;
+  static bool set = false;
+  MM_TRY_CUDA(smem_limit_once(k_srt_build, kSrtBuildSmem, st, set));
+  k_srt_build<<<(unsigned)n_groups, kWinThreads, kSrtBuildSmem, s>>>(groups, block_off, slot, ang2, ent, ent_ang,
+                                                                    first_slot);
+  return cudaGetLastError();
+}
+
 // ---- chunk walking shared by the un-point and point kernels ------------------------------------
 // A warp takes CPI = 32 / LPC chunks at a time, LPC = min(32, W / 4) lanes per chunk.  Inside a
 // chunk [lo, lo + len) the lanes walk aligned quads of 4 samples [a0, a1) (a0 = lo rounded up to
@@ -206,23 +335,23 @@ cudaError_t launch_win_build(const PGroup* groups, int64_t n_groups, const int64
 struct ChunkWalk {
   int lpc, cpi, sub, ql;
 };
-__device__ __forceinline__ ChunkWalk chunk_walk(const PGroup& G, int lane) {
+__device__ __forceinline__ ChunkWalk chunk_walk(int log_u, int lane) {
   ChunkWalk w;
-  w.lpc = G.log_w >= 7 ? 32 : (1 << (G.log_w - 2));
+  w.lpc = log_u >= 7 ? 32 : (1 << (log_u - 2));
   w.cpi = 32 / w.lpc;
   w.sub = lane / w.lpc;
   w.ql = lane % w.lpc;
   return w;
 }
 
-// Visit every sample of chunk c: f_quad(base, q4) for aligned quads (samples base + 4 q4 .. + 3),
-// f_one(i) for the single samples of the ragged ends.  Global sample indices are 64-bit.
+// Visit every sample of unit c (pieces of 2^lu samples): f_quad(base, q4) for aligned quads (samples
+// base + 4 q4 .. + 3), f_one(i) for the single samples of the ragged ends.  Global sample indices are 64-bit.
 template <typename FQ, typename F1>
-__device__ __forceinline__ void visit_chunk(const PGroup& G, const int64_t* __restrict__ block_off, int c,
-                                            const ChunkWalk& w, FQ f_quad, F1 f_one) {
+__device__ __forceinline__ void visit_unit(const PGroup& G, const int64_t* __restrict__ block_off, int c, int lu,
+                                           const ChunkWalk& w, FQ f_quad, F1 f_one) {
   int64_t lo;
   int len;
-  group_chunk(G, block_off, c, lo, len);
+  group_unit(G, block_off, c, lu, lo, len);
   if (len <= 0) return;
   const int64_t a0 = (lo + 3) & ~(int64_t)3;
   const int head = (int)min((int64_t)len, a0 - lo);
@@ -254,25 +383,84 @@ __device__ __forceinline__ void prefetch_chunk(const T* base, int64_t lo, int le
 template <typename T>
 __device__ __forceinline__ T ld_point(const T* p, bool keep) { return keep ? __ldg(p) : __ldcs(p); }
 
-// Padded shared-memory indices of slot k.  A lane holds 4 consecutive samples, so one warp-wide
+// Padded shared-memory index of slot k's accumulators.  A lane holds 4 consecutive samples, so one warp-wide
 // access touches slots about 4 x (pixels per sample) apart; one padding word per 32 scalar slots
-// (accumulators) or one padding float4 per 8 slots (map window) keeps strides of 1, 2, 4 and 8
-// slots in distinct banks.
+// keeps strides of 1, 2, 4 and 8 slots in distinct banks.
 __device__ __forceinline__ int acc_index(int k) { return k + (k >> 5); }
-__device__ __forceinline__ int win_index(int k) { return k + (k >> 3); }
 constexpr int kAccStride = kWinCap + kWinCap / 32;
-constexpr int kWinEntries = kWinCap + kWinCap / 8;
+
+// Rows of a group (one per detector chunk) in shared memory: first sample and length, 12 bytes a row.
+struct RowTab {
+  int64_t* lo;
+  int32_t* len;
+  __device__ RowTab(void* base, int dets) : lo(reinterpret_cast<int64_t*>(base)), len(reinterpret_cast<int32_t*>(lo + dets)) {}
+  __device__ __forceinline__ void load(const PGroup& G, const int64_t* __restrict__ block_off) {
+    for (int c = threadIdx.x; c < G.n_blk; c += blockDim.x) {
+      int64_t l;
+      int n;
+      group_chunk(G, block_off, c, l, n);
+      lo[c] = l;
+      len[c] = n;
+    }
+  }
+};
+static size_t row_tab_bytes(int dets) { return (size_t)dets * 12; }
+
+// Aligned quads of a group's rows: a warp takes 128 samples at a time, LPC = min(32, W / 4) lanes per
+// row, quad q of a row being samples [lo - lo % 4 + 4 q, + 4).  A row that does not start on a multiple
+// of 4 has one quad more, W / 4, which is visited apart.
+struct QuadWalk {
+  int lu, ls, lpc, cpi, sub, ql, n_units;
+};
+__device__ __forceinline__ QuadWalk quad_walk(const PGroup& G, int lane) {
+  QuadWalk w;
+  w.lu = min(G.log_w, 7);
+  w.ls = G.log_w - w.lu;
+  w.lpc = 1 << (w.lu - 2);
+  w.cpi = 32 / w.lpc;
+  w.sub = lane / w.lpc;
+  w.ql = lane % w.lpc;
+  w.n_units = G.n_blk << w.ls;
+  return w;
+}
+
+// The group's map entries into shared memory by asynchronous 16-byte copies: all gathers of a thread are
+// in flight at once (with loads through registers the fill took 34 of 175 us, 67M samples).
+__device__ __forceinline__ void fill_window(float4* win, const float4* __restrict__ x, const int32_t* __restrict__ pix,
+                                            int n_slots) {
+  constexpr int U = 8;
+  for (int k0 = threadIdx.x; k0 < n_slots; k0 += U * blockDim.x) {
+    int32_t p[U];
+#pragma unroll
+    for (int j = 0; j < U; j++) {
+      const int k = k0 + j * blockDim.x;
+      p[j] = k < n_slots ? __ldg(pix + k) : -1;
+    }
+#pragma unroll
+    for (int j = 0; j < U; j++)
+      if (p[j] >= 0)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(win + k0 + j * blockDim.x)),
+                     "l"(x + p[j])
+                     : "memory");
+  }
+}
 
 // t = P x over the windows: one CTA per group, the group's map entries of column r in shared
-// memory, then one coalesced pass over the group's samples.  MULTI: the group's problem (one
-// column) comes from probs[G.prob].
+// memory, then one coalesced pass over the group's samples, each lane's next slots and angles loaded
+// while it works on the current ones (and the first before the window is filled).  Bound by HBM:
+// 10 B per sample (slot 2, angle 4, t 4); 256 detectors x 4 x 65,536 samples: 144 us, 4.7 TB/s (175 us
+// before the window was filled by asynchronous copies, 4 x 65,536 samples: 55 -> 5 us).  MULTI: the group's problem (one column) comes from
+// probs[G.prob].
+constexpr int kUnpointThreads = 256;
 template <bool MULTI>
-__global__ void __launch_bounds__(kWinThreads, 3) k_unpoint_win32(
+__global__ void __launch_bounds__(kUnpointThreads, 6) k_unpoint_win32(
     const PGroup* __restrict__ groups, const int64_t* __restrict__ block_off,
     const uint16_t* __restrict__ slot, const int32_t* __restrict__ slot_pix, const float* __restrict__ ang2,
     const float4* __restrict__ x4, int64_t x_stride4, int nrhs, const int32_t* __restrict__ done,
-    int done_stride, float* __restrict__ t, int64_t t_stride, const WinProb* __restrict__ probs) {
-  extern __shared__ float4 win[];   // [kWinEntries], slot k at win_index(k)
+    int done_stride, float* __restrict__ t, int64_t t_stride, const WinProb* __restrict__ probs, WinSize size) {
+  extern __shared__ float4 win[];   // [size.slots], then the row table
+  RowTab rt(win + size.slots, size.dets);
   const PGroup G = groups[blockIdx.x];
   if constexpr (MULTI) {
     const WinProb& pp = probs[G.prob];
@@ -284,53 +472,88 @@ __global__ void __launch_bounds__(kWinThreads, 3) k_unpoint_win32(
     t = pp.t;
     done = pp.done;
   }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const ChunkWalk cw = chunk_walk(G, lane);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+  const QuadWalk w = quad_walk(G, lane);
   const bool keep = nrhs > 1;
+  rt.load(G, block_off);
+  __syncthreads();
   for (int r = 0; r < nrhs; r++) {
     if (done != nullptr && done[(int64_t)r * done_stride] != 0) continue;
     const float4* x = x4 + r * x_stride4;
     float* tr = t + r * t_stride;
-    __syncthreads();   // the previous column's window is no longer read
-    for (int k = threadIdx.x; k < G.n_slots; k += kWinThreads)
-      win[win_index(k)] = __ldg(x + __ldg(slot_pix + G.slot_off + k));
-    __syncthreads();
     auto value = [&](uint32_t sl, float a) -> float {
       if (sl == kNoSlot) return 0.f;
       float cs, sn;
       weights_of_angle(a, cs, sn);
-      const float4 m = win[win_index((int)sl)];
+      const float4 m = win[sl];
       return m.x + cs * m.y + sn * m.z;
     };
-    for (int c0 = warp * cw.cpi; c0 < G.n_blk; c0 += kWarps * cw.cpi) {
-      const int c = c0 + cw.sub;
-      if (c >= G.n_blk) continue;
-      if (c + kWarps * cw.cpi < G.n_blk) {
-        int64_t lo;
-        int len;
-        group_chunk(G, block_off, c + kWarps * cw.cpi, lo, len);
-        prefetch_chunk(slot, lo, len, cw);
-        prefetch_chunk(ang2, lo, len, cw);
+    // quad q of row c: its samples and the ones of them inside the row, [e0, e1); a sample outside it is a
+    // neighbouring row's (of any group: its slot is below size.slots too) or past the end (kNoSlot)
+    struct Quad {
+      int64_t i;
+      int e0, e1;
+      uint2 s;
+      float4 a;
+    };
+    auto load = [&](int c, int q, Quad& d) {
+      const int64_t lo = rt.lo[c];
+      const int a = (int)(lo & 3), end = a + rt.len[c];
+      d.i = lo - a + 4 * (int64_t)q;
+      d.e0 = q == 0 ? a : 0;
+      d.e1 = min(4, end - 4 * q);
+      if (d.e1 > d.e0) {
+        d.s = ld_point(reinterpret_cast<const uint2*>(slot + d.i), keep);
+        d.a = ld_point(reinterpret_cast<const float4*>(ang2 + d.i), keep);
       }
-      visit_chunk(
-          G, block_off, c, cw,
-          [&](int64_t a0, int q) {
-            const int64_t i = a0 + 4 * (int64_t)q;
-            const uint2 s2 = ld_point(reinterpret_cast<const uint2*>(slot + i), keep);
-            const float4 a = ld_point(reinterpret_cast<const float4*>(ang2 + i), keep);
-            float4 v;
-            v.x = value(s2.x & 0xFFFFu, a.x);
-            v.y = value(s2.x >> 16, a.y);
-            v.z = value(s2.y & 0xFFFFu, a.z);
-            v.w = value(s2.y >> 16, a.w);
-            __stcs(reinterpret_cast<float4*>(tr + i), v);
-          },
-          [&](int64_t i) { __stcs(tr + i, value(ld_point(slot + i, keep), ld_point(ang2 + i, keep))); });
+    };
+    auto emit = [&](const Quad& d) {
+      if (d.e1 <= d.e0) return;
+      float4 v;
+      v.x = value(d.s.x & 0xFFFFu, d.a.x);
+      v.y = value(d.s.x >> 16, d.a.y);
+      v.z = value(d.s.y & 0xFFFFu, d.a.z);
+      v.w = value(d.s.y >> 16, d.a.w);
+      if (d.e1 - d.e0 == 4) {
+        __stcs(reinterpret_cast<float4*>(tr + d.i), v);
+      } else {
+        if (d.e0 <= 0 && d.e1 > 0) __stcs(tr + d.i, v.x);
+        if (d.e0 <= 1 && d.e1 > 1) __stcs(tr + d.i + 1, v.y);
+        if (d.e0 <= 2 && d.e1 > 2) __stcs(tr + d.i + 2, v.z);
+        if (d.e0 <= 3 && d.e1 > 3) __stcs(tr + d.i + 3, v.w);
+      }
+    };
+    auto load_unit = [&](int u, Quad& d) {
+      d.e0 = d.e1 = 0;
+      if (u < w.n_units) load(u >> w.ls, ((u & ((1 << w.ls) - 1)) << (w.lu - 2)) + w.ql, d);
+    };
+    Quad cur, nxt;
+    const int step = warps * w.cpi;
+    int u = warp * w.cpi + w.sub;
+    load_unit(u, cur);
+    if (r > 0) __syncthreads();   // the previous column's window is no longer read
+    fill_window(win, x, slot_pix + G.slot_off, G.n_slots);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    for (; u < w.n_units; u += step) {
+      load_unit(u + step, nxt);
+      emit(cur);
+      cur = nxt;
+    }
+    for (int c = threadIdx.x; c < G.n_blk; c += blockDim.x) {   // the last quad of rows off a multiple of 4
+      if ((int)(rt.lo[c] & 3) + rt.len[c] > (1 << G.log_w)) {
+        load(c, 1 << (G.log_w - 2), cur);
+        emit(cur);
+      }
     }
   }
 }
+constexpr size_t kUnpointSmem = (size_t)kWinCap * sizeof(float4) + 512 * 12;   // most of any group
 
-cudaError_t launch_unpoint_win32(const PGroup* groups, int64_t n_groups, const int64_t* block_off,
+static int unpoint_threads(const WinSize& z) { return std::min(z.threads, kUnpointThreads); }
+static size_t unpoint_smem(const WinSize& z) { return (size_t)z.slots * sizeof(float4) + row_tab_bytes(z.dets); }
+
+cudaError_t launch_unpoint_win32(const PGroup* groups, int64_t n_groups, const WinSize& size, const int64_t* block_off,
                                  const uint16_t* slot, const int32_t* slot_pix, const float* ang2,
                                  const float* x4, int64_t x_stride, int nrhs, const int32_t* done,
                                  int done_stride, float* t, int64_t t_stride, cudaStream_t s) {
@@ -339,124 +562,175 @@ cudaError_t launch_unpoint_win32(const PGroup* groups, int64_t n_groups, const i
   static cudaError_t st = cudaSuccess;
   static bool set = false;
   MM_TRY_CUDA(smem_limit_once(k_unpoint_win32<false>, kUnpointSmem, st, set));
-  k_unpoint_win32<false><<<(unsigned)n_groups, kWinThreads, kUnpointSmem, s>>>(
+  k_unpoint_win32<false><<<(unsigned)n_groups, unpoint_threads(size), unpoint_smem(size), s>>>(
       groups, block_off, slot, slot_pix, ang2, reinterpret_cast<const float4*>(x4), x_stride / 4, nrhs, done,
-      done_stride, t, t_stride, nullptr);
+      done_stride, t, t_stride, nullptr, size);
   return cudaGetLastError();
 }
 
-cudaError_t launch_unpoint_win32_multi(const PGroup* groups, int64_t n_groups, const WinProb* probs,
+cudaError_t launch_unpoint_win32_multi(const PGroup* groups, int64_t n_groups, const WinSize& size, const WinProb* probs,
                                        cudaStream_t s) {
   if (n_groups == 0) return cudaSuccess;
   if (n_groups > 0x7fffffffLL || probs == nullptr) return cudaErrorInvalidValue;
   static cudaError_t st = cudaSuccess;
   static bool set = false;
   MM_TRY_CUDA(smem_limit_once(k_unpoint_win32<true>, kUnpointSmem, st, set));
-  k_unpoint_win32<true><<<(unsigned)n_groups, kWinThreads, kUnpointSmem, s>>>(
-      groups, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 1, nullptr, 0, nullptr, 0, probs);
+  k_unpoint_win32<true><<<(unsigned)n_groups, unpoint_threads(size), unpoint_smem(size), s>>>(
+      groups, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 1, nullptr, 0, nullptr, 0, probs, size);
   return cudaGetLastError();
 }
 
-// y += P^T u over the windows: one CTA per group and column, samples summed per slot in shared
-// memory (three FP32 shared-memory adds per sample), then one float4 global atomic per distinct
-// pixel of the group.
-constexpr size_t kPointSmem = (size_t)3 * kAccStride * sizeof(float);
+// y += P^T u by run sums: one CTA per group.  The group's u goes to shared memory by 16-byte
+// asynchronous copies; then every lane walks 32 consecutive pixel-sorted entries (position, angle),
+// sums u, u cos 2psi, u sin 2psi of a run of equal pixels in registers and adds each run to the map
+// with one float4 atomic (a pixel's sum arrives in one piece except where a lane's range cuts it).
+// Bound by HBM: 10 B per sample (entry 2, angle 4, u 4).  The three FP32 shared-memory additions per
+// sample that it replaces are loops of compare-and-swap on this machine and kept the shared-memory pipe
+// at 83 to 87% (20 shared wavefronts per 32 samples, here 4): 256 detectors x 4 x 524,288 samples 1.52
+// -> 1.08 ms, 64 x 262,144 64 -> 42 us, 4 x 65,536 86 -> 8 us (with the groups of build_windows).
 template <bool MULTI>
-__global__ void __launch_bounds__(kWinThreads, 3) k_point_win32(
-    const PGroup* __restrict__ groups, const int64_t* __restrict__ block_off,
-    const uint16_t* __restrict__ slot, const int32_t* __restrict__ slot_pix, const float* __restrict__ ang2,
-    const float* __restrict__ u, int64_t u_stride, int nrhs, const int32_t* __restrict__ done, int done_stride,
-    float4* __restrict__ y4, int64_t y_stride4, const WinProb* __restrict__ probs) {
-  extern __shared__ float acc[];   // [3][kAccStride]
+__global__ void __launch_bounds__(kWinThreads, 2) k_point_sorted(
+    const PGroup* __restrict__ groups, const int64_t* __restrict__ block_off, const uint4* __restrict__ ent,
+    const float4* __restrict__ ent_ang, const uint16_t* __restrict__ first_slot,
+    const int32_t* __restrict__ slot_pix, const float* __restrict__ u, int64_t u_stride, int nrhs,
+    const int32_t* __restrict__ done, int done_stride, float4* __restrict__ y4, int64_t y_stride4,
+    const WinProb* __restrict__ probs, WinSize size) {
+  extern __shared__ __align__(16) float us[];   // n_blk rows of W + 4, then a zero; after them the row table
   const PGroup G = groups[blockIdx.x];
   if constexpr (MULTI) {
     const WinProb& pp = probs[G.prob];
     block_off = pp.block_off;
-    slot = pp.slot;
+    ent = pp.srt_ent;
+    ent_ang = pp.srt_ang;
+    first_slot = pp.srt_slot;
     slot_pix = pp.slot_pix;
-    ang2 = pp.ang2;
     u = pp.u;
     y4 = reinterpret_cast<float4*>(pp.y);
     done = pp.done;
   }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const ChunkWalk cw = chunk_walk(G, lane);
-  const int n_pad = acc_index(G.n_slots);
-  const bool keep = nrhs > 1;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+  const int row = srt_row(G.log_w);
+  const QuadWalk w = quad_walk(G, lane);
+  RowTab rt(us + size.rows, size.dets);
+  const int32_t* __restrict__ pix = slot_pix + G.slot_off;
+  rt.load(G, block_off);
   for (int r = 0; r < nrhs; r++) {
     if (done != nullptr && done[(int64_t)r * done_stride] != 0) continue;
     const float* ur = u + r * u_stride;
-    for (int k = threadIdx.x; k < n_pad; k += kWinThreads) {
-      acc[k] = 0.f;
-      acc[kAccStride + k] = 0.f;
-      acc[2 * kAccStride + k] = 0.f;
+    // this warp's first block of entries and half of its angles, on their way during the staging
+    uint4 e[4];
+    float4 a[4];
+    int sl = kNoSlot;
+    if (warp < G.n_srt) {
+      const int64_t blk = G.srt_off + warp;
+      sl = __ldg(first_slot + blk * 32 + lane);
+#pragma unroll
+      for (int o = 0; o < 4; o++) {
+        e[o] = __ldg(ent + blk * (kSrtBlock / 8) + o * 32 + lane);
+        a[o] = __ldg(ent_ang + blk * (kSrtBlock / 4) + o * 32 + lane);
+      }
     }
-    __syncthreads();
-    auto add = [&](uint32_t sl, float a, float y) {
-      if (sl == kNoSlot) return;
-      float cs, sn;
-      weights_of_angle(a, cs, sn);
-      const int k = acc_index((int)sl);
-      atomicAdd(acc + k, y);
-      atomicAdd(acc + kAccStride + k, cs * y);
-      atomicAdd(acc + 2 * kAccStride + k, sn * y);
+    __syncthreads();   // the rows are there, the previous column's u is no longer read
+    auto copy = [&](int c, int q) {
+      const int64_t lo = rt.lo[c];
+      const int a0 = (int)(lo & 3), len = rt.len[c];
+      if (len > 0 && 4 * q < a0 + len)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(us + c * row + 4 * q)),
+                     "l"(ur + lo - a0 + 4 * q)
+                     : "memory");
     };
-    // warps take contiguous ranges of the group's chunks (detectors), so warps running at the
-    // same time sit far apart on the focal plane and rarely add to the same pixel at once
-    const int n_it = (G.n_blk + cw.cpi - 1) / cw.cpi;
-    const int per = (n_it + kWarps - 1) / kWarps;
-    for (int it = warp * per; it < min(n_it, (warp + 1) * per); it++) {
-      const int c = it * cw.cpi + cw.sub;
-      if (c >= G.n_blk) continue;
-      visit_chunk(
-          G, block_off, c, cw,
-          [&](int64_t a0, int q) {
-            const int64_t i = a0 + 4 * (int64_t)q;
-            const uint2 s2 = ld_point(reinterpret_cast<const uint2*>(slot + i), keep);
-            const float4 a = ld_point(reinterpret_cast<const float4*>(ang2 + i), keep);
-            const float4 y = __ldcs(reinterpret_cast<const float4*>(ur + i));
-            add(s2.x & 0xFFFFu, a.x, y.x);
-            add(s2.x >> 16, a.y, y.y);
-            add(s2.y & 0xFFFFu, a.z, y.z);
-            add(s2.y >> 16, a.w, y.w);
-          },
-          [&](int64_t i) { add(ld_point(slot + i, keep), ld_point(ang2 + i, keep), __ldcs(ur + i)); });
-    }
+    for (int c0 = warp * w.cpi + w.sub; c0 < w.n_units; c0 += warps * w.cpi)
+      copy(c0 >> w.ls, ((c0 & ((1 << w.ls) - 1)) << (w.lu - 2)) + w.ql);
+    for (int c = threadIdx.x; c < G.n_blk; c += blockDim.x) copy(c, 1 << (G.log_w - 2));
+    if (threadIdx.x == 0) us[G.n_blk * row] = 0.f;
+    asm volatile("cp.async.commit_group;\ncp.async.wait_all;" ::: "memory");
     __syncthreads();
     float4* yr = y4 + r * y_stride4;
-    for (int k = threadIdx.x; k < G.n_slots; k += kWinThreads) {
-      const int32_t p = __ldg(slot_pix + G.slot_off + k);
-      const int j = acc_index(k);
-      atomicAdd(yr + p, make_float4(acc[j], acc[kAccStride + j], acc[2 * kAccStride + j], 0.f));
+    for (int b = warp; b < G.n_srt; b += warps) {
+      const int64_t blk = G.srt_off + b;
+      const uint4* ep = ent + blk * (kSrtBlock / 8) + lane;
+      const float4* ap = ent_ang + blk * (kSrtBlock / 4) + lane;
+      if (b != warp) {
+        sl = __ldg(first_slot + blk * 32 + lane);
+#pragma unroll
+        for (int o = 0; o < 4; o++) {
+          e[o] = __ldg(ep + o * 32);
+          a[o] = __ldg(ap + o * 32);
+        }
+      }
+      if (sl == kNoSlot) continue;
+      int32_t p = __ldg(pix + sl);
+      float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+      auto one = [&](uint32_t en, float an) {
+        if (en & kSrtRun) {   // a new run: the previous pixel's sum is complete
+          atomicAdd(yr + p, make_float4(s0, s1, s2, 0.f));
+          p = __ldg(pix + ++sl);
+          s0 = s1 = s2 = 0.f;
+        }
+        const float y = us[en & 0x7FFFu];
+        float cs, sn;
+        weights_of_angle(an, cs, sn);
+        s0 += y;
+        s1 = fmaf(cs, y, s1);
+        s2 = fmaf(sn, y, s2);
+      };
+#pragma unroll
+      for (int o = 0; o < 4; o++) {
+        // angle quads 2 o and 2 o + 1: four are held, the next two are loaded as these are used
+        const int h = (2 * o) & 3;
+        const float4 a0 = a[h], a1 = a[h + 1];
+        if (o < 2) {
+          a[h] = __ldg(ap + (2 * o + 4) * 32);
+          a[h + 1] = __ldg(ap + (2 * o + 5) * 32);
+        }
+        one(e[o].x & 0xFFFFu, a0.x);
+        one(e[o].x >> 16, a0.y);
+        one(e[o].y & 0xFFFFu, a0.z);
+        one(e[o].y >> 16, a0.w);
+        one(e[o].z & 0xFFFFu, a1.x);
+        one(e[o].z >> 16, a1.y);
+        one(e[o].w & 0xFFFFu, a1.z);
+        one(e[o].w >> 16, a1.w);
+      }
+      atomicAdd(yr + p, make_float4(s0, s1, s2, 0.f));
     }
-    __syncthreads();   // the next column clears the sums
   }
 }
 
-cudaError_t launch_point_win32(const PGroup* groups, int64_t n_groups, const int64_t* block_off,
-                               const uint16_t* slot, const int32_t* slot_pix, const float* ang2,
-                               const float* u, int64_t u_stride, int nrhs, const int32_t* done,
-                               int done_stride, float* y4, int64_t y_stride, cudaStream_t s) {
+static cudaError_t point_sorted_attr() {
+  constexpr int kMost = (kWinMaxSamples / 32 * ((1 << 5) + 4) + 4) * (int)sizeof(float) + 512 * 12;
+  static const cudaError_t e = [] {
+    cudaError_t r = cudaFuncSetAttribute(k_point_sorted<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+    if (r == cudaSuccess)
+      r = cudaFuncSetAttribute(k_point_sorted<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+    return r;
+  }();
+  return e;
+}
+static int point_sorted_threads(const WinSize& z) { return 32 * std::min(kWinThreads / 32, std::max(1, z.blocks)); }
+
+cudaError_t launch_point_sorted(const PGroup* groups, int64_t n_groups, const WinSize& size,
+                                const int64_t* block_off, const uint16_t* ent, const float* ent_ang,
+                                const uint16_t* first_slot, const int32_t* slot_pix, const float* u,
+                                int64_t u_stride, int nrhs, const int32_t* done, int done_stride, float* y4,
+                                int64_t y_stride, cudaStream_t s) {
   if (n_groups == 0 || nrhs <= 0) return cudaSuccess;
   if (n_groups > 0x7fffffffLL || u_stride % 4 != 0) return cudaErrorInvalidValue;
-  static cudaError_t st = cudaSuccess;
-  static bool set = false;
-  MM_TRY_CUDA(smem_limit_once(k_point_win32<false>, kPointSmem, st, set));
-  k_point_win32<false><<<(unsigned)n_groups, kWinThreads, kPointSmem, s>>>(
-      groups, block_off, slot, slot_pix, ang2, u, u_stride, nrhs, done, done_stride, reinterpret_cast<float4*>(y4),
-      y_stride / 4, nullptr);
+  MM_TRY_CUDA(point_sorted_attr());
+  k_point_sorted<false><<<(unsigned)n_groups, point_sorted_threads(size), (size_t)size.rows * sizeof(float) + row_tab_bytes(size.dets), s>>>(
+      groups, block_off, reinterpret_cast<const uint4*>(ent), reinterpret_cast<const float4*>(ent_ang), first_slot,
+      slot_pix, u, u_stride, nrhs, done, done_stride, reinterpret_cast<float4*>(y4), y_stride / 4, nullptr, size);
   return cudaGetLastError();
 }
 
-cudaError_t launch_point_win32_multi(const PGroup* groups, int64_t n_groups, const WinProb* probs,
-                                     cudaStream_t s) {
+cudaError_t launch_point_sorted_multi(const PGroup* groups, int64_t n_groups, const WinSize& size,
+                                      const WinProb* probs, cudaStream_t s) {
   if (n_groups == 0) return cudaSuccess;
   if (n_groups > 0x7fffffffLL || probs == nullptr) return cudaErrorInvalidValue;
-  static cudaError_t st = cudaSuccess;
-  static bool set = false;
-  MM_TRY_CUDA(smem_limit_once(k_point_win32<true>, kPointSmem, st, set));
-  k_point_win32<true><<<(unsigned)n_groups, kWinThreads, kPointSmem, s>>>(
-      groups, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 1, nullptr, 0, nullptr, 0, probs);
+  MM_TRY_CUDA(point_sorted_attr());
+  k_point_sorted<true><<<(unsigned)n_groups, point_sorted_threads(size), (size_t)size.rows * sizeof(float) + row_tab_bytes(size.dets), s>>>(
+      groups, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 1, nullptr, 0, nullptr, 0, probs, size);
   return cudaGetLastError();
 }
 
@@ -587,7 +861,7 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_seg32(
   const int64_t stride = seg_stride(G.n_blk, ls);
   PGroup S = G;   // the current sub-window as a group of window 2^log_s
   S.log_w = ls;
-  const ChunkWalk cw = chunk_walk(S, lane);
+  const ChunkWalk cw = chunk_walk(S.log_w, lane);
   const int n_pad = acc_index(G.n_slots);
   for (int r = 0; r < nrhs; r++) {
     if (done != nullptr && done[(int64_t)r * done_stride] != 0) continue;
@@ -622,8 +896,8 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_seg32(
         int len;
         group_chunk(S, block_off, c, lo, len);
         const int l0 = c << ls;
-        visit_chunk(
-            S, block_off, c, cw,
+        visit_unit(
+            S, block_off, c, S.log_w, cw,
             [&](int64_t a0, int q) {
               const int64_t i = a0 + 4 * (int64_t)q;
               const float4 v = __ldcs(reinterpret_cast<const float4*>(ur + i));
@@ -782,8 +1056,9 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_win_df(
     const int32_t* __restrict__ done, int done_stride, double* __restrict__ y4, int64_t y_stride) {
   extern __shared__ unsigned long long acc64[];   // [3][kAccStride]
   const PGroup G = groups[blockIdx.x];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const ChunkWalk cw = chunk_walk(G, lane);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+  const int lu = unit_log(G, warps), n_units = G.n_blk << (G.log_w - lu);
+  const ChunkWalk cw = chunk_walk(lu, lane);
   const int n_pad = acc_index(G.n_slots);
   for (int r = 0; r < nrhs; r++) {
     if (done != nullptr && done[(int64_t)r * done_stride] != 0) continue;
@@ -791,7 +1066,7 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_win_df(
     if (ub == 0u) continue;   // u = 0: nothing to add
     double* yr = y4 + r * y_stride;
     if (ub >= 0x7f800000u) {   // a non-finite u: poison the outputs so the solver sees it
-      for (int k = threadIdx.x; k < G.n_slots; k += kWinThreads)
+      for (int k = threadIdx.x; k < G.n_slots; k += blockDim.x)
         atomicAdd(yr + 4 * (int64_t)__ldg(slot_pix + G.slot_off + k), __longlong_as_double(0x7ff8000000000000ll));
       continue;
     }
@@ -803,7 +1078,7 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_win_df(
     const float sc = fast ? __int_as_float((ks - 32 + 127) << 23) : 0.f;
     const double unit = __longlong_as_double((long long)(1023 - ks) << 52);   // 2^-ks
     const float2* ur = u + r * u_stride;
-    for (int k = threadIdx.x; k < n_pad; k += kWinThreads) {
+    for (int k = threadIdx.x; k < n_pad; k += blockDim.x) {
       acc64[k] = 0ull;
       acc64[kAccStride + k] = 0ull;
       acc64[2 * kAccStride + k] = 0ull;
@@ -824,22 +1099,22 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_win_df(
         atomicAdd(acc64 + 2 * kAccStride + k, (unsigned long long)fixed_of(sy, ks));
       }
     };
-    const int n_it = (G.n_blk + cw.cpi - 1) / cw.cpi;
-    const int per = (n_it + kWarps - 1) / kWarps;
+    const int n_it = (n_units + cw.cpi - 1) / cw.cpi;
+    const int per = (n_it + warps - 1) / warps;
     const int it_end = min(n_it, (warp + 1) * per);
     for (int it = warp * per; it < it_end; it++) {
       const int c = it * cw.cpi + cw.sub;
-      if (c >= G.n_blk) continue;
-      if (it + 1 < it_end && c + cw.cpi < G.n_blk) {
+      if (c >= n_units) continue;
+      if (it + 1 < it_end && c + cw.cpi < n_units) {
         int64_t lo;
         int len;
-        group_chunk(G, block_off, c + cw.cpi, lo, len);
+        group_unit(G, block_off, c + cw.cpi, lu, lo, len);
         prefetch_chunk(slot, lo, len, cw);
         prefetch_chunk(wdf, lo, len, cw);
         prefetch_chunk(ur, lo, len, cw);
       }
-      visit_chunk(
-          G, block_off, c, cw,
+      visit_unit(
+          G, block_off, c, lu, cw,
           [&](int64_t a0, int q) {
             const int64_t i = a0 + 4 * (int64_t)q;
             const uint2 s2 = __ldcs(reinterpret_cast<const uint2*>(slot + i));
@@ -851,7 +1126,7 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_win_df(
           [&](int64_t i) { add(__ldcs(slot + i), __ldcs(wdf + i), __ldcs(ur + i)); });
     }
     __syncthreads();
-    for (int k = threadIdx.x; k < G.n_slots; k += kWinThreads) {
+    for (int k = threadIdx.x; k < G.n_slots; k += blockDim.x) {
       const int64_t p = __ldg(slot_pix + G.slot_off + k);
       const int j = acc_index(k);
       atomicAdd(yr + 4 * p, (double)(long long)acc64[j] * unit);
@@ -862,7 +1137,7 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_win_df(
   }
 }
 
-cudaError_t launch_point_win_df(const PGroup* groups, int64_t n_groups, const int64_t* block_off,
+cudaError_t launch_point_win_df(const PGroup* groups, int64_t n_groups, const WinSize& size, const int64_t* block_off,
                                 const uint16_t* slot, const int32_t* slot_pix, const float4* wdf,
                                 const float2* u, int64_t u_stride, const uint32_t* amax, int nrhs,
                                 const int32_t* done, int done_stride, double* y4, int64_t y_stride,
@@ -872,7 +1147,7 @@ cudaError_t launch_point_win_df(const PGroup* groups, int64_t n_groups, const in
   static cudaError_t st = cudaSuccess;
   static bool set = false;
   MM_TRY_CUDA(smem_limit_once(k_point_win_df, kPointDfSmem, st, set));
-  k_point_win_df<<<(unsigned)n_groups, kWinThreads, kPointDfSmem, s>>>(groups, block_off, slot, slot_pix, wdf, u,
+  k_point_win_df<<<(unsigned)n_groups, size.threads, kPointDfSmem, s>>>(groups, block_off, slot, slot_pix, wdf, u,
                                                                          u_stride, amax, nrhs, done, done_stride, y4,
                                                                          y_stride);
   return cudaGetLastError();

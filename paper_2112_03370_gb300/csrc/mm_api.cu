@@ -464,19 +464,33 @@ int build_segments(Plan* P, int steps, cudaStream_t s) {
 // detectors halved, until every group fits; then each group's pixel-sorted slot table and every
 // sample's slot are written.
 int build_windows(Plan* P, cudaStream_t s) {
-  constexpr int kWinDets = 512;
-  const int64_t kWinSamples = P->win_samples;
+  // samples per group: 16384 when that leaves every SM its three CTAs twice over, down to 1024 for
+  // small plans (262,144 samples: 256 groups instead of 8 of 32768, P 55 -> 5 us and P^T 86 -> 8 us)
+  int64_t kWinSamples = P->win_samples;
+  if (kWinSamples <= 0) {
+    kWinSamples = kWinMaxSamples;
+    while (kWinSamples > 1024 && P->N / kWinSamples < 6 * sm_count()) kWinSamples /= 2;
+  }
+  P->win_size = WinSize{};
+  P->win_size.threads = (int)std::min<int64_t>(kWinThreads, std::max<int64_t>(64, kWinSamples / 4));
   constexpr int kMinLogW = 5;
+  const int kWinDets = (int)std::min<int64_t>(512, kWinSamples >> kMinLogW);
   // a rebuild (autotuning) replaces the previous windows; captured graphs must be captured again
   if (P->groups) {
     P->buf_gen++;
-    P->bytes -= (size_t)P->n_groups * sizeof(PGroup) + (size_t)P->N * sizeof(uint16_t) +
+    P->bytes -= (size_t)P->n_groups * sizeof(PGroup) + (size_t)(P->N + 3) * sizeof(uint16_t) +
                 (size_t)std::max<int64_t>(P->n_slots_total, 1) * sizeof(int32_t);
     dfree(P->groups);
     dfree(P->slot);
     dfree(P->slot_pix);
     P->n_groups = 0;
     P->groups_host.clear();
+  }
+  if (P->srt_ent) {
+    P->bytes -= (size_t)P->n_srt * (kSrtBlock * 6 + 64);
+    dfree(P->srt_ent);
+    dfree(P->srt_ang);
+    dfree(P->srt_slot);
   }
   if (P->seg_ent) {
     P->bytes -= (size_t)P->n_ent * (sizeof(uint32_t) + sizeof(float)) + (size_t)P->n_sub_total * sizeof(int32_t);
@@ -557,10 +571,19 @@ int build_windows(Plan* P, cudaStream_t s) {
   });
   int64_t total = 0;
   const bool seg = P->precision == MM_FP32 && P->use_seg;   // pixel-sorted sub-windows (FP32 P^T)
-  int64_t n_ent = 0, n_sub = 0;
+  int64_t n_ent = 0, n_sub = 0, n_srt = 0;
   for (PGroup& g : done) {
     g.slot_off = total;
     total += g.n_slots;
+    int64_t samples = 0;
+    for (int c = 0; c < g.n_blk; c++) {
+      const int b = g.b0 + c * g.b_stride;
+      samples += std::min<int64_t>(std::max<int64_t>(0, off[b + 1] - off[b] - g.w0), (int64_t)1 << g.log_w);
+    }
+    g.srt_off = n_srt;
+    g.n_srt = (int32_t)((samples + kSrtBlock - 1) / kSrtBlock);
+    n_srt += g.n_srt;
+    P->win_size.cover(WinSize{0, g.n_slots, g.n_blk, g.n_blk * srt_row(g.log_w) + 4, g.n_srt});
     const int ls = seg_log_s(g.n_blk, g.log_w, P->seg_sub);
     g.sub0 = (int32_t)n_sub;
     g.ent_off = n_ent;
@@ -572,7 +595,9 @@ int build_windows(Plan* P, cudaStream_t s) {
   P->n_slots_total = total;
   P->win_repeat = total > 0 ? (double)P->N / (double)total : 0.0;
   MM_TRY(dalloc(P, &P->groups, done.size()));
-  MM_TRY(dalloc(P, &P->slot, P->N));
+  // the un-point kernel reads whole quads: up to 3 slots past the end, which must be valid ones
+  MM_TRY(dalloc(P, &P->slot, P->N + 3));
+  MM_CUDA(cudaMemsetAsync(P->slot + P->N, 0xFF, 3 * sizeof(uint16_t), s));
   MM_TRY(dalloc(P, &P->slot_pix, (size_t)std::max<int64_t>(total, 1)));
   int32_t* err = nullptr;
   MM_TRY(scr.alloc(&err, 1));
@@ -584,6 +609,14 @@ int build_windows(Plan* P, cudaStream_t s) {
   MM_CUDA(cudaStreamSynchronize(s));
   if (herr != 0) return fail(MM_ECUDA, "pixel windows: slot tables do not match the counts");
   P->groups_host = std::move(done);
+  if (P->precision == MM_FP32) {   // sorted entries of the FP32 P^T
+    P->n_srt = n_srt;
+    MM_TRY(dalloc(P, &P->srt_ent, (size_t)n_srt * kSrtBlock));
+    MM_TRY(dalloc(P, &P->srt_ang, (size_t)n_srt * kSrtBlock));
+    MM_TRY(dalloc(P, &P->srt_slot, (size_t)n_srt * 32));
+    MM_CUDA(launch_srt_build(P->groups, P->n_groups, P->block_off_dev, P->slot, P->ang2, P->srt_ent, P->srt_ang,
+                             P->srt_slot, s));
+  }
   if (seg) {
     MM_TRY(dalloc(P, &P->seg_ent, (size_t)n_ent));
     MM_TRY(dalloc(P, &P->seg_ang, (size_t)n_ent));
@@ -690,7 +723,7 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
   MM_TRY(dalloc(P, &P->w32, P->N));
   if (P->df64) MM_TRY(dalloc(P, &P->wdf, P->N));
   const bool windows = (P->precision == MM_FP32 || P->df64) && P->algo == MM_TPLZ_FFT && !P->no_windows;
-  if (windows && P->precision == MM_FP32) MM_TRY(dalloc(P, &P->ang2, P->N));
+  if (windows && P->precision == MM_FP32) MM_TRY(dalloc(P, &P->ang2, P->N + 3));   // quads read past the end
   MM_CUDA(launch_weights(P->psi, P->N, P->w64, P->w32, P->df64 ? P->wdf : nullptr, P->ang2, s));
   MM_CUDA(launch_bd_accum(pix, P->w64, P->block_off_dev, P->c0_blk, nb, P->N, B6, hits, s));
   MM_CUDA(launch_bd_finalize(B6, hits, P->n_pix, P->cond_max, keep, inv6, s));
@@ -944,7 +977,7 @@ int df_ninv_point(Plan* P, int g, const int32_t* done, int done_stride, double* 
   a.y_stride = df_stride(P);
   a.amax = P->amax;
   MM_CUDA(launch_ninv_df(a, s));
-  MM_CUDA(launch_point_win_df(P->groups, P->n_groups, P->block_off_dev, P->slot, P->slot_pix, P->wdf, P->udf,
+  MM_CUDA(launch_point_win_df(P->groups, P->n_groups, P->win_size, P->block_off_dev, P->slot, P->slot_pix, P->wdf, P->udf,
                               df_stride(P), P->amax, g, done, done_stride, y4, P->n_obs * 4, s));
   return MM_OK;
 }
@@ -1091,14 +1124,15 @@ int ensure_t32(Plan* P, int nrhs) {
 }
 
 // y4 += P^T u (FP32) of a plan with pixel windows: segment reduction over the pixel-sorted
-// sub-windows, or per-sample shared-memory sums over the windows
+// sub-windows, or run sums over the pixel-sorted groups
 cudaError_t point32(Plan* P, const float* u, int64_t u_stride, int nrhs, const int32_t* done, int done_stride,
                     float* y4, int64_t y_stride, cudaStream_t s) {
   if (P->use_seg && P->seg_ent)
     return launch_point_seg32(P->groups, P->n_groups, P->block_off_dev, P->seg_ent, P->seg_ang, P->seg_kept,
                               P->slot_pix, P->seg_sub, u, u_stride, nrhs, done, done_stride, y4, y_stride, s);
-  return launch_point_win32(P->groups, P->n_groups, P->block_off_dev, P->slot, P->slot_pix, P->ang2, u, u_stride,
-                            nrhs, done, done_stride, y4, y_stride, s);
+  return launch_point_sorted(P->groups, P->n_groups, P->win_size, P->block_off_dev, P->srt_ent,
+                             P->srt_ang, P->srt_slot, P->slot_pix, u, u_stride, nrhs, done, done_stride, y4,
+                             y_stride, s);
 }
 
 // y32 (accumulated, pre-zeroed) += A x32 in FP32, [nrhs][n_obs][4] float.  Profiling events: mid
@@ -1136,7 +1170,7 @@ int apply32_internal(Plan* P, const float* x32, float* y32, int nrhs, cudaStream
     for (int r0 = 0; r0 < nrhs; r0 += kc) {
       const int g = std::min(kc, nrhs - r0);
       const int32_t* dn = done ? done + (int64_t)r0 * done_stride : nullptr;
-      MM_CUDA(launch_unpoint_win32(P->groups, P->n_groups, P->block_off_dev, P->slot, P->slot_pix, P->ang2,
+      MM_CUDA(launch_unpoint_win32(P->groups, P->n_groups, P->win_size, P->block_off_dev, P->slot, P->slot_pix, P->ang2,
                                    x32 + (size_t)r0 * ms, ms, g, dn, done_stride, P->t32, ts, s));
       if (mid && r0 == 0) MM_CUDA(cudaEventRecord(mid, s));
       MM_TRY(ninv32(P, P->t32, P->u32, ts, g, dn, done_stride, s));
@@ -1443,6 +1477,7 @@ struct Server {
   PGroup* wgroups_dev = nullptr;
   size_t wgroups_cap = 0;
   int64_t n_wgroups = 0;
+  WinSize wsize;                   // the largest group of any running plan
   WinProb* wprobs_dev = nullptr;
   size_t wprobs_cap = 0;
   TileDesc* ntiles_dev[kNinvSizes] = {};   // one list (and launch) per tile size
@@ -1458,7 +1493,7 @@ struct Server {
 size_t estimate_footprint(const Request& r) {
   int64_t N = 0;
   for (int64_t v : r.block_len) N += v;
-  // pointing (pixel, angle, reduced angle, window slot), FP32, FP64 and df64 weights, un-pointed
+  // pointing (pixel, angle, reduced angle, window slot, sorted entries), FP32, FP64 and df64 weights, un-pointed
   // FP32 and df64 buffers, N^-1 t in FP32 and df64 and the TOD: 100 bytes per sample
   return (size_t)N * 100 + (size_t)r.desc.n_pix * 480 + ((size_t)64 << 20);
 }
@@ -1581,6 +1616,7 @@ int rebuild_launch(Server* S) {
   std::vector<PGroup> wgroups;
   std::vector<WinProb> wprobs;
   int halo = 0;
+  WinSize wsize;
   S->tw32 = nullptr;
   for (const float2*& tw : S->ntw32) tw = nullptr;
   for (size_t i = 0; i < S->running.size(); i++) {
@@ -1602,8 +1638,10 @@ int rebuild_launch(Server* S) {
         g.prob = (int32_t)wprobs.size();
         wgroups.push_back(g);
       }
-      wprobs.push_back(WinProb{P->block_off_dev, P->slot, P->slot_pix, P->ang2, r->cg->p32, P->t32, P->u32,
-                               r->cg->q32, halt});
+      wprobs.push_back(WinProb{P->block_off_dev, P->slot, P->slot_pix, P->ang2,
+                               reinterpret_cast<const uint4*>(P->srt_ent), reinterpret_cast<const float4*>(P->srt_ang),
+                               P->srt_slot, r->cg->p32, P->t32, P->u32, r->cg->q32, halt});
+      wsize.cover(P->win_size);
       const int sz = P->ninv_logm - kNinvLogMin;
       S->ntw32[sz] = P->ntw32;
       for (TileDesc td : P->nsegs_host) {
@@ -1638,6 +1676,7 @@ int rebuild_launch(Server* S) {
   S->n_tiles = (int64_t)tiles.size();
   S->halo = halo;
   S->n_wgroups = (int64_t)wgroups.size();
+  S->wsize = wsize;
   S->dirty = false;
   return MM_OK;
 }
@@ -1645,7 +1684,7 @@ int rebuild_launch(Server* S) {
 // one A-application of every running FP32 request (accumulated into its zeroed q32)
 int enqueue_multi_apply(Server* S, cudaStream_t s) {
   if (S->n_wgroups > 0) {
-    MM_CUDA(launch_unpoint_win32_multi(S->wgroups_dev, S->n_wgroups, S->wprobs_dev, s));
+    MM_CUDA(launch_unpoint_win32_multi(S->wgroups_dev, S->n_wgroups, S->wsize, S->wprobs_dev, s));
     for (int k = 0; k < kNinvSizes; k++) {
       TileArgs a{};
       a.tiles = S->ntiles_dev[k];
@@ -1655,7 +1694,7 @@ int enqueue_multi_apply(Server* S, cudaStream_t s) {
       a.probs = S->nprobs_dev;
       MM_CUDA(launch_ninv32(kNinvLogMin + k, a, s));
     }
-    MM_CUDA(launch_point_win32_multi(S->wgroups_dev, S->n_wgroups, S->wprobs_dev, s));
+    MM_CUDA(launch_point_sorted_multi(S->wgroups_dev, S->n_wgroups, S->wsize, S->wprobs_dev, s));
   }
   if (S->n_tiles > 0) {
     TileArgs a{};
@@ -2400,7 +2439,7 @@ int mm_autotune(mm_plan_t plan, int max_width, mm_tune_info* out, void* stream) 
     out->big_tiles = P->use_big ? 1 : 0;
   }
   // 2. samples per pixel-window group: larger groups repeat more pixels but stream shorter chunks
-  const int win_c[] = {8192, 16384, 32768, 65536};
+  const int win_c[] = {2048, 4096, 8192, kWinMaxSamples};
   best = 1e300;
   int best_win = P->win_samples;
   for (int v : win_c) {

@@ -83,6 +83,37 @@ struct PGroup {
   int64_t w0;        // window start, samples from each block's start
   int64_t slot_off;  // first entry of the group's pixel-sorted slot table
   int64_t ent_off;   // first pixel-sorted entry of the group's sub-windows
+  int64_t srt_off;   // first block of sorted entries (P^T by sorted runs), in blocks of kSrtBlock
+  int32_t n_srt;     // blocks of sorted entries
+  int32_t pad;
+};
+
+// Sorted entries of a group (FP32 P^T by run sums, k_point_sorted): its kept samples ordered by slot,
+// in blocks of 32 lanes x 32 entries.  Lane l of block k holds the consecutive entries
+// [32 (32 k + l), 32 (32 k + l + 1)), stored interleaved so that a warp's vector loads are contiguous:
+// an entry is 15 bits of position in the group's staged u plus a flag on the first entry of a slot's
+// run, with its angle beside it and the slot of every lane's first entry.  A group holds at most
+// kWinMaxSamples samples, staged as one row of W + 4 floats per detector chunk (the chunk's samples
+// from their 16-byte boundary on), then a zero that padding entries point to.
+constexpr int kWinMaxSamples = 16384;
+constexpr int kSrtBlock = 1024;
+constexpr uint32_t kSrtRun = 0x8000u;      // first entry of a run
+__host__ __device__ inline int srt_row(int log_w) { return (1 << log_w) + 4; }
+
+// The largest group of a launch of the window kernels: their CTAs and shared memory are sized by it.
+struct WinSize {
+  int32_t threads = 0;   // threads that the groups' samples keep busy (at most kWinThreads)
+  int32_t slots = 0;     // distinct pixels
+  int32_t dets = 0;      // rows
+  int32_t rows = 0;      // staged floats of the rows and the zero (a multiple of 4)
+  int32_t blocks = 0;    // blocks of sorted entries
+  void cover(const WinSize& o) {
+    threads = threads > o.threads ? threads : o.threads;
+    slots = slots > o.slots ? slots : o.slots;
+    dets = dets > o.dets ? dets : o.dets;
+    rows = rows > o.rows ? rows : o.rows;
+    blocks = blocks > o.blocks ? blocks : o.blocks;
+  }
 };
 
 // Per-problem pointers of the multi-problem window launches of a server step (every running
@@ -94,6 +125,9 @@ struct WinProb {
   const uint16_t* slot;
   const int32_t* slot_pix;
   const float* ang2;
+  const uint4* srt_ent;
+  const float4* srt_ang;
+  const uint16_t* srt_slot;
   const float* x;    // [n_obs][4]
   float* t;          // [N]
   const float* u;    // [N]
@@ -214,7 +248,12 @@ struct Plan {
   float2* ntw32 = nullptr;             // twiddle image
   bool steps_given = false;            // the caller or the autotuner chose tile_steps
   int32_t tile_steps = 0;              // FP32 tiles walked per segment
-  int32_t win_samples = 32768;         // target samples per pixel-window group
+  int32_t win_samples = 0;             // target samples per pixel-window group (0: from the plan's size)
+  WinSize win_size;                    // largest group, for the launches of the window kernels
+  uint16_t* srt_ent = nullptr;         // [n_srt][kSrtBlock] sorted entries (FP32 plans, interleaved)
+  float* srt_ang = nullptr;            // [n_srt][kSrtBlock] their angles
+  uint16_t* srt_slot = nullptr;        // [n_srt][32] slot of each lane's first entry (kNoSlot: none)
+  int64_t n_srt = 0;
   int32_t tuned_width = 0;             // block width chosen by mm_autotune (0: not tuned)
 
   // tensor-core Toeplitz product (MM_TPLZ_GEMM plans)
@@ -383,15 +422,18 @@ cudaError_t launch_tiles_fp64(int mode, const TileArgs& a, cudaStream_t s);
 cudaError_t launch_win_build(const PGroup* groups, int64_t n_groups, const int64_t* block_off,
                              const int32_t* lpix, int32_t* n_slots_out, uint16_t* slot, int32_t* slot_pix,
                              cudaStream_t s);
+// sorted entries, their angles and first slots of every group (groups' srt_off and n_srt set)
+cudaError_t launch_srt_build(const PGroup* groups, int64_t n_groups, const int64_t* block_off, const uint16_t* slot,
+                             const float* ang2, uint16_t* ent, float* ent_ang, uint16_t* first_slot, cudaStream_t s);
 // t [nrhs][t_stride] = P x (FP32, weights from psi in registers) over the windows
-cudaError_t launch_unpoint_win32(const PGroup* groups, int64_t n_groups, const int64_t* block_off,
+cudaError_t launch_unpoint_win32(const PGroup* groups, int64_t n_groups, const WinSize& size, const int64_t* block_off,
                                  const uint16_t* slot, const int32_t* slot_pix, const float* psi,
                                  const float* x4, int64_t x_stride, int nrhs, const int32_t* done,
                                  int done_stride, float* t, int64_t t_stride, cudaStream_t s);
 // y4 [nrhs][y_stride] (FP64 map) += P^T u for df64 u ((hi, lo) pairs [nrhs][u_stride]) over the
 // windows: per group, 64-bit fixed-point sums in shared memory scaled by amax[r] (bits of the
 // column's max |u|), then one FP64 atomic per pixel and component
-cudaError_t launch_point_win_df(const PGroup* groups, int64_t n_groups, const int64_t* block_off,
+cudaError_t launch_point_win_df(const PGroup* groups, int64_t n_groups, const WinSize& size, const int64_t* block_off,
                                 const uint16_t* slot, const int32_t* slot_pix, const float4* wdf,
                                 const float2* u, int64_t u_stride, const uint32_t* amax, int nrhs,
                                 const int32_t* done, int done_stride, double* y4, int64_t y_stride,
@@ -406,17 +448,19 @@ cudaError_t launch_point_seg32(const PGroup* groups, int64_t n_groups, const int
                                const int32_t* slot_pix, int sub_cap, const float* u, int64_t u_stride,
                                int nrhs, const int32_t* done, int done_stride, float* y4, int64_t y_stride,
                                cudaStream_t s);
-// y4 [nrhs][y_stride] += P^T u (FP32) over the windows, u [nrhs][u_stride]
-cudaError_t launch_point_win32(const PGroup* groups, int64_t n_groups, const int64_t* block_off,
-                               const uint16_t* slot, const int32_t* slot_pix, const float* psi,
-                               const float* u, int64_t u_stride, int nrhs, const int32_t* done,
-                               int done_stride, float* y4, int64_t y_stride, cudaStream_t s);
+// y4 [nrhs][y_stride] += P^T u (FP32) by run sums over the sorted entries, u [nrhs][u_stride] (a
+// multiple of 4)
+cudaError_t launch_point_sorted(const PGroup* groups, int64_t n_groups, const WinSize& size,
+                                const int64_t* block_off, const uint16_t* ent, const float* ent_ang,
+                                const uint16_t* first_slot, const int32_t* slot_pix, const float* u,
+                                int64_t u_stride, int nrhs, const int32_t* done, int done_stride, float* y4,
+                                int64_t y_stride, cudaStream_t s);
 // the same two operators for several problems in one launch (continuous batching): groups from
 // every problem's plan, each with its prob index into probs (one column per problem)
-cudaError_t launch_unpoint_win32_multi(const PGroup* groups, int64_t n_groups, const WinProb* probs,
+cudaError_t launch_unpoint_win32_multi(const PGroup* groups, int64_t n_groups, const WinSize& size, const WinProb* probs,
                                        cudaStream_t s);
-cudaError_t launch_point_win32_multi(const PGroup* groups, int64_t n_groups, const WinProb* probs,
-                                     cudaStream_t s);
+cudaError_t launch_point_sorted_multi(const PGroup* groups, int64_t n_groups, const WinSize& size,
+                                      const WinProb* probs, cudaStream_t s);
 // multiprocessors of the current device (cached per device)
 int sm_count();
 // df64 tiles and their data preparation (k_df64.cu)
