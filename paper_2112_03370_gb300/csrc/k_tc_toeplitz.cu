@@ -1,7 +1,6 @@
 // Banded block-Toeplitz product u = T(c_b) t (Eq. MADCAP; stbmm of Sect. 3.1) as a GEMM on the
 // fifth-generation tensor cores (tcgen05), in 3xTF32: the alternative to the overlap-save FFT for
-// small half-bandwidths, chosen by measurement (MM_TPLZ_GEMM, and MM_TPLZ_AUTO below the measured
-// crossover).
+// small half-bandwidths (MM_TPLZ_GEMM; MM_TPLZ_AUTO takes the FFT tiles, which measured faster).
 //
 // A block's samples are cut into rows of B = 32 (row k holds samples 32k .. 32k + 31 of the block).
 // With T_J[i][r] = c_{|32 J + r - i|} (0 beyond lambda), output row k is

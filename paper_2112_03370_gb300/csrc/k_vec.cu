@@ -1,5 +1,8 @@
 // Pixel-domain and time-domain elementwise kernels: P / P^T in FP64, the banded Toeplitz product by
 // its definition, block-Jacobi apply, layout conversions and the fused CG kernels of Algorithm 1.
+#include <cooperative_groups.h>
+
+#include "df64.cuh"
 #include "mm_internal.cuh"
 #include "mm_cg.cuh"
 
@@ -134,6 +137,33 @@ __global__ void k_unpack4to3(const double* __restrict__ x4, int64_t n_tot, doubl
     x3[3 * i + 1] = x4[4 * i + 1];
     x3[3 * i + 2] = x4[4 * i + 2];
   }
+}
+
+// ABI map [n_tot][3] -> the FP32 operators' padded map, their output map cleared on the way, and back:
+// one launch on each side of an FP32 A x instead of two and a memset
+__global__ void k_in32(const double* __restrict__ x3, int64_t n_tot, float4* __restrict__ x4, float4* __restrict__ y4) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_tot; i += (int64_t)gridDim.x * blockDim.x) {
+    x4[i] = make_float4((float)x3[3 * i], (float)x3[3 * i + 1], (float)x3[3 * i + 2], 0.f);
+    y4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
+__global__ void k_out32(const float4* __restrict__ y4, int64_t n_tot, double* __restrict__ y3) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_tot; i += (int64_t)gridDim.x * blockDim.x) {
+    const float4 v = y4[i];
+    y3[3 * i] = v.x;
+    y3[3 * i + 1] = v.y;
+    y3[3 * i + 2] = v.z;
+  }
+}
+cudaError_t launch_in32(const double* x3, int64_t n_tot, float* x4, float* y4, cudaStream_t s) {
+  if (n_tot == 0) return cudaSuccess;
+  k_in32<<<grid_for(n_tot), kNT, 0, s>>>(x3, n_tot, reinterpret_cast<float4*>(x4), reinterpret_cast<float4*>(y4));
+  return cudaGetLastError();
+}
+cudaError_t launch_out32(const float* y4, int64_t n_tot, double* y3, cudaStream_t s) {
+  if (n_tot == 0) return cudaSuccess;
+  k_out32<<<grid_for(n_tot), kNT, 0, s>>>(reinterpret_cast<const float4*>(y4), n_tot, y3);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_pack3to4(const double* x3, int64_t n, int nrhs, double* x4, cudaStream_t s) {
@@ -473,7 +503,8 @@ __global__ void k_cg_update(CgWork w) {
 // Residual replacement (FP32 path): r = b - A x with A x in FP64 (in q), z = M r, new beta.
 __global__ void k_cg_replace(CgWork w) {
   const int col = blockIdx.y;
-  if (w.scal[col].done) return;
+  // a fused column that is not paused has formed its next p: it waits for its own turn
+  if (w.scal[col].done || (w.fused && !w.scal[col].paused)) return;
   const double* b = col4(w.b, w, col);
   const double* ax = col4(w.q, w, col);
   double* r = col4(w.r, w, col);
@@ -535,6 +566,303 @@ __global__ void k_cg_true_res(CgWork w) {
   }
   double t[1];
   if (grid_sum<1>(v, w, col, t) && threadIdx.x == 0) w.scal[col].rr_true = t[0];
+}
+
+// ---- the rest of an iteration after q = A p, and the next p, in one cooperative launch ----------
+// <p, q> and alpha; x, r, z, ||r||^2, <r, z>, stop rule and beta; p = z + beta p and the cleared q: the
+// same arithmetic as k_cg_dot_pq, k_cg_update and k_cg_pupdate with two grid barriers in the place of
+// launches.  Every CTA sums the partials in the same order, so all of them take the same decisions and
+// CTA 0 alone writes the scalars.  Bound by latency on small maps (reductions and barriers) and by the
+// FP64 pipe (about 30 operations per pixel at 1/64 of the FP32 rate).  4096 pixels: 21 us in three
+// launches -> 11; 65,536 pixels: 28 -> 19 (cold caches, both).  Columns that are done or paused only
+// take part in the barriers.
+namespace {
+constexpr int kStepMaxParts = 1024;           // partial sums per column (ensure_cg)
+
+// Sum of v over the CTA, in a fixed order, in thread 0.  On the FP64 pipe an addition costs a warp 16
+// cycles however many lanes take part, so the tree halves the warps before it shuffles.
+template <int NT, int K>
+__device__ __forceinline__ void step_cta_sum(double (&v)[K], double (*sh)[NT]) {
+  const int tid = threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < K; k++) sh[k][tid] = v[k];
+  __syncthreads();
+#pragma unroll
+  for (int o = NT / 2; o >= 32; o >>= 1) {
+    if (tid < o) {
+#pragma unroll
+      for (int k = 0; k < K; k++) {
+        v[k] += sh[k][tid + o];
+        if (o > 32) sh[k][tid] = v[k];
+      }
+    }
+    if (o > 32) __syncthreads();
+  }
+  if (tid < 32) {
+#pragma unroll
+    for (int k = 0; k < K; k++)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+  }
+}
+// Sum of the CTAs' partials (K values at part[4 b + first]), in a fixed order, in lane 0 of warp 0
+template <int K>
+__device__ __forceinline__ void step_part_sum(const double* part, int first, double (&v)[K]) {
+#pragma unroll
+  for (int k = 0; k < K; k++) v[k] = 0.0;
+  for (unsigned b = threadIdx.x; b < gridDim.x; b += 32)
+#pragma unroll
+    for (int k = 0; k < K; k++) v[k] += __ldcg(part + 4 * b + first + k);
+#pragma unroll
+  for (int k = 0; k < K; k++)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+}
+__device__ __forceinline__ void load_q_bits(const CgWork& w, int col, int64_t i, double& q0, double& q1, double& q2) {
+  if (w.fp32) {   // widened with integer instructions: the conversion runs on the FP64 pipe
+    const float4 v = reinterpret_cast<const float4*>(w.q32)[(int64_t)col * w.n + i];
+    q0 = f32_to_f64_bits(v.x); q1 = f32_to_f64_bits(v.y); q2 = f32_to_f64_bits(v.z);
+  } else {
+    load_q(w, col, i, q0, q1, q2);
+  }
+}
+}  // namespace
+
+// REG: at most one pixel per thread, kept in registers from phase to phase with the loads of the second
+// phase in flight over the first barrier; otherwise the phases loop over the pixels.
+template <int NT, bool REG>
+__global__ void __launch_bounds__(NT, 512 / NT) k_cg_step(CgWork base, const CgWork* __restrict__ list) {
+  cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+  __shared__ double sh[2][NT];
+  __shared__ double s_val[2];
+  __shared__ int s_flag;
+  const CgWork w = list ? list[blockIdx.y] : base;
+  const int col = list ? 0 : blockIdx.y;
+  CgScalars& S = w.scal[col];
+  const bool run = S.halt == 0;   // CTA 0 writes the scalars after the second barrier only
+  const double rz = S.rz, bnorm2 = S.bnorm2;
+  const int since_rep = S.since_rep, iters = S.iters;
+  double2* const p = reinterpret_cast<double2*>(col4(w.p, w, col));
+  double2* const x = reinterpret_cast<double2*>(col4(w.x, w, col));
+  double2* const r = reinterpret_cast<double2*>(col4(w.r, w, col));
+  double2* const z = reinterpret_cast<double2*>(col4(w.z, w, col));
+  double* part = w.partials + (int64_t)col * kStepMaxParts * 4;
+  const int64_t i0 = (int64_t)blockIdx.x * NT + threadIdx.x, step = (int64_t)gridDim.x * NT;
+  // a pixel of the second phase: p, q, x, r and the preconditioner block
+  struct Px {
+    double2 p01, x01, r01;
+    double p2, x2, r2, q0, q1, q2, m[6];
+  } c;
+  auto load_rest = [&](int64_t i) {
+    c.x01 = x[2 * i]; c.x2 = x[2 * i + 1].x;
+    c.r01 = r[2 * i]; c.r2 = r[2 * i + 1].x;
+    const double2* m = reinterpret_cast<const double2*>(w.minv + 6 * i);
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      const double2 v = __ldg(m + k);
+      c.m[2 * k] = v.x;
+      c.m[2 * k + 1] = v.y;
+    }
+  };
+  auto load_pq = [&](int64_t i) {
+    c.p01 = p[2 * i]; c.p2 = p[2 * i + 1].x;
+    load_q_bits(w, col, i, c.q0, c.q1, c.q2);
+  };
+  if (run) {
+    double v[1] = {0.0};
+    if constexpr (REG) {
+      if (i0 < w.n) {
+        load_pq(i0);
+        load_rest(i0);
+        v[0] = c.p01.x * c.q0 + c.p01.y * c.q1 + c.p2 * c.q2;
+      }
+    } else {
+      for (int64_t i = i0; i < w.n; i += step) {
+        load_pq(i);
+        v[0] += c.p01.x * c.q0 + c.p01.y * c.q1 + c.p2 * c.q2;
+      }
+    }
+    step_cta_sum<NT, 1>(v, sh);
+    if (threadIdx.x == 0) __stcg(part + 4 * blockIdx.x, v[0]);
+  }
+  grid.sync();
+  bool broke = false;
+  if (run) {
+    if (threadIdx.x < 32) {
+      double v[1];
+      step_part_sum<1>(part, 0, v);
+      if (threadIdx.x == 0) {
+        const double alpha = rz / v[0];
+        s_val[0] = v[0];
+        s_val[1] = alpha;
+        s_flag = !(v[0] > 0.0) || !isfinite(alpha);
+      }
+    }
+    __syncthreads();
+    broke = s_flag != 0;
+  }
+  const double pq = s_val[0], alpha = s_val[1];
+  double z0 = 0.0, z1 = 0.0, z2 = 0.0;
+  if (run && !broke) {
+    double v[2] = {0.0, 0.0};
+    auto update = [&](int64_t i) {
+      c.x01.x += alpha * c.p01.x;
+      c.x01.y += alpha * c.p01.y;
+      x[2 * i] = c.x01;
+      x[2 * i + 1] = make_double2(c.x2 + alpha * c.p2, 0.0);
+      const double r0 = c.r01.x - alpha * c.q0, r1 = c.r01.y - alpha * c.q1, r2 = c.r2 - alpha * c.q2;
+      r[2 * i] = make_double2(r0, r1);
+      r[2 * i + 1] = make_double2(r2, 0.0);
+      bd3(c.m, r0, r1, r2, z0, z1, z2);
+      z[2 * i] = make_double2(z0, z1);
+      z[2 * i + 1] = make_double2(z2, 0.0);
+      v[0] += r0 * r0 + r1 * r1 + r2 * r2;
+      v[1] += r0 * z0 + r1 * z1 + r2 * z2;
+    };
+    if constexpr (REG) {
+      if (i0 < w.n) update(i0);
+    } else {
+      for (int64_t i = i0; i < w.n; i += step) {
+        load_pq(i);
+        load_rest(i);
+        update(i);
+      }
+    }
+    step_cta_sum<NT, 2>(v, sh);
+    if (threadIdx.x == 0) {
+      __stcg(part + 4 * blockIdx.x + 1, v[0]);
+      __stcg(part + 4 * blockIdx.x + 2, v[1]);
+    }
+  }
+  grid.sync();
+  if (!run) return;
+  if (broke) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      S.pq = pq;
+      S.alpha = 0.0;
+      S.halt = 1;
+      if (w.fp32 && since_rep > 0 && isfinite(pq)) {   // as in k_cg_dot_pq
+        S.paused = 1;
+        S.restart_req = 1;
+      } else {
+        S.status = MM_EBREAKDOWN;
+        S.done = 1;
+      }
+    }
+    return;
+  }
+  if (threadIdx.x < 32) {
+    double v[2];
+    step_part_sum<2>(part, 1, v);
+    if (threadIdx.x == 0) {
+      const double beta = v[1] / rz;
+      int status = MM_OK;
+      bool paused = false, done = false;
+      if (v[0] < (w.fp32 ? 0.25 : 1.0) * w.tol2 * bnorm2) {   // as in k_cg_update
+        if (w.fp32) paused = true;
+        else done = true;
+      } else if (!isfinite(v[0]) || !isfinite(beta)) {
+        status = MM_EBREAKDOWN;
+        done = true;
+      } else if (iters + 1 >= w.max_iter) {
+        status = MM_ENOTCONV;
+        done = true;
+      } else if (w.fp32 && since_rep + 1 >= w.rel_every) {
+        paused = true;
+      }
+      s_val[0] = beta;
+      s_flag = paused || done;
+      if (blockIdx.x == 0) {
+        S.pq = pq;
+        S.alpha = alpha;
+        S.iters = iters + 1;
+        S.since_rep = since_rep + 1;
+        S.rr = v[0];
+        S.rz_prev = rz;
+        S.rz = v[1];
+        S.beta = beta;
+        if (paused) S.paused = 1;
+        if (done) {
+          S.done = 1;
+          if (status != MM_OK) S.status = status;
+        }
+        if (paused || done) S.halt = 1;
+      }
+    }
+  }
+  __syncthreads();
+  if (s_flag != 0) return;   // p waits for the replaced residual's beta
+  const double beta = s_val[0];
+  auto next_p = [&](int64_t i) {
+    c.p01.x = z0 + beta * c.p01.x;
+    c.p01.y = z1 + beta * c.p01.y;
+    c.p2 = z2 + beta * c.p2;
+    p[2 * i] = c.p01;
+    p[2 * i + 1] = make_double2(c.p2, 0.0);
+    if (w.fp32) {
+      reinterpret_cast<float4*>(w.p32)[(int64_t)col * w.n + i] =
+          make_float4((float)c.p01.x, (float)c.p01.y, (float)c.p2, 0.f);
+      reinterpret_cast<float4*>(w.q32)[(int64_t)col * w.n + i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+      double2* q = reinterpret_cast<double2*>(col4(w.q, w, col));
+      q[2 * i] = make_double2(0.0, 0.0);
+      q[2 * i + 1] = make_double2(0.0, 0.0);
+    }
+  };
+  if constexpr (REG) {
+    if (i0 < w.n) next_p(i0);
+  } else {
+    for (int64_t i = i0; i < w.n; i += step) {
+      const double2 z01 = z[2 * i];
+      z0 = z01.x;
+      z1 = z01.y;
+      z2 = z[2 * i + 1].x;
+      c.p01 = p[2 * i];
+      c.p2 = p[2 * i + 1].x;
+      next_p(i);
+    }
+  }
+}
+
+// The device holds 512 threads of k_cg_step per SM at once (__launch_bounds__).  Few pixels go to CTAs of
+// 128 threads so that more SMs share their FP64 work, more pixels to one CTA of 512 per SM.
+template <int NT>
+static int step_capacity() {
+  static const int per_sm = [] {
+    int a = 0, b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_cg_step<NT, true>, NT, 0) != cudaSuccess) a = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_cg_step<NT, false>, NT, 0) != cudaSuccess) b = 0;
+    return a < b ? a : b;
+  }();
+  return per_sm * sm_count();
+}
+bool cg_step_fits(int columns) { return columns > 0 && columns <= step_capacity<512>() && columns <= step_capacity<128>(); }
+
+template <int NT>
+static cudaError_t launch_step(const CgWork* w, const CgWork* list, int cols, int64_t n_max, cudaStream_t s) {
+  const int64_t need = (n_max + NT - 1) / NT;
+  int64_t g = need;
+  if (g > step_capacity<NT>() / cols) g = step_capacity<NT>() / cols;
+  if (g > kStepMaxParts) g = kStepMaxParts;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)g, (unsigned)cols);
+  cfg.blockDim = dim3(NT);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const CgWork one = list ? CgWork{} : *w;
+  return g >= need ? cudaLaunchKernelEx(&cfg, k_cg_step<NT, true>, one, list)
+                   : cudaLaunchKernelEx(&cfg, k_cg_step<NT, false>, one, list);
+}
+
+cudaError_t launch_cg_step(const CgWork* w, const CgWork* list, int count, int64_t n_max, cudaStream_t s) {
+  const int cols = list ? count : w->nrhs;
+  if (!cg_step_fits(cols) || n_max <= 0) return cudaErrorInvalidValue;
+  if (n_max * cols <= (int64_t)128 * sm_count()) return launch_step<128>(w, list, cols, n_max, s);
+  return launch_step<512>(w, list, cols, n_max, s);
 }
 
 cudaError_t launch_cg(CgKernel k, const CgWork& w, cudaStream_t s) {

@@ -62,7 +62,7 @@ struct CgState {
   CgScalars* scal_host = nullptr;   // pinned
   // cached graph of `chunk` iterations
   cudaGraphExec_t exec = nullptr;
-  int g_nrhs = -1, g_fp32 = -1, g_chunk = -1, g_maxit = -1, g_prec = -1;
+  int g_nrhs = -1, g_fp32 = -1, g_chunk = -1, g_maxit = -1, g_prec = -1, g_rel = -1;
   double g_tol2 = -1.0;
   uint64_t g_buf_gen = ~0ull;       // plan buffer generation the graph's pointers belong to
 };
@@ -640,8 +640,10 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
   // P->precision: arithmetic of the CG-iteration operators; P->df64: FP64-class ones in df64
   P->precision = (d->precision == MM_FP32 || d->precision == MM_FP32_DF64) ? MM_FP32 : MM_FP64;
   P->algo = (d->toeplitz_algo == MM_TPLZ_DIRECT) ? MM_TPLZ_DIRECT : MM_TPLZ_FFT;
+  // MM_TPLZ_AUTO takes the FFT tiles at every lambda: A x on 33.5M samples, FFT against GEMM: lambda 0
+  // 262 and 278 us, 32: 266 and 310, 64: 267 and 338, 128: 268 and 498; on 262,144 samples 40 to 42 us both
   P->tc = P->precision == MM_FP32 && P->algo == MM_TPLZ_FFT && d->lambda <= kTcMaxJ0 * 32 &&
-          (d->toeplitz_algo == MM_TPLZ_GEMM || (d->toeplitz_algo == MM_TPLZ_AUTO && d->lambda <= kTcAutoLambda));
+          d->toeplitz_algo == MM_TPLZ_GEMM;
   P->df64 = (d->precision == MM_DF64 || d->precision == MM_FP32_DF64) && P->algo == MM_TPLZ_FFT;
   P->cond_max = d->cond_max > 0 ? d->cond_max : 1e3;
   P->use_seg = d->pt_sub > 0;
@@ -1272,14 +1274,19 @@ CgWork make_work(Plan* P, CgState* c, int nrhs, bool fp32, double tol, int max_i
 }
 
 // One PCG iteration: p = z + beta p; q = A p; alpha; x, r, z, beta (z = M_2lvl r when dw != null).
+// Fused works (w.fused) have formed p before: q = A p, then the rest and the next p in one launch.
 int enqueue_iteration(Plan* P, const CgWork& w, int nrhs, bool fp32, cudaStream_t s,
                       const DeflWork* dw = nullptr) {
-  MM_CUDA(launch_cg(CG_PUPDATE, w, s));
+  if (!w.fused) MM_CUDA(launch_cg(CG_PUPDATE, w, s));
   const int32_t* halt = reinterpret_cast<const int32_t*>(w.scal) + kHaltOffsetInts;
   if (fp32) {
     MM_TRY(apply32_internal(P, w.p32, w.q32, nrhs, s, halt, kScalStrideInts));
   } else {
     MM_TRY(apply64_internal(P, w.p, w.q, nrhs, s, halt, kScalStrideInts));
+  }
+  if (w.fused) {
+    MM_CUDA(launch_cg_step(&w, nullptr, 0, w.n, s));
+    return MM_OK;
   }
   MM_CUDA(launch_cg(CG_DOT_PQ, w, s));
   MM_CUDA(launch_cg(CG_UPDATE, w, s));
@@ -1445,6 +1452,9 @@ struct Request {
   Clock::time_point t_submit, t_admit;
 };
 
+constexpr int kServerCheck = 4;    // iterations between the server's looks at the requests' scalars
+constexpr int kStepBatch = 64;     // requests whose CG steps share a launch
+
 struct Server {
   size_t budget = 0;
   int max_slots = 1;
@@ -1486,6 +1496,10 @@ struct Server {
   const float2* ntw32[kNinvSizes] = {};    // twiddle image of a running plan with that tile size
   ProbPtrs* nprobs_dev = nullptr;
   size_t nprobs_cap = 0;
+  CgWork* works_dev = nullptr;     // CG state of the running FP32 requests
+  size_t works_cap = 0;
+  int n_works = 0;
+  int64_t works_n_max = 0;         // most pixels of one of them
   const float2* tw32 = nullptr;    // twiddles of a running request's plan (the same in every plan)
   bool dirty = true;
 };
@@ -1548,9 +1562,13 @@ int start_request(Server* S, Request* r, cudaStream_t ps) {
   MM_TRY(ensure_cg(P, 1, r->fp32, &r->cg, ps));
   if (!r->fp32) MM_TRY(ensure_df(P, 1));
   r->w = make_work(P, r->cg, 1, r->fp32, r->opts.tol, r->opts.max_iter);
+  const int rel_every = r->opts.reliable_every > 0 ? r->opts.reliable_every : 50;
+  r->w.fused = 1;
+  r->w.rel_every = (rel_every + kServerCheck - 1) / kServerCheck * kServerCheck;
   MM_CUDA(cudaMallocHost((void**)&r->scal_host, sizeof(CgScalars)));
   MM_CUDA(launch_pack3to4(r->b_dev, P->n_obs, 1, r->cg->b, ps));
   MM_CUDA(launch_cg(CG_INIT, r->w, ps));
+  MM_CUDA(launch_cg(CG_PUPDATE, r->w, ps));
   MM_CUDA(cudaStreamSynchronize(ps));   // the server thread uses the state on its own stream
   r->t_admit = Clock::now();
   return MM_OK;
@@ -1615,6 +1633,8 @@ int rebuild_launch(Server* S) {
   std::vector<ProbPtrs> probs, nprobs;
   std::vector<PGroup> wgroups;
   std::vector<WinProb> wprobs;
+  std::vector<CgWork> works;
+  S->works_n_max = 0;
   int halo = 0;
   WinSize wsize;
   S->tw32 = nullptr;
@@ -1624,6 +1644,8 @@ int rebuild_launch(Server* S) {
     if (!r->fp32) continue;   // FP64-class requests run their own iterations
     Plan* P = r->plan;
     const int32_t* halt = reinterpret_cast<const int32_t*>(r->cg->scal) + kHaltOffsetInts;
+    works.push_back(r->w);
+    S->works_n_max = std::max(S->works_n_max, r->w.n);
     if (!S->tw32) S->tw32 = P->tw32;
     ProbPtrs pp{};
     pp.lpix = P->lpix;
@@ -1672,6 +1694,8 @@ int rebuild_launch(Server* S) {
   MM_TRY(upload_list(nprobs, S->nprobs_dev, S->nprobs_cap, S->stream));
   MM_TRY(upload_list(wgroups, S->wgroups_dev, S->wgroups_cap, S->stream));
   MM_TRY(upload_list(wprobs, S->wprobs_dev, S->wprobs_cap, S->stream));
+  MM_TRY(upload_list(works, S->works_dev, S->works_cap, S->stream));
+  S->n_works = (int)works.size();
   MM_CUDA(cudaStreamSynchronize(S->stream));   // host vectors go out of scope
   S->n_tiles = (int64_t)tiles.size();
   S->halo = halo;
@@ -1761,16 +1785,13 @@ void server_loop(Server* S) {
     // windows), the FP64-class requests' own operator launches after them
     cudaStream_t s = S->stream;
     bool ok = true;
-    for (Request* r : S->running)
-      if (r->fp32) ok = ok && launch_cg(CG_PUPDATE, r->w, s) == cudaSuccess;
     ok = ok && enqueue_multi_apply(S, s) == MM_OK;
+    // the rest of every FP32 request's iteration in one launch per kStepBatch requests
+    for (int k = 0; k < S->n_works; k += kStepBatch)
+      ok = ok && launch_cg_step(nullptr, S->works_dev + k, std::min(kStepBatch, S->n_works - k), S->works_n_max, s) ==
+                     cudaSuccess;
     for (Request* r : S->running) {
-      if (r->fp32) {
-        ok = ok && launch_cg(CG_DOT_PQ, r->w, s) == cudaSuccess;
-        ok = ok && launch_cg(CG_UPDATE, r->w, s) == cudaSuccess;
-      } else {
-        ok = ok && enqueue_iteration(r->plan, r->w, 1, false, s) == MM_OK;
-      }
+      if (!r->fp32) ok = ok && enqueue_iteration(r->plan, r->w, 1, false, s) == MM_OK;
       r->launched += 1;
     }
     if (!ok) {
@@ -1778,7 +1799,7 @@ void server_loop(Server* S) {
       continue;
     }
     step += 1;
-    if (step % 4 != 0) continue;
+    if (step % kServerCheck != 0) continue;
     for (Request* r : S->running)
       ok = ok && cudaMemcpyAsync(r->scal_host, r->cg->scal, sizeof(CgScalars), cudaMemcpyDeviceToHost, s) ==
                      cudaSuccess;
@@ -1793,8 +1814,7 @@ void server_loop(Server* S) {
     for (size_t k = 0; k < S->running.size(); k++) {
       Request* r = S->running[k];
       const CgScalars sc = *r->scal_host;
-      const int rel_every = r->opts.reliable_every > 0 ? r->opts.reliable_every : 50;
-      const bool replace = r->fp32 && !sc.done && (sc.paused || sc.since_rep >= rel_every);
+      const bool replace = r->fp32 && !sc.done && sc.paused;
       const bool report = !r->fp32 && sc.done;
       if (!replace && !report) continue;
       Plan* P = r->plan;
@@ -1805,6 +1825,7 @@ void server_loop(Server* S) {
                                               kScalStrideInts)
                            : apply64_internal(P, r->cg->x, r->cg->q, 1, s)) == MM_OK &&
                   launch_cg(replace ? CG_REPLACE : CG_TRUE_RES, r->w, s) == cudaSuccess &&
+                  (!replace || launch_cg(CG_PUPDATE, r->w, s) == cudaSuccess) &&
                   cudaMemcpyAsync(r->scal_host, r->cg->scal, sizeof(CgScalars), cudaMemcpyDeviceToHost, s) ==
                       cudaSuccess;
     }
@@ -2055,16 +2076,16 @@ int mm_apply_A(mm_plan_t plan, const double* x, double* y, int nrhs, void* strea
   const bool fp32 = P->precision == MM_FP32 && P->algo != MM_TPLZ_DIRECT;
   MM_TRY(ensure_maps(P, nrhs, fp32));
   const size_t n4 = (size_t)nrhs * P->n_obs * 4;
-  MM_CUDA(launch_pack3to4(x, P->n_obs, nrhs, P->map64_in, s));
   if (fp32) {
-    MM_CUDA(launch_to32(P->map64_in, (int64_t)(n4 / 4), P->map32_in, s));
-    MM_CUDA(cudaMemsetAsync(P->map32_out, 0, n4 * sizeof(float), s));
+    const int64_t n_tot = (int64_t)nrhs * P->n_obs;
+    MM_CUDA(launch_in32(x, n_tot, P->map32_in, P->map32_out, s));
     MM_TRY(apply32_internal(P, P->map32_in, P->map32_out, nrhs, s));
-    MM_CUDA(launch_to64(P->map32_out, (int64_t)(n4 / 4), P->map64_out, s));
-  } else {
-    MM_CUDA(cudaMemsetAsync(P->map64_out, 0, n4 * sizeof(double), s));
-    MM_TRY(apply64_internal(P, P->map64_in, P->map64_out, nrhs, s));
+    MM_CUDA(launch_out32(P->map32_out, n_tot, y, s));
+    return MM_OK;
   }
+  MM_CUDA(launch_pack3to4(x, P->n_obs, nrhs, P->map64_in, s));
+  MM_CUDA(cudaMemsetAsync(P->map64_out, 0, n4 * sizeof(double), s));
+  MM_TRY(apply64_internal(P, P->map64_in, P->map64_out, nrhs, s));
   MM_CUDA(launch_unpack4to3(P->map64_out, P->n_obs, nrhs, y, s));
   return MM_OK;
 }
@@ -2115,6 +2136,9 @@ static int pcg_solve_impl(Plan* P, const double* b, const TodSrc* tod, double* x
     MM_TRY(ensure_defl_work(P, dst, nrhs, w.n_blocks, &dw, s));
     dwp = &dw;
   }
+  // replacements fall on the host checks: rel_every rounded up to the iterations between them
+  w.fused = !dwp && cg_step_fits(nrhs);
+  w.rel_every = (rel_every + chunk - 1) / chunk * chunk;
 
   cudaEvent_t ev;
   MM_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
@@ -2127,6 +2151,7 @@ static int pcg_solve_impl(Plan* P, const double* b, const TodSrc* tod, double* x
     MM_CUDA(launch_pack3to4(b, P->n_obs, nrhs, c->b, s));
   }
   MM_CUDA(launch_cg(CG_INIT, w, s));
+  if (w.fused) MM_CUDA(launch_cg(CG_PUPDATE, w, s));
   if (dwp) MM_CUDA(launch_defl_step(dw, w, s));
 
   // graph of `chunk` iterations, cached on the plan
@@ -2134,7 +2159,7 @@ static int pcg_solve_impl(Plan* P, const double* b, const TodSrc* tod, double* x
   // reads (t, df64 and direct-path scratch, deflation space and its work arrays) was reallocated.
   if (opts->profile == 0 && (!c->exec || c->g_nrhs != nrhs || c->g_fp32 != (int)fp32 || c->g_chunk != chunk ||
       c->g_tol2 != w.tol2 || c->g_maxit != opts->max_iter || c->g_prec != opts->precond ||
-      c->g_buf_gen != P->buf_gen)) {
+      c->g_rel != w.rel_every || c->g_buf_gen != P->buf_gen)) {
     if (c->exec) {
       cudaGraphExecDestroy(c->exec);
       c->exec = nullptr;
@@ -2155,12 +2180,16 @@ static int pcg_solve_impl(Plan* P, const double* b, const TodSrc* tod, double* x
     c->g_tol2 = w.tol2;
     c->g_maxit = opts->max_iter;
     c->g_prec = opts->precond;
+    c->g_rel = w.rel_every;
     c->g_buf_gen = P->buf_gen;
   }
 
+  // kernels of an iteration: its A-application counted as one (three per column on the direct path),
+  // and p, <p, q> and the updates in three launches or one
+  const int apply_kernels = (fp32 || P->algo != MM_TPLZ_DIRECT) ? 1 : 3 * nrhs, cg_kernels = w.fused ? 1 : 3;
   std::vector<int> timed_out(nrhs, 0);
   const bool profile = opts->profile != 0;
-  int64_t n_kernels = 2;   // pack + init
+  int64_t n_kernels = w.fused ? 3 : 2;   // pack + init (+ the first p)
   // profile mode: event pairs around every tile launch, summed at each host sync
   struct EvPair { cudaEvent_t a, b, m, m2; int is64; };
   std::vector<EvPair> pool, pending;
@@ -2230,7 +2259,7 @@ static int pcg_solve_impl(Plan* P, const double* b, const TodSrc* tod, double* x
     for (int r = 0; r < nrhs; r++) {
       const CgScalars& sc = c->scal_host[r];
       if (!sc.done) all_done = false;
-      if (!sc.done && fp32 && (sc.paused || sc.since_rep >= rel_every)) need_rep = true;
+      if (!sc.done && fp32 && (sc.paused || (!w.fused && sc.since_rep >= rel_every))) need_rep = true;
     }
     if (all_done) break;
     const double el_us =
@@ -2245,6 +2274,10 @@ static int pcg_solve_impl(Plan* P, const double* b, const TodSrc* tod, double* x
       MM_TRY(timed_apply64(reinterpret_cast<const int32_t*>(c->scal) + kDoneOffsetInts));
       MM_CUDA(launch_cg(CG_REPLACE, w, s));
       n_kernels += 1;
+      if (w.fused) {
+        MM_CUDA(launch_cg(CG_PUPDATE, w, s));
+        n_kernels += 1;
+      }
       if (dwp) {
         DeflWork dr = dw;
         dr.restart = 1;
@@ -2255,11 +2288,11 @@ static int pcg_solve_impl(Plan* P, const double* b, const TodSrc* tod, double* x
     }
     if (!profile) {
       MM_CUDA(cudaGraphLaunch(c->exec, s));
-      n_kernels += (int64_t)chunk * ((fp32 || P->algo != MM_TPLZ_DIRECT ? 4 : 3 + 3 * nrhs) + (dwp ? 2 : 0));
+      n_kernels += (int64_t)chunk * (apply_kernels + cg_kernels + (dwp ? 2 : 0));
       if (fp32) n32 += chunk; else n64 += chunk;
     } else {
       for (int k = 0; k < chunk; k++) {
-        MM_CUDA(launch_cg(CG_PUPDATE, w, s));
+        if (!w.fused) MM_CUDA(launch_cg(CG_PUPDATE, w, s));
         EvPair e{};
         MM_TRY(take_pair(fp32 ? 0 : 1, &e));
         MM_CUDA(cudaEventRecord(e.a, s));
@@ -2270,9 +2303,13 @@ static int pcg_solve_impl(Plan* P, const double* b, const TodSrc* tod, double* x
         }
         MM_CUDA(cudaEventRecord(e.b, s));
         pending.push_back(e);
-        MM_CUDA(launch_cg(CG_DOT_PQ, w, s));
-        MM_CUDA(launch_cg(CG_UPDATE, w, s));
-        n_kernels += (fp32 || P->algo != MM_TPLZ_DIRECT) ? 4 : 3 + 3 * nrhs;
+        if (w.fused) {
+          MM_CUDA(launch_cg_step(&w, nullptr, 0, w.n, s));
+        } else {
+          MM_CUDA(launch_cg(CG_DOT_PQ, w, s));
+          MM_CUDA(launch_cg(CG_UPDATE, w, s));
+        }
+        n_kernels += apply_kernels + cg_kernels;
         if (dwp) {
           MM_CUDA(launch_defl_step(dw, w, s));
           n_kernels += 2;
@@ -3349,6 +3386,7 @@ void mm_server_destroy(mm_server_t server) {
   for (TileDesc* t : S->ntiles_dev)
     if (t) cudaFree(t);
   if (S->nprobs_dev) cudaFree(S->nprobs_dev);
+  if (S->works_dev) cudaFree(S->works_dev);
   if (S->wgroups_dev) cudaFree(S->wgroups_dev);
   if (S->wprobs_dev) cudaFree(S->wprobs_dev);
   if (S->stream) cudaStreamDestroy(S->stream);

@@ -38,6 +38,9 @@ struct CgWork {
   int32_t fp32;       // mixed-precision path
   double tol2;        // eps^2
   int32_t max_iter;   // a column stops with MM_ENOTCONV after this many iterations
+  int32_t fused;      // iterations run as A p then k_cg_step (which already forms the next p)
+  int32_t rel_every;  // fused mixed-precision path: a column pauses for its residual replacement after
+                      // this many iterations since the last one
   const double* minv; // [n][6]
   const double* b;    // [nrhs][n][4]
   double* x;
@@ -55,6 +58,11 @@ struct CgWork {
 enum CgKernel { CG_INIT, CG_PUPDATE, CG_DOT_PQ, CG_UPDATE, CG_REPLACE, CG_TRUE_RES };
 
 cudaError_t launch_cg(CgKernel k, const CgWork& w, cudaStream_t s);
+// Everything of an iteration after A p, and the next iteration's p, in one cooperative launch: of the
+// columns of *w, or of `count` works of one column each (list, device memory; n_max the most pixels).
+// Refused (cudaErrorInvalidValue) when the columns do not fit the device at once; see cg_step_fits.
+cudaError_t launch_cg_step(const CgWork* w, const CgWork* list, int count, int64_t n_max, cudaStream_t s);
+bool cg_step_fits(int columns);
 int cg_blocks_for(int64_t n);
 
 }  // namespace mm

@@ -156,8 +156,6 @@ __host__ __device__ inline int64_t seg_stride(int n_blk, int log_s) {
 // block, 3xTF32 tcgen05 MMAs over the 2 J0 + 1 row shifts, J0 = ceil(lambda / 32) <= kTcMaxJ0.
 // ---------------------------------------------------------------------------------------------
 constexpr int kTcMaxJ0 = 4;                 // lambda <= 128
-constexpr int kTcAutoLambda = 64;           // MM_TPLZ_AUTO picks the tensor cores up to this lambda
-                                            // (measured crossover against the FFT tiles)
 struct TcTile {
   int32_t blk;   // block
   int32_t k0;    // first 32-sample row of the tile within the block
@@ -492,6 +490,9 @@ cudaError_t launch_point64(const int32_t* lpix, const double2* w64, int64_t N, c
 cudaError_t launch_mask_d(const int32_t* lpix, const void* d, int d_is_fp32, int64_t N,
                           double* out, cudaStream_t s);
 cudaError_t launch_pack3to4(const double* x3, int64_t n, int nrhs, double* x4, cudaStream_t s);
+// ABI map -> FP32 map x4 with the output map y4 cleared, and FP32 map -> ABI map (n_tot pixels)
+cudaError_t launch_in32(const double* x3, int64_t n_tot, float* x4, float* y4, cudaStream_t s);
+cudaError_t launch_out32(const float* y4, int64_t n_tot, double* y3, cudaStream_t s);
 cudaError_t launch_unpack4to3(const double* x4, int64_t n, int nrhs, double* x3, cudaStream_t s);
 cudaError_t launch_to32(const double* x4, int64_t n4, float* y4, cudaStream_t s);
 cudaError_t launch_to64(const float* x4, int64_t n4, double* y4, cudaStream_t s);
