@@ -144,10 +144,13 @@ __device__ __forceinline__ void dft_small(C (&a)[R]) {
 // Twiddle factors W_M^k, k in [0, M), from a two-level table in shared memory:
 // W_M^k = hi[k >> 6] * lo[k & 63] with lo[i] = W_M^i (64 entries) and hi[i] = W_M^{64 i}
 // (M / 64 entries); one complex product, accurate to a few ulp.
+// `full` (global memory): W_M^k itself at full[k * fs].
 template <typename C>
 struct TwiddleTab {
   const C* lo;
   const C* hi;
+  const C* full;
+  int fs;
   __device__ __forceinline__ C operator()(int k) const { return c_mul(hi[k >> 6], lo[k & 63]); }
 };
 constexpr int twiddle_tab_entries(int m) { return 64 + m / 64; }
@@ -156,19 +159,26 @@ constexpr int twiddle_tab_entries(int m) { return 64 + m / 64; }
 template <typename C>
 __device__ __forceinline__ C ldg_c(const C* p) { return __ldg(p); }
 
-// Fill the shared table from the global table tw[k] = W_M^k (called by all threads, then sync).
+// Fill the shared table from the global table tw[k * fs] = W_M^k (called by all threads, then sync).
 template <typename C, int MFULL, int NT>
-__device__ __forceinline__ TwiddleTab<C> load_twiddle_tab(C* tab_sm, const C* __restrict__ tw) {
+__device__ __forceinline__ TwiddleTab<C> load_twiddle_tab(C* tab_sm, const C* __restrict__ tw, int fs = 1) {
   for (int i = threadIdx.x; i < twiddle_tab_entries(MFULL); i += NT) {
-    tab_sm[i] = (i < 64) ? ldg_c(tw + i) : ldg_c(tw + 64 * (i - 64));
+    tab_sm[i] = (i < 64) ? ldg_c(tw + i * fs) : ldg_c(tw + 64 * (i - 64) * fs);
   }
-  return TwiddleTab<C>{tab_sm, tab_sm + 64};
+  return TwiddleTab<C>{tab_sm, tab_sm + 64, tw, fs};
 }
 
-// Twiddles w_j = W_C^{n1 j} = W_M^{n1 j (M / C)}, j = 1..R-1: powers 1, 2, 4, 8 from the table,
-// the rest as products of two of those.
+// Twiddles w_j = W_C^{n1 j} = W_M^{n1 j (M / C)}, j = 1..R-1: FP32 powers 1, 2, 4, 8 from the table,
+// the rest as products of two of those.  FP64 and double-float products cost as much as a quarter of
+// the butterfly on the pipes that bound those tiles, so their twiddles are read from global memory
+// (L2 holds the table).
 template <int R, typename C>
 __device__ __forceinline__ void twiddles(const TwiddleTab<C>& tw, int base_idx, C (&w)[R]) {
+  if constexpr (sizeof(C) == 16) {
+#pragma unroll
+    for (int j = 1; j < R; j++) w[j] = ldg_c(tw.full + j * base_idx * tw.fs);
+    return;
+  }
   w[1] = tw(base_idx);
   if constexpr (R > 2) {
     w[2] = tw(2 * base_idx);
@@ -326,14 +336,14 @@ struct SmemFFT {
       __syncthreads();
     }
   }
-  static_assert(NP16 == 3, "the tiles use 2^13 or 2^14 points per CTA");
+  static_assert(NP16 == 2 || NP16 == 3, "the tiles use 2^11 to 2^14 points per CTA");
 
   template <typename C>
   __device__ static void forward(C* sm, const TwiddleTab<C>& tw, const C* ptab) {
     if constexpr (UNROLL_PASSES) {
       pass16<0, true>(sm, tw, ptab);
       pass16<1, true>(sm, tw, ptab);
-      pass16<2, true>(sm, tw, ptab);
+      if constexpr (NP16 > 2) pass16<2, true>(sm, tw, ptab);
     } else {
 #pragma unroll 1
       for (int p = 0; p < NP16; p++) pass16_rt<true>(sm, tw, ptab, p);
@@ -360,7 +370,7 @@ struct SmemFFT {
   __device__ static void inverse(C* sm, const TwiddleTab<C>& tw, const C* ptab) {
     pass_rem<false>(sm, tw);
     if constexpr (UNROLL_PASSES) {
-      pass16<2, false>(sm, tw, ptab);
+      if constexpr (NP16 > 2) pass16<2, false>(sm, tw, ptab);
       pass16<1, false>(sm, tw, ptab);
       pass16<0, false>(sm, tw, ptab);
     } else {

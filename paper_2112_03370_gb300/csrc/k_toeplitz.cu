@@ -490,10 +490,17 @@ __device__ __forceinline__ void fused_rem_pair(C* sm, const C* __restrict__ tab,
 
 // One overlap-save tile (CL = 1) or half a tile (CL = 2) per CTA.
 // LOGM: log2 of the complex points of the whole tile (L = 2^(LOGM + 1) real samples); the FP32
-// 2-CTA tiles use LOGM = kLogM + 1 (65536 samples, each CTA a 16384-point half)
+// 2-CTA tiles use LOGM = kLogM + 1 (65536 samples, each CTA a 16384-point half), the FP64 and df64
+// tiles of one CTA LOGM = 11 to 13 (choose_logm64).
+// CTA size: one radix-16 butterfly per thread and pass where that fits
+constexpr int tile_threads(int cl, int logm) {
+  const int ms = 1 << (logm - (cl == 2 ? 1 : 0));
+  return ms / 16 < kTileThreads ? ms / 16 : kTileThreads;
+}
 template <typename T, int CL, int MODE, bool MULTI = false, int LOGM = kLogM>
-__global__ void __launch_bounds__(kTileThreads, 1) k_tile(const TileArgs a_in) {
-  constexpr int NT = kTileThreads;
+__global__ void __launch_bounds__(tile_threads(CL, LOGM), kTileThreads / tile_threads(CL, LOGM)) k_tile(const TileArgs a_in) {
+  constexpr int NT = tile_threads(CL, LOGM);
+  constexpr bool SEG = CL == 1 && std::is_same<T, float>::value;   // walks segments of tiles
   using C = typename V2<T>::t;
   constexpr int MT = 1 << LOGM;   // complex points of the tile
   constexpr int LT = 2 * MT;      // real samples of the tile
@@ -521,7 +528,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile(const TileArgs a_in) {
   // both CTAs of a cluster read the same flag, so they leave together
   if (a.done != nullptr && a.done[(int64_t)rhs * a.done_stride] != 0) return;
   const C* __restrict__ tw_g = reinterpret_cast<const C*>(a.tw);
-  const TwiddleTab<C> tw = load_twiddle_tab<C, MT, NT>(tw_sm, tw_g);
+  const TwiddleTab<C> tw = load_twiddle_tab<C, MT, NT>(tw_sm, tw_g, LOGM < kLogM ? kM / MT : 1);
   const C* __restrict__ tab =
       reinterpret_cast<const C*>(a.tab) + ((int64_t)seg.tab * CL + rank) * MS;
   const T sc = (T)seg.scale;
@@ -533,7 +540,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile(const TileArgs a_in) {
   __syncthreads();
 
   float umax = 0.f;   // MODE_NINV_T df64 tiles: largest |u| this thread wrote
-  const int n_steps = (CL == 1) ? seg.n_steps : 1;   // only the FP32 kernel walks segments
+  const int n_steps = SEG ? seg.n_steps : 1;
   for (int step = 0; step < n_steps; step++) {
     TileDesc td = seg;
     td.in0 = seg.in0 + (int64_t)step * seg.vstep;
@@ -542,7 +549,24 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile(const TileArgs a_in) {
 
     // ---- gather: packed complex input (CL = 2: with the first radix-2 DIF step) ----
     // quad q holds complex values 2q, 2q + 1 (real samples in0 + 4q .. + 3)
-    if constexpr (CL == 1) {
+    if constexpr (CL == 1 && !SEG) {
+      for (int q0 = threadIdx.x; q0 < HALF_Q; q0 += NQ * NT) {
+        int64_t g[NQ];
+        T v[NQ][4];
+#pragma unroll
+        for (int u = 0; u < NQ; u++) g[u] = q0 + u * NT < HALF_Q ? td.in0 + 4 * (int64_t)(q0 + u * NT) : td.blk_hi;
+        gather_quads<T, MODE, NQ>(a, rhs, td, g, v);
+#pragma unroll
+        for (int u = 0; u < NQ; u++) {
+          const int q = q0 + u * NT;
+          if (q < HALF_Q) {
+            sm[smem_pad(2 * q)] = C{v[u][0], v[u][1]};
+            sm[smem_pad(2 * q + 1)] = C{v[u][2], v[u][3]};
+          }
+        }
+      }
+      __syncthreads();
+    } else if constexpr (CL == 1) {
       int q_first = 0;
       if (step > 0) {   // the previous tile's last L - vstep samples are this tile's first ones
         for (int n = threadIdx.x; n < 2 * halo_q; n += NT)
@@ -602,7 +626,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile(const TileArgs a_in) {
       __syncthreads();
     }
 
-    if constexpr (CL == 1 && LOGM == 14) {
+    if constexpr (SEG) {
       FFT::forward16(sm, tw, ptab);
       fused_rem_pair(sm, tab, sc);
       __syncthreads();
@@ -690,7 +714,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile(const TileArgs a_in) {
       cl.sync();
       other = cl.map_shared_rank(sm, rank ^ 1);
     }
-    if constexpr (CL == 1) {
+    if constexpr (SEG) {
       constexpr int NB = 8;
       const int n_lo = r_lo >> 1, n_hi = (r_hi + 1) >> 1;
       for (int n0 = n_lo + threadIdx.x; n0 < n_hi; n0 += NB * NT) {
@@ -726,8 +750,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile(const TileArgs a_in) {
             for (int h = 0; h < 2; h++) {
               const int n = 2 * q + h - rank * MS;      // local complex index
               C z = sm[smem_pad(n)];
-              const C o = other[smem_pad(n)];
-              z = (rank == 0) ? c_add(z, o) : c_sub(o, z);
+              if constexpr (CL == 2) {
+                const C o = other[smem_pad(n)];
+                z = (rank == 0) ? c_add(z, o) : c_sub(o, z);
+              }
               y[u][2 * h] = z.x;
               y[u][2 * h + 1] = z.y;
             }
@@ -778,7 +804,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile(const TileArgs a_in) {
     if constexpr (CL == 2) cg::this_cluster().sync();
     else __syncthreads();   // the next tile overwrites the buffer
   }
-  if constexpr (MODE == MODE_NINV_T && CL == 2 && std::is_same<T, df>::value) {
+  if constexpr (MODE == MODE_NINV_T && std::is_same<T, df>::value) {
     if (a.amax != nullptr) {   // non-negative floats order like their bit patterns
       for (int o = 16; o > 0; o >>= 1) umax = fmaxf(umax, __shfl_xor_sync(0xffffffffu, umax, o));
       if ((threadIdx.x & 31) == 0) atomicMax(a.amax + rhs, __float_as_uint(umax));
@@ -796,6 +822,17 @@ constexpr size_t kSmemBytes32Big =
 constexpr size_t kSmemBytes64 =
     (size_t)(smem_pad(kM / 2) + twiddle_tab_entries(kM) + SmemFFT<kLogM - 1, kM, kTileThreads>::kPassTabEntries) *
     sizeof(double2);
+
+// FP64 and df64 tiles of one CTA
+template <int LOGM>
+constexpr size_t smem64_of() {
+  return (size_t)(smem_pad(1 << LOGM) + twiddle_tab_entries(1 << LOGM) +
+                  SmemFFT<LOGM, (1 << LOGM), tile_threads(1, LOGM)>::kPassTabEntries) *
+         sizeof(double2);
+}
+static size_t smem64(int logm) {
+  return logm == 13 ? smem64_of<13>() : logm == 12 ? smem64_of<12>() : smem64_of<11>();
+}
 
 int tile_kernels_init() {
   static int done = 0;
@@ -816,6 +853,21 @@ int tile_kernels_init() {
   MM_SET((k_tile<double, 2, MODE_NINV>), kSmemBytes64);
   MM_SET((k_tile<df, 2, MODE_APPLY_T>), kSmemBytes64);
   MM_SET((k_tile<df, 2, MODE_NINV_T>), kSmemBytes64);
+  MM_SET((k_tile<double, 1, MODE_APPLY, false, 13>), smem64(13));
+  MM_SET((k_tile<double, 1, MODE_RHS, false, 13>), smem64(13));
+  MM_SET((k_tile<double, 1, MODE_NINV, false, 13>), smem64(13));
+  MM_SET((k_tile<double, 1, MODE_APPLY, false, 12>), smem64(12));
+  MM_SET((k_tile<double, 1, MODE_RHS, false, 12>), smem64(12));
+  MM_SET((k_tile<double, 1, MODE_NINV, false, 12>), smem64(12));
+  MM_SET((k_tile<double, 1, MODE_APPLY, false, 11>), smem64(11));
+  MM_SET((k_tile<double, 1, MODE_RHS, false, 11>), smem64(11));
+  MM_SET((k_tile<double, 1, MODE_NINV, false, 11>), smem64(11));
+  MM_SET((k_tile<df, 1, MODE_APPLY_T, false, 13>), smem64(13));
+  MM_SET((k_tile<df, 1, MODE_NINV_T, false, 13>), smem64(13));
+  MM_SET((k_tile<df, 1, MODE_APPLY_T, false, 12>), smem64(12));
+  MM_SET((k_tile<df, 1, MODE_NINV_T, false, 12>), smem64(12));
+  MM_SET((k_tile<df, 1, MODE_APPLY_T, false, 11>), smem64(11));
+  MM_SET((k_tile<df, 1, MODE_NINV_T, false, 11>), smem64(11));
   MM_SET((k_tile<float, 2, MODE_NINV_T, false, kLogM + 1>), kSmemBytes32Big);
 #undef MM_SET
   if (e == cudaSuccess) {
@@ -834,7 +886,7 @@ static cudaError_t launch_tiles(const TileArgs& a, size_t smem, cudaStream_t s) 
   if (n_cta > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)n_cta);
-  cfg.blockDim = dim3(kTileThreads);
+  cfg.blockDim = dim3(tile_threads(CL, LOGM));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -919,24 +971,34 @@ cudaError_t launch_tiles_fp32_multi(const TileArgs& a, int halo_samples, cudaStr
 
 int fp32_max_halo_samples() { return (int)((kSmemMax - kSmemBytes32) / sizeof(float)); }
 
+// FP64 and df64 tiles of 2^(logm + 1) samples: one CTA for logm 11 to 13, a 2-CTA cluster for 14
+template <typename T, int MODE>
+static cudaError_t launch_tiles64(int logm, const TileArgs& a, cudaStream_t s) {
+  if (logm == 14) return launch_tiles<T, 2, MODE>(a, kSmemBytes64, s);
+  if (logm == 13) return launch_tiles<T, 1, MODE, false, 13>(a, smem64(13), s);
+  if (logm == 12) return launch_tiles<T, 1, MODE, false, 12>(a, smem64(12), s);
+  if (logm == 11) return launch_tiles<T, 1, MODE, false, 11>(a, smem64(11), s);
+  return cudaErrorInvalidValue;
+}
+
 // df64 tiles: input t (float2 hi/lo pairs [nrhs][x_stride], x_stride a multiple of 4), output
 // accumulated into the FP64 map y [nrhs][n_obs][4]
-cudaError_t launch_tiles_df(const TileArgs& a, cudaStream_t s) {
+cudaError_t launch_tiles_df(int logm, const TileArgs& a, cudaStream_t s) {
   if (a.x_stride % 4 != 0) return cudaErrorInvalidValue;
-  return launch_tiles<df, 2, MODE_APPLY_T>(a, kSmemBytes64, s);
+  return launch_tiles64<df, MODE_APPLY_T>(logm, a, s);
 }
 
 // df64 u = N^-1 t: t and u (hi, lo) pairs [nrhs][x_stride] / [nrhs][y_stride] (multiples of 4),
 // a.amax (per column, zeroed by the caller) receives the bits of max |u|
-cudaError_t launch_ninv_df(const TileArgs& a, cudaStream_t s) {
+cudaError_t launch_ninv_df(int logm, const TileArgs& a, cudaStream_t s) {
   if (a.x_stride % 4 != 0 || a.y_stride % 4 != 0) return cudaErrorInvalidValue;
-  return launch_tiles<df, 2, MODE_NINV_T>(a, kSmemBytes64, s);
+  return launch_tiles64<df, MODE_NINV_T>(logm, a, s);
 }
 
-cudaError_t launch_tiles_fp64(int mode, const TileArgs& a, cudaStream_t s) {
-  if (mode == MODE_APPLY) return launch_tiles<double, 2, MODE_APPLY>(a, kSmemBytes64, s);
-  if (mode == MODE_RHS) return launch_tiles<double, 2, MODE_RHS>(a, kSmemBytes64, s);
-  if (mode == MODE_NINV) return launch_tiles<double, 2, MODE_NINV>(a, kSmemBytes64, s);
+cudaError_t launch_tiles_fp64(int logm, int mode, const TileArgs& a, cudaStream_t s) {
+  if (mode == MODE_APPLY) return launch_tiles64<double, MODE_APPLY>(logm, a, s);
+  if (mode == MODE_RHS) return launch_tiles64<double, MODE_RHS>(logm, a, s);
+  if (mode == MODE_NINV) return launch_tiles64<double, MODE_NINV>(logm, a, s);
   return cudaErrorInvalidValue;
 }
 
@@ -981,25 +1043,28 @@ cudaError_t launch_spectra(const double* band_rows, int32_t n_tab, int32_t lambd
 }
 
 // (a_k, b_k) of the pair update for every storage position of a tile of 2^LOGM complex points
-// split over CL CTAs (the storage order of each CTA's transform)
+// split over CL CTAs (the storage order of each CTA's transform).  H and costab belong to the
+// 2^(LOGM + 1)-sample circulant, or to the kL-sample one for shorter tiles, which sample the same
+// symbol more coarsely.
 template <int CL, int LOGM>
 __global__ void k_pair_table(const double* __restrict__ H, const double* __restrict__ costab,
                              int32_t n_tab, void* __restrict__ out, int fp32) {
   constexpr int M = 1 << LOGM, L = 2 * M;
   constexpr int LOGMS = LOGM - (CL == 2 ? 1 : 0);
   constexpr int MS = 1 << LOGMS;
-  using FFT = SmemFFT<LOGMS, M, kTileThreads>;
+  using FFT = SmemFFT<LOGMS, M, tile_threads(CL, LOGM)>;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)n_tab * M) return;
   const int tab = (int)(idx / M);
   const int rem = (int)(idx % M);
   const int rank = rem / MS, j = rem % MS;
   const int k = CL * FFT::freq_of(j) + rank;       // global frequency, 0 <= k < M
-  const double* h = H + (int64_t)tab * (M + 1);
-  const double S = 0.5 * (h[k] + h[M - k]);
-  const double D = 0.5 * (h[k] - h[M - k]);
-  const double cth = costab[k];
-  const double sth = costab[(k - L / 4) & (L - 1)];
+  constexpr int HS = LOGM < kLogM ? kM / M : 1;
+  const double* h = H + (int64_t)tab * (M * HS + 1);
+  const double S = 0.5 * (h[k * HS] + h[(M - k) * HS]);
+  const double D = 0.5 * (h[k * HS] - h[(M - k) * HS]);
+  const double cth = costab[k * HS];
+  const double sth = costab[(k * HS - L * HS / 4) & (L * HS - 1)];
   const double inv_m = 1.0 / (double)M;
   const double av = (S - D * sth) * inv_m;
   const double bv = D * cth * inv_m;
@@ -1007,14 +1072,16 @@ __global__ void k_pair_table(const double* __restrict__ H, const double* __restr
   else reinterpret_cast<double2*>(out)[idx] = make_double2(av, bv);
 }
 
-cudaError_t launch_pair_tables(const double* H, int32_t n_tab, const double* costab, double2* tab64,
+cudaError_t launch_pair_tables(const double* H, int32_t n_tab, const double* costab, int logm64, double2* tab64,
                                float2* tab32, cudaStream_t s) {
   if (n_tab == 0) return cudaSuccess;
-  const int64_t n = (int64_t)n_tab * kM;
-  const int nt = 256;
-  const unsigned nb = (unsigned)((n + nt - 1) / nt);
-  k_pair_table<kCl64, kLogM><<<nb, nt, 0, s>>>(H, costab, n_tab, tab64, 0);
-  k_pair_table<kCl32, kLogM><<<nb, nt, 0, s>>>(H, costab, n_tab, tab32, 1);
+  auto blocks = [&](int logm) { return (unsigned)((((int64_t)n_tab << logm) + 255) / 256); };
+  k_pair_table<kCl32, kLogM><<<blocks(kLogM), 256, 0, s>>>(H, costab, n_tab, tab32, 1);
+  if (logm64 == 14) k_pair_table<2, 14><<<blocks(14), 256, 0, s>>>(H, costab, n_tab, tab64, 0);
+  else if (logm64 == 13) k_pair_table<1, 13><<<blocks(13), 256, 0, s>>>(H, costab, n_tab, tab64, 0);
+  else if (logm64 == 12) k_pair_table<1, 12><<<blocks(12), 256, 0, s>>>(H, costab, n_tab, tab64, 0);
+  else if (logm64 == 11) k_pair_table<1, 11><<<blocks(11), 256, 0, s>>>(H, costab, n_tab, tab64, 0);
+  else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 

@@ -420,6 +420,30 @@ int choose_ninv_logm(const std::vector<int64_t>& off, int lam, bool shared) {
   return best;
 }
 
+// Tile size of the FP64 and df64 tiles: the least estimated time over 4096- to 32768-sample tiles.  Their
+// arithmetic bounds them (FP64 at 1/64 of the FP32 rate; a double-float operation is about ten FP32 ones),
+// so a tile costs its points times the butterfly levels (and about three levels of pointwise work)
+// wherever it runs, and a 32768-sample tile takes two SMs.  4 blocks x 65,536 samples, lambda 1024, FP64 A
+// x: 297 us on 12 tiles of 32768 samples (24 SMs), 60 us on 132 of 4096.
+int choose_logm64(const std::vector<int64_t>& off, int lam) {
+  int best = kLogM;
+  double best_t = 1e300;
+  for (int logm = kLogM; logm >= 11; logm--) {
+    const int64_t vmax = ((int64_t)2 << logm) - 2 * (int64_t)lam - 4;
+    if (vmax <= 0) break;
+    int64_t n = 0;
+    for (size_t b = 0; b + 1 < off.size(); b++) n += (off[b + 1] - off[b] + vmax - 1) / vmax;
+    const int64_t sms = logm == kLogM ? sm_count() / 2 : sm_count();
+    const double work = (double)(1 << (logm == kLogM ? logm - 1 : logm)) * (logm + 3);
+    const double t = (double)((n + sms - 1) / sms) * work;
+    if (t < best_t) {
+      best_t = t;
+      best = logm;
+    }
+  }
+  return best;
+}
+
 // FP32 segments of up to `steps` consecutive tiles (replacing previous ones: captured graphs
 // must be captured again): of the fused tiles, and of k_ninv32 when it is built (at most 4 tiles there,
 // where walking only spares the twiddle tables)
@@ -755,13 +779,14 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
   MM_TRY(scr.alloc(&costab_d, kL));
   MM_TRY(scr.alloc(&H, (size_t)P->n_tab * (kM + 1)));
   MM_TRY(dalloc(P, &P->tab32, (size_t)P->n_tab * kM));
-  MM_TRY(dalloc(P, &P->tab64, (size_t)P->n_tab * kM));
+  P->logm64 = choose_logm64(P->block_off, lam);
+  MM_TRY(dalloc(P, &P->tab64, (size_t)P->n_tab << P->logm64));
   MM_TRY(dalloc(P, &P->tw32, kM));
   MM_TRY(dalloc(P, &P->tw64, kM));
   MM_CUDA(cudaMemcpyAsync(rows_d, rows.data(), rows.size() * sizeof(double), cudaMemcpyHostToDevice, s));
   MM_CUDA(cudaMemcpyAsync(costab_d, costab.data(), kL * sizeof(double), cudaMemcpyHostToDevice, s));
   MM_CUDA(launch_spectra(rows_d, P->n_tab, lam, H, costab_d, s));
-  MM_CUDA(launch_pair_tables(H, P->n_tab, costab_d, P->tab64, P->tab32, s));
+  MM_CUDA(launch_pair_tables(H, P->n_tab, costab_d, P->logm64, P->tab64, P->tab32, s));
   MM_CUDA(launch_twiddles(P->tw64, P->tw32, costab_d, s));
   // FP32 N^-1 on 65536-sample tiles (2-CTA clusters) when a 32768-sample tile would keep less than
   // 5/8 of its outputs: tables built here, used when mm_autotune measures them faster
@@ -805,15 +830,16 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
     MM_CUDA(cudaStreamSynchronize(s));   // host vectors go out of scope
   }
   if (P->df64) {
-    MM_TRY(dalloc(P, &P->tabdf, (size_t)P->n_tab * kM));
+    MM_TRY(dalloc(P, &P->tabdf, (size_t)P->n_tab << P->logm64));
     MM_TRY(dalloc(P, &P->twdf, kM));
-    MM_CUDA(launch_c64_to_df(P->tab64, (int64_t)P->n_tab * kM, P->tabdf, s));
+    MM_CUDA(launch_c64_to_df(P->tab64, (int64_t)P->n_tab << P->logm64, P->tabdf, s));
     MM_CUDA(launch_c64_to_df(P->tw64, kM, P->twdf, s));
   }
   std::vector<double> Hh((size_t)P->n_tab * (kM + 1));
   MM_CUDA(cudaMemcpyAsync(Hh.data(), H, Hh.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
 
-  std::vector<TileDesc> tiles = make_tiles(P->block_off, bt, lam, 1, 0, nullptr);
+  std::vector<TileDesc> tiles = make_tiles(P->block_off, bt, lam, 1, 0, nullptr, (int64_t)2 << P->logm64);
+  P->n_tiles32 = (int64_t)make_tiles(P->block_off, bt, lam, 1, 0, nullptr).size();
   P->n_tiles = (int64_t)tiles.size();
   MM_TRY(dalloc(P, &P->tiles, tiles.size()));
   MM_CUDA(cudaMemcpyAsync(P->tiles, tiles.data(), tiles.size() * sizeof(TileDesc), cudaMemcpyHostToDevice, s));
@@ -829,7 +855,7 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
   P->steps_given = d->tile_steps > 0;
   // FP32 segments: enough of them to keep every SM busy (about 8 per SM), at most 16 tiles each
   const int64_t steps = d->tile_steps > 0 ? d->tile_steps
-                                           : std::max<int64_t>(1, std::min<int64_t>(16, P->n_tiles / (8 * sm_count())));
+                                           : std::max<int64_t>(1, std::min<int64_t>(16, P->n_tiles32 / (8 * sm_count())));
   MM_TRY(build_segments(P, (int)steps, s));
   MM_CUDA(cudaStreamSynchronize(s));
 
@@ -971,14 +997,14 @@ int df_ninv_point(Plan* P, int g, const int32_t* done, int done_stride, double* 
   a.done_stride = done_stride;
   if (!P->groups) {
     a.y = y4;
-    MM_CUDA(launch_tiles_df(a, s));
+    MM_CUDA(launch_tiles_df(P->logm64, a, s));
     return MM_OK;
   }
   MM_CUDA(cudaMemsetAsync(P->amax, 0, (size_t)g * sizeof(uint32_t), s));
   a.y = P->udf;
   a.y_stride = df_stride(P);
   a.amax = P->amax;
-  MM_CUDA(launch_ninv_df(a, s));
+  MM_CUDA(launch_ninv_df(P->logm64, a, s));
   MM_CUDA(launch_point_win_df(P->groups, P->n_groups, P->win_size, P->block_off_dev, P->slot, P->slot_pix, P->wdf, P->udf,
                               df_stride(P), P->amax, g, done, done_stride, y4, P->n_obs * 4, s));
   return MM_OK;
@@ -1048,7 +1074,7 @@ int apply64_internal(Plan* P, const double* x4, double* y4, int nrhs, cudaStream
   a.y_stride = P->n_obs * 4;
   a.done = done;
   a.done_stride = done_stride;
-  MM_CUDA(launch_tiles_fp64(MODE_APPLY, a, s));
+  MM_CUDA(launch_tiles_fp64(P->logm64, MODE_APPLY, a, s));
   return MM_OK;
 }
 
@@ -1950,7 +1976,7 @@ int mm_apply_Ninv(mm_plan_t plan, const double* t, double* y, void* stream) {
   a.x_stride = P->N;
   a.y = y;
   a.y_stride = P->N;
-  MM_CUDA(launch_tiles_fp64(MODE_NINV, a, s));
+  MM_CUDA(launch_tiles_fp64(P->logm64, MODE_NINV, a, s));
   return MM_OK;
 }
 
@@ -2049,7 +2075,7 @@ int mm_rhs(mm_plan_t plan, const void* d, int d_is_fp32, int nrhs, double* b, vo
       a.nrhs = nrhs;
       a.x = d;
       a.y = P->map64_out;
-      MM_CUDA(launch_tiles_fp64(MODE_RHS, a, s));
+      MM_CUDA(launch_tiles_fp64(P->logm64, MODE_RHS, a, s));
     } else {   // one column at a time through the plan's N-sample FP64 buffer
       MM_TRY(ensure_td(P));
       for (int r = 0; r < nrhs; r++) {
@@ -2058,7 +2084,7 @@ int mm_rhs(mm_plan_t plan, const void* d, int d_is_fp32, int nrhs, double* b, vo
         a.nrhs = 1;
         a.x = P->td_a;
         a.y = P->map64_out + (size_t)r * P->n_obs * 4;
-        MM_CUDA(launch_tiles_fp64(MODE_RHS, a, s));
+        MM_CUDA(launch_tiles_fp64(P->logm64, MODE_RHS, a, s));
       }
     }
   }
@@ -2448,7 +2474,7 @@ int mm_autotune(mm_plan_t plan, int max_width, mm_tune_info* out, void* stream) 
   int best_steps = P->tile_steps;
   P->steps_given = true;
   for (int v : steps_c) {
-    if (v > 1 && P->n_tiles / v < sm_count()) continue;   // fewer segments than SMs
+    if (v > 1 && P->n_tiles32 / v < sm_count()) continue;   // fewer segments than SMs
     MM_TRY(build_segments(P, v, P->stream));
     double ms = 0.0;
     bool pass = false;

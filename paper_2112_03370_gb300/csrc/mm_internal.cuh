@@ -221,15 +221,17 @@ struct Plan {
   // Toeplitz FFT state
   int32_t n_tab = 0;
   float2* tab32 = nullptr;             // [n_tab][M]
-  double2* tab64 = nullptr;            // [n_tab][M]
+  double2* tab64 = nullptr;            // [n_tab][2^logm64]
   float2* tw32 = nullptr;              // [M]
   double2* tw64 = nullptr;             // [M]
-  float4* tabdf = nullptr;             // [n_tab][M] df64 pair tables (df64 plans)
+  float4* tabdf = nullptr;             // [n_tab][2^logm64] df64 pair tables (df64 plans)
   float4* twdf = nullptr;              // [M] df64 twiddles
   float2* tdf = nullptr;               // [nrhs][N4] un-pointed df64 input, N4 = N rounded up to 4
   size_t tdf_cap = 0;
   float4* mapdf = nullptr;             // [nrhs][n_obs][2] df64 map: (I hi, I lo, Q hi, Q lo), (U hi, U lo, 0, 0)
   size_t mapdf_cap = 0;
+  int logm64 = kLogM;                  // FP64 and df64 tiles: log2 of their complex points
+  int64_t n_tiles32 = 0;               // 32768-sample tiles of the blocks
   TileDesc* tiles = nullptr;           // FP64 tiles (one per descriptor)
   int64_t n_tiles = 0;
   TileDesc* segs = nullptr;            // FP32 segments (several tiles per descriptor)
@@ -380,7 +382,8 @@ cudaError_t launch_validate(const int32_t* pix, const float* psi, int64_t N, int
 cudaError_t launch_spectra(const double* band_rows, int32_t n_tab, int32_t lambda,
                            double* H /* [n_tab][M+1] */, const double* costab /* [L] */,
                            cudaStream_t s, int logm = kLogM);
-cudaError_t launch_pair_tables(const double* H, int32_t n_tab, const double* costab,
+// pair tables of the FP64 / df64 tiles of 2^(logm64 + 1) samples and of the fused FP32 tiles
+cudaError_t launch_pair_tables(const double* H, int32_t n_tab, const double* costab, int logm64,
                                double2* tab64, float2* tab32, cudaStream_t s);
 // FP32 pair tables of the 65536-sample 2-CTA tiles: tab32 [n_tab][2 kM]
 cudaError_t launch_pair_table32_big(const double* H, int32_t n_tab, const double* costab, float2* tab32,
@@ -412,7 +415,7 @@ int ninv32_init();
 cudaError_t launch_unpoint32(const int32_t* lpix, const float2* w32, int64_t N, const float* x4,
                              int64_t x_stride, int nrhs, const int32_t* done, int done_stride, float* t,
                              int64_t t_stride, cudaStream_t s);
-cudaError_t launch_tiles_fp64(int mode, const TileArgs& a, cudaStream_t s);
+cudaError_t launch_tiles_fp64(int logm, int mode, const TileArgs& a, cudaStream_t s);
 
 // pixel windows (k_window.cu)
 // count (slot_tab == nullptr: n_slots of every group, -1 when over kWinCap) or fill (slots and
@@ -462,9 +465,9 @@ cudaError_t launch_point_sorted_multi(const PGroup* groups, int64_t n_groups, co
 // multiprocessors of the current device (cached per device)
 int sm_count();
 // df64 tiles and their data preparation (k_df64.cu)
-cudaError_t launch_tiles_df(const TileArgs& a, cudaStream_t s);
+cudaError_t launch_tiles_df(int logm, const TileArgs& a, cudaStream_t s);
 // df64 u = N^-1 t (pairs in, pairs out), per-column max |u| into a.amax
-cudaError_t launch_ninv_df(const TileArgs& a, cudaStream_t s);
+cudaError_t launch_ninv_df(int logm, const TileArgs& a, cudaStream_t s);
 cudaError_t launch_weights_df(const float* psi, int64_t N, float4* wdf, cudaStream_t s);
 cudaError_t launch_c64_to_df(const double2* in, int64_t n, float4* out, cudaStream_t s);
 cudaError_t launch_map_to_df(const double* m4, int64_t n_pix4, float4* out, cudaStream_t s);
