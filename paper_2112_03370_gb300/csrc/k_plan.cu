@@ -85,16 +85,14 @@ __global__ void k_bd_accum(const int32_t* __restrict__ pix, const double2* __res
       }
       continue;
     }
-    // first lane of this lane's run of equal pixels (a max-scan of the run heads)
-    int head = (lane == 0 || p_prev != p) ? lane : 0;
-#pragma unroll
+    // first lane of this lane's run of equal pixels
+    const uint32_t heads = __ballot_sync(0xffffffffu, lane == 0 || p_prev != p);
+    const int head = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+    // segmented inclusive sums: the run's last lane holds the run's totals.  Only as many steps as the
+    // warp's longest run takes: the six FP64 additions of a step cost about as much as a sample's products
+    // (16.8M samples in runs of 2: 1.17 ms with all five steps, 0.40 ms now)
     for (int o = 1; o < 32; o <<= 1) {
-      const int h = __shfl_up_sync(0xffffffffu, head, o);
-      if (lane >= o) head = max(head, h);
-    }
-    // segmented inclusive sums: the run's last lane holds the run's totals
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
+      if (!__any_sync(0xffffffffu, lane - head >= o)) break;
 #pragma unroll
       for (int k = 0; k < 6; k++) {
         const double t = __shfl_up_sync(0xffffffffu, v[k], o);
@@ -302,12 +300,6 @@ cudaError_t launch_localize(const int32_t* pix, const int32_t* keep, const int32
   return cudaGetLastError();
 }
 
-// (cos 2psi, sin 2psi) once per sample in FP64 (the FP64 pipe runs at 1/64 of the FP32 rate, so the
-// sine and cosine are taken once): w64 as is, w32 as their FP32 roundings, wdf (if non-null) split
-// into df64 (hi, lo) pairs
-// One FP64 sincos of 2 psi per sample: the FP64 weights, their FP32 roundings, (wdf non-null) their
-// df64 split, and the angle 2 psi reduced to [-pi, pi] in FP64 and rounded once to FP32 (the FP32
-// window kernels evaluate the weights from it in registers).
 // cos(k pi/32), sin(k pi/32), k = 0 .. 63 (values of the circular functions rounded to FP64)
 __device__ const double2 kSinCosPi32[64] = {
     {1.0, 0.0}, {0.9951847266721969, 0.0980171403295606},
@@ -343,50 +335,84 @@ __device__ const double2 kSinCosPi32[64] = {
     {0.9238795325112867, -0.3826834323650898}, {0.9569403357322088, -0.2902846772544624},
     {0.9807852804032304, -0.19509032201612828}, {0.9951847266721969, -0.0980171403295606}};
 
-// (cos x, sin x) in FP64 by table lookup and angle addition (the table-driven method of
-// P. T. P. Tang, ACM TOMS 1989-91): x = k pi/32 + r with k = rint(32 x / pi) and r = x - k pi/32
-// by a two-constant Cody-Waite reduction (pi/32 = H + L, H = fl64(pi/32): k H is taken exactly
-// inside one FMA, k L has an error far below 1e-30 for |k| < 2^40); |r| <= pi/64, where the Taylor
-// series of sin r to r^9 and of cos r to r^8 leave truncation errors below 1e-19; then
+// FP64 -> FP32, rounded to nearest even, by moving and rounding the encoding with integer instructions (the
+// conversion instruction runs on the FP64 pipe, 1/64 of the FP32 rate).  |d| below 2^-126 gives a signed zero,
+// magnitudes of 2^128 and more and NaN do not occur here (weights and their remainders).
+__device__ __forceinline__ float f64_to_f32_bits(double d) {
+  const uint64_t u = (uint64_t)__double_as_longlong(d);
+  const uint32_t sign = (uint32_t)(u >> 32) & 0x80000000u;
+  const uint64_t mag = u & 0x7fffffffffffffffull;
+  if (mag < ((uint64_t)(1023 - 126) << 52)) return __uint_as_float(sign);
+  const uint64_t r = mag + 0x0fffffffull + ((mag >> 29) & 1);   // round the 29 dropped bits, ties to even
+  return __uint_as_float(sign | ((uint32_t)(r >> 29) - (896u << 23)));
+}
+
+// (cos x, sin x), x = 2 psi, in FP64 by table lookup and angle addition (the table-driven method of
+// P. T. P. Tang, ACM TOMS 1989-91): x = k pi/32 + r with k = rint(32 x / pi) and r = x - k pi/32 by a
+// two-constant Cody-Waite reduction (pi/32 = H + L, H = fl64(pi/32); k H is taken exactly inside one FMA);
 //   cos x = C_k cos r - S_k sin r,  sin x = S_k cos r + C_k sin r,  (C_k, S_k) = table[k mod 64].
-// About 20 FP64 operations instead of a general sincos (on GB300 FP64 runs at 1/64 of the FP32
-// rate, and the plan spends most of this kernel's time there).
-__device__ __forceinline__ void sincos_tab(double x, double& sn, double& cs) {
-  if (!(fabs(x) < 1e9)) {   // far outside any angle a scan produces: the general routine
-    sincos(x, &sn, &cs);
+// GB300 runs FP64, and conversions to and from it, at 1/64 of the FP32 rate.  FP64 is kept where the result's
+// 53 bits are formed (the reduction, r + (sin r - r), 1 + (cos r - 1) and the four products); the small parts
+// sin r - r and cos r - 1 (below 2e-5 and 1.3e-3 for |r| <= pi/64 and a little) come from double-float
+// Taylor series on the FP32 pipes, 48 bits of them being below 2^-57 absolute.  Within 1.6e-16 of the exact
+// values, 5.7e-17 rms, in a CPU check against 113-bit arithmetic over |psi| < 16384 (with the series in FP64:
+// 1.5e-16, 5.7e-17 rms).  16.8M samples, all outputs: 1.06 ms with the series in FP64 -> 0.42 ms.
+__device__ __forceinline__ void sincos_x2(float psi, double& sn, double& cs) {
+  const float x = 2.f * psi;   // exact
+  if (!(fabsf(x) < 32768.f)) {   // outside any angle a scan produces: the general routine
+    sincos((double)psi * 2.0, &sn, &cs);
     return;
   }
   constexpr double kH = 0.09817477042468103;       // fl64(pi / 32)
   constexpr double kL = 3.827021247335479e-18;     // pi / 32 - kH
-  constexpr double k32OverPi = 10.185916357881302;  // 32 / pi
-  const double kd = rint(x * k32OverPi);
-  double r = fma(-kd, kH, x);
-  r = fma(-kd, kL, r);
-  const double z = r * r;
-  const double sr = r * fma(z, fma(z, fma(z, fma(z, 1.0 / 362880.0, -1.0 / 5040.0), 1.0 / 120.0), -1.0 / 6.0), 1.0);
-  const double cr =
-      fma(z, fma(z, fma(z, fma(z, 1.0 / 40320.0, -1.0 / 720.0), 1.0 / 24.0), -0.5), 1.0);
-  const double2 t = kSinCosPi32[(int)((long long)kd & 63)];
+  const float kf = rintf(x * 10.185916357881302f);   // 32 / pi
+  const double kd = f32_to_f64_bits(kf);
+  const double r = fma(-kd, kL, fma(-kd, kH, f32_to_f64_bits(x)));
+  const float rh = f64_to_f32_bits(r);
+  const df rd = df_make(rh, f64_to_f32_bits(r - f32_to_f64_bits(rh)));
+  const df z = rd * rd;
+  const float zh = z.hi;
+  // sin r - r = r z (-1/6 + z (1/120 + z (-1/5040 + z / 362880)))
+  const df sp = df(-1.0 / 6.0) + z * (df(1.0 / 120.0) + df_make(zh * __fmaf_rn(zh, 2.7557319e-6f, -1.9841270e-4f), 0.f));
+  const df dsn = rd * (z * sp);
+  // cos r - 1 = z (-1/2 + z (1/24 + z (-1/720 + z / 40320)))
+  const df cp = df(1.0 / 24.0) + df_make(zh * __fmaf_rn(zh, 2.4801587e-5f, -1.3888889e-3f), 0.f);
+  const df dcs = z * (df(-0.5) + z * cp);
+  const double sr = r + df_to_double(dsn), cr = 1.0 + df_to_double(dcs);
+  const double2 t = kSinCosPi32[(int)kf & 63];
   cs = fma(t.x, cr, -t.y * sr);
   sn = fma(t.y, cr, t.x * sr);
 }
 
+// One evaluation of (cos 2 psi, sin 2 psi) per sample: the FP64 weights, their FP32 roundings, (wdf non-null)
+// their df64 split, and the angle 2 psi reduced to [-pi, pi] and rounded to FP32 (the FP32 window kernels
+// evaluate the weights from it in registers).
 __global__ void k_weights(const float* __restrict__ psi, int64_t N, double2* __restrict__ w64,
                           float2* __restrict__ w32, float4* __restrict__ wdf, float* __restrict__ ang2) {
   constexpr double kTwoPi = 6.283185307179586476925;
+  constexpr float kP0 = (float)kTwoPi, kP1 = (float)(kTwoPi - (double)kP0);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const double a = 2.0 * (double)psi[i];
+    const float p = psi[i];
     double s, c;
-    sincos_tab(a, s, c);
+    sincos_x2(p, s, c);
     w64[i] = make_double2(c, s);
-    w32[i] = make_float2((float)c, (float)s);
-    if (wdf) {
-      const df dc(c), ds(s);
-      wdf[i] = make_float4(dc.hi, dc.lo, ds.hi, ds.lo);
-    }
+    const float ch = f64_to_f32_bits(c), sh = f64_to_f32_bits(s);
+    w32[i] = make_float2(ch, sh);
+    if (wdf)
+      wdf[i] = make_float4(ch, f64_to_f32_bits(c - f32_to_f64_bits(ch)), sh, f64_to_f32_bits(s - f32_to_f64_bits(sh)));
     if (ang2) {
-      ang2[i] = (float)fma(-rint(a * (1.0 / kTwoPi)), kTwoPi, a);
+      const float x = 2.f * p;
+      if (fabsf(x) < 32768.f) {   // x - k 2 pi, the products with 2 pi in two FP32 parts, error-free sums
+        const float k = rintf(x * 0.15915494f);
+        const float p0 = __fmul_rn(k, kP0), e0 = __fmaf_rn(k, kP0, -p0);
+        float a, b;
+        two_sum(x, -p0, a, b);
+        ang2[i] = __fadd_rn(a, __fadd_rn(b, -__fmaf_rn(k, kP1, e0)));
+      } else {
+        const double a = 2.0 * (double)p;
+        ang2[i] = (float)fma(-rint(a * (1.0 / kTwoPi)), kTwoPi, a);
+      }
     }
   }
 }

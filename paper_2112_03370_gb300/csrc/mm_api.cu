@@ -785,7 +785,9 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
   MM_TRY(dalloc(P, &P->tw64, kM));
   MM_CUDA(cudaMemcpyAsync(rows_d, rows.data(), rows.size() * sizeof(double), cudaMemcpyHostToDevice, s));
   MM_CUDA(cudaMemcpyAsync(costab_d, costab.data(), kL * sizeof(double), cudaMemcpyHostToDevice, s));
-  MM_CUDA(launch_spectra(rows_d, P->n_tab, lam, H, costab_d, s));
+  double2* spec = nullptr;
+  MM_TRY(scr.alloc(&spec, spectra_scratch(P->n_tab)));
+  MM_CUDA(launch_spectra(rows_d, P->n_tab, lam, H, costab_d, spec, s));
   MM_CUDA(launch_pair_tables(H, P->n_tab, costab_d, P->logm64, P->tab64, P->tab32, s));
   MM_CUDA(launch_twiddles(P->tw64, P->tw32, costab_d, s));
   // FP32 N^-1 on 65536-sample tiles (2-CTA clusters) when a 32768-sample tile would keep less than
@@ -802,7 +804,9 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
     MM_TRY(dalloc(P, &P->tab32_big, (size_t)P->n_tab * mb));
     MM_TRY(dalloc(P, &P->tw32_big, mb));
     MM_CUDA(cudaMemcpyAsync(cb_d, cb.data(), lb * sizeof(double), cudaMemcpyHostToDevice, s));
-    MM_CUDA(launch_spectra(rows_d, P->n_tab, lam, Hb, cb_d, s, kLogM + 1));
+    double2* spec_b = nullptr;
+    MM_TRY(scr.alloc(&spec_b, spectra_scratch(P->n_tab, kLogM + 1)));
+    MM_CUDA(launch_spectra(rows_d, P->n_tab, lam, Hb, cb_d, spec_b, s, kLogM + 1));
     MM_CUDA(launch_pair_table32_big(Hb, P->n_tab, cb_d, P->tab32_big, s));
     MM_CUDA(launch_twiddles(nullptr, P->tw32_big, cb_d, s, kLogM + 1));
     const std::vector<TileDesc> sb = make_tiles(P->block_off, bt, lam, 1, 0, nullptr, lb);

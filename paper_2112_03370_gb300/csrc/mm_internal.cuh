@@ -378,10 +378,12 @@ cudaError_t launch_weights(const float* psi, int64_t N, double2* w64, float2* w3
                            cudaStream_t s);
 cudaError_t launch_validate(const int32_t* pix, const float* psi, int64_t N, int64_t n_pix,
                             int32_t* bad, cudaStream_t s);
-// spectra of the L-point circulants, L = 2^(logm + 1): H [n_tab][M + 1], costab [L]
+// spectra of the L-point circulants, L = 2^(logm + 1): H [n_tab][M + 1], costab [L], scratch
+// [spectra_scratch(n_tab, logm)]
+size_t spectra_scratch(int32_t n_tab, int logm = kLogM);
 cudaError_t launch_spectra(const double* band_rows, int32_t n_tab, int32_t lambda,
                            double* H /* [n_tab][M+1] */, const double* costab /* [L] */,
-                           cudaStream_t s, int logm = kLogM);
+                           double2* scratch, cudaStream_t s, int logm = kLogM);
 // pair tables of the FP64 / df64 tiles of 2^(logm64 + 1) samples and of the fused FP32 tiles
 cudaError_t launch_pair_tables(const double* H, int32_t n_tab, const double* costab, int logm64,
                                double2* tab64, float2* tab32, cudaStream_t s);
