@@ -3015,14 +3015,13 @@ int mm_deflation_build(mm_plan_t plan, const double* b, int m, int precision, vo
   const int64_t n = P->n_obs, n4 = 4 * n;
   Scratch scr;
   double *v_prev = nullptr, *v = nullptr, *wv = nullptr, *av = nullptr, *part = nullptr, *dot = nullptr;
-  double *alpha_d = nullptr, *beta_d = nullptr, *work = nullptr, *U = nullptr, *X = nullptr, *wvals = nullptr,
+  double *alpha_d = nullptr, *beta_d = nullptr, *X = nullptr, *wvals = nullptr,
          *E = nullptr, *gpart = nullptr;
   float *V32 = nullptr, *AV32 = nullptr, *x32 = nullptr, *y32 = nullptr;
   const int nblk = 4 * sm_count();
   MM_TRY(scr.alloc(&v_prev, n4)); MM_TRY(scr.alloc(&v, n4)); MM_TRY(scr.alloc(&wv, n4)); MM_TRY(scr.alloc(&av, n4));
   MM_TRY(scr.alloc(&part, nblk)); MM_TRY(scr.alloc(&dot, 2));
   MM_TRY(scr.alloc(&alpha_d, kMaxDefl)); MM_TRY(scr.alloc(&beta_d, kMaxDefl));
-  MM_TRY(scr.alloc(&work, kMaxDefl * kMaxDefl)); MM_TRY(scr.alloc(&U, kMaxDefl * kMaxDefl));
   MM_TRY(scr.alloc(&X, kMaxDefl * kMaxDefl)); MM_TRY(scr.alloc(&wvals, kMaxDefl));
   MM_TRY(scr.alloc(&E, kMaxDefl * kMaxDefl));
   MM_TRY(scr.alloc(&gpart, (size_t)blk_ctas() * kMaxBlk * kMaxBlk));
@@ -3078,7 +3077,7 @@ int mm_deflation_build(mm_plan_t plan, const double* b, int m, int precision, vo
   for (int i = 0; i + 1 < k; i++) bpad[i] = betas[i];
   MM_CUDA(cudaMemcpyAsync(alpha_d, alphas.data(), k * sizeof(double), cudaMemcpyHostToDevice, s));
   MM_CUDA(cudaMemcpyAsync(beta_d, bpad.data(), kMaxDefl * sizeof(double), cudaMemcpyHostToDevice, s));
-  MM_CUDA(launch_tridiag_eig(alpha_d, beta_d, k, work, wvals, X, s));
+  MM_CUDA(launch_tridiag_eig(alpha_d, beta_d, k, wvals, X, s));
   // replace the plan's space
   DeflState* d = reinterpret_cast<DeflState*>(P->defl);
   if (!d) {
@@ -3095,9 +3094,8 @@ int mm_deflation_build(mm_plan_t plan, const double* b, int m, int precision, vo
   MM_CUDA(launch_bcombine(d->Z, 0, nullptr, k, V32, k, X, k, 1.0, 0, n, nullptr, blk_ctas(), nullptr, s));
   MM_CUDA(launch_bcombine(d->Zp, 0, nullptr, k, AV32, k, X, k, 1.0, 0, n, nullptr, blk_ctas(), nullptr, s));
   MM_CUDA(launch_bgram(d->Z, k, nullptr, d->Zp, 0, k, nullptr, n, gpart, blk_ctas(), E, s));
-  MM_CUDA(launch_pinv_sym(E, k, 1e-12, work, U, wvals + 0, d->Einv, s));
+  MM_CUDA(launch_pinv_sym(E, k, 1e-12, d->Einv, s));
   std::vector<double> th(k);
-  MM_CUDA(launch_tridiag_eig(alpha_d, beta_d, k, work, wvals, X, s));   // Ritz values again (wvals reused)
   MM_CUDA(cudaMemcpyAsync(th.data(), wvals, k * sizeof(double), cudaMemcpyDeviceToHost, s));
   MM_CUDA(cudaStreamSynchronize(s));
   d->theta = th;
@@ -3124,10 +3122,9 @@ int mm_deflation_build_apriori(mm_plan_t plan, int precision, void* stream) {
   const int64_t n = P->n_obs, n4 = 4 * n;
   Scratch scr;
   int32_t* hits = nullptr;
-  double *E = nullptr, *work = nullptr, *U = nullptr, *wvals = nullptr, *gpart = nullptr;
+  double *E = nullptr, *gpart = nullptr;
   MM_TRY(scr.alloc(&hits, (size_t)k * n));
-  MM_TRY(scr.alloc(&E, kMaxDefl * kMaxDefl)); MM_TRY(scr.alloc(&work, kMaxDefl * kMaxDefl));
-  MM_TRY(scr.alloc(&U, kMaxDefl * kMaxDefl)); MM_TRY(scr.alloc(&wvals, kMaxDefl));
+  MM_TRY(scr.alloc(&E, kMaxDefl * kMaxDefl));
   MM_TRY(scr.alloc(&gpart, (size_t)blk_ctas() * kMaxBlk * kMaxBlk));
   DeflState* d = reinterpret_cast<DeflState*>(P->defl);
   if (!d) {
@@ -3155,7 +3152,7 @@ int mm_deflation_build_apriori(mm_plan_t plan, int precision, void* stream) {
   }
   // E = Z^T Z', Einv = pinv(E)
   MM_CUDA(launch_bgram(d->Z, k, nullptr, d->Zp, 0, k, nullptr, n, gpart, blk_ctas(), E, s));
-  MM_CUDA(launch_pinv_sym(E, k, 1e-12, work, U, wvals, d->Einv, s));
+  MM_CUDA(launch_pinv_sym(E, k, 1e-12, d->Einv, s));
   MM_CUDA(cudaStreamSynchronize(s));
   d->theta.assign(k, 0.0);
   d->k = k;
