@@ -5,6 +5,7 @@
 // Search blocks (Z, A Z, P, A P, M R) are float32; X, R and every t x t matrix are float64.
 // Tall-skinny products run on the FP32 units (GB300's FP64 rate is 1/64 of FP32) with FP64
 // accumulation across CTAs; the solver's accuracy is restored by FP64 residual checks.
+#include "df64.cuh"
 #include "mm_block.cuh"
 #include "mm_internal.cuh"
 
@@ -21,7 +22,7 @@ constexpr int kNT = 256;
 
 // The same partial Gram products for small blocks (ta <= MA, tb <= MB): every thread streams its
 // pixels (grid-stride, coalesced) and keeps the ta tb dot products in registers; then a block
-// reduction in FP64.  (The staged kernel above keeps most threads idle when t is small.)
+// reduction in FP64.  (The staged kernel below keeps most threads idle when t is small.)
 template <typename TB, int MA, int MB>
 __global__ void __launch_bounds__(kNT) k_bgram_small(const float4* __restrict__ A, int ta,
                                                       const int* __restrict__ idx_a,
@@ -91,23 +92,29 @@ static void bgram_small(const float* A, int ta, const int* idx_a, const void* B,
                                                        reinterpret_cast<const float4*>(B), tb, idx_b, n, part);
 }
 
-// The same partial Gram products for wide blocks: 64 x 64 pairs over 256 threads, each thread a
-// 4 x 4 tile of (i, j) in registers; kGR pixels of both blocks staged per step as
-// [pixel][component][column] (rows padded to keep 16-byte alignment and spread the staging stores
-// over banks), so a thread's four a values and four b values of one pixel component are two
-// 16-byte shared loads for 16 FMAs.
+// The same partial Gram products for wide blocks, NC = 16, 32 or 64 columns on each side: each thread a
+// 4 x 4 tile of (i, j) in registers, (NC / 4)^2 threads for all pairs and 256 / that many groups of threads on
+// different pixels; kGR 64 / NC pixels of both blocks staged per step as [pixel][component][column] (rows
+// padded to keep 16-byte alignment and spread the staging stores over banks), so a thread's four a values
+// and four b values of one pixel component are two 16-byte shared loads for 16 FMAs.  The groups' totals
+// meet in FP64 at the end.  With 64-column tiles for 16 columns 240 of the 256 threads multiplied zeros and
+// added them in FP64: 65,536 pixels, 16 x 16 columns 88 -> 42 us.
 constexpr int kGR = 24;   // 2 x 19.6 KB of static shared memory
-constexpr int kGRow = kMaxBlk + 4;
-template <typename TB>
+template <typename TB, int NC>
 __global__ void __launch_bounds__(kNT) k_bgram_tiled(const float4* __restrict__ A, int ta,
                                                       const int* __restrict__ idx_a,
                                                       const TB* __restrict__ B, int tb,
                                                       const int* __restrict__ idx_b, int64_t n,
                                                       double* __restrict__ out_part) {
-  static_assert(kNT == 256 && kMaxBlk == 64, "16 x 16 threads of 4 x 4 pairs");
-  __shared__ __align__(16) float sa[kGR][3][kGRow];
-  __shared__ __align__(16) float sb[kGR][3][kGRow];
-  const int ti = threadIdx.x >> 4, tj = threadIdx.x & 15;
+  static_assert(kNT == 256 && kMaxBlk == 64 && (NC == 16 || NC == 32 || NC == 64), "256 threads of 4 x 4 pairs");
+  constexpr int kTiles = NC / 4, kGroups = kNT / (kTiles * kTiles), kPix = kGR * 64 / NC, kRow = NC + 4;
+  constexpr int kHalf = kPix * 3 * kRow;
+  static_assert(2 * kHalf * 4 >= NC * NC * 8, "the totals reuse the staging buffers");
+  __shared__ __align__(16) float smem[2 * kHalf];
+  float(*sa)[3][kRow] = reinterpret_cast<float(*)[3][kRow]>(smem);
+  float(*sb)[3][kRow] = reinterpret_cast<float(*)[3][kRow]>(smem + kHalf);
+  const int grp = threadIdx.x / (kTiles * kTiles), in = threadIdx.x % (kTiles * kTiles);
+  const int ti = in / kTiles, tj = in % kTiles;
   double tot[4][4];   // FP64 totals of the per-chunk FP32 sums (two-level summation)
 #pragma unroll
   for (int u = 0; u < 4; u++)
@@ -115,11 +122,11 @@ __global__ void __launch_bounds__(kNT) k_bgram_tiled(const float4* __restrict__ 
     for (int v = 0; v < 4; v++) tot[u][v] = 0.0;
   const int64_t per = (n + gridDim.x - 1) / gridDim.x;
   const int64_t p0 = (int64_t)blockIdx.x * per, p1 = min(n, p0 + per);
-  for (int64_t base = p0; base < p1; base += kGR) {
-    const int cnt = (int)min((int64_t)kGR, p1 - base);
+  for (int64_t base = p0; base < p1; base += kPix) {
+    const int cnt = (int)min((int64_t)kPix, p1 - base);
     // staging: consecutive threads take consecutive pixels of one column (coalesced loads)
-    for (int e = threadIdx.x; e < kGR * kMaxBlk; e += kNT) {
-      const int r = e % kGR, i = e / kGR;
+    for (int e = threadIdx.x; e < kPix * NC; e += kNT) {
+      const int r = e % kPix, i = e / kPix;
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
       if (r < cnt && i < ta) v = __ldg(A + (int64_t)(idx_a ? idx_a[i] : i) * n + base + r);
       sa[r][0][i] = v.x; sa[r][1][i] = v.y; sa[r][2][i] = v.z;
@@ -130,8 +137,9 @@ __global__ void __launch_bounds__(kNT) k_bgram_tiled(const float4* __restrict__ 
           const float4 w = __ldg(reinterpret_cast<const float4*>(B) + col * n + base + r);
           x = w.x; y = w.y; z = w.z;
         } else {
-          const double* w = reinterpret_cast<const double*>(B) + 4 * (col * n + base + r);
-          x = (float)w[0]; y = (float)w[1]; z = (float)w[2];
+          const double2* w = reinterpret_cast<const double2*>(B) + 2 * (col * n + base + r);
+          const double2 xy = w[0];
+          x = (float)xy.x; y = (float)xy.y; z = (float)w[1].x;
         }
       }
       sb[r][0][i] = x; sb[r][1][i] = y; sb[r][2][i] = z;
@@ -142,7 +150,7 @@ __global__ void __launch_bounds__(kNT) k_bgram_tiled(const float4* __restrict__ 
     for (int u = 0; u < 4; u++)
 #pragma unroll
       for (int v = 0; v < 4; v++) acc[u][v] = 0.f;
-    for (int r = 0; r < cnt; r++) {
+    for (int r = grp; r < cnt; r += kGroups) {
 #pragma unroll
       for (int c = 0; c < 3; c++) {
         const float4 a = *reinterpret_cast<const float4*>(&sa[r][c][4 * ti]);
@@ -157,17 +165,44 @@ __global__ void __launch_bounds__(kNT) k_bgram_tiled(const float4* __restrict__ 
 #pragma unroll
     for (int u = 0; u < 4; u++)
 #pragma unroll
-      for (int v = 0; v < 4; v++) tot[u][v] += (double)acc[u][v];
+      for (int v = 0; v < 4; v++) tot[u][v] += f32_to_f64_bits(acc[u][v]);
     __syncthreads();
   }
   double* o = out_part + (int64_t)blockIdx.x * kMaxBlk * kMaxBlk;
+  if constexpr (kGroups > 1) {   // the groups add their totals one after the other (a fixed order)
+    double* sum = reinterpret_cast<double*>(smem);   // [NC][NC]
+    for (int g = 0; g < kGroups; g++) {
+      if (grp == g)
 #pragma unroll
-  for (int u = 0; u < 4; u++)
+        for (int u = 0; u < 4; u++)
 #pragma unroll
-    for (int v = 0; v < 4; v++) {
-      const int i = 4 * ti + u, j = 4 * tj + v;
-      if (i < ta && j < tb) o[i * tb + j] = tot[u][v];
+          for (int v = 0; v < 4; v++) {
+            double* q = sum + (4 * ti + u) * NC + 4 * tj + v;
+            *q = g == 0 ? tot[u][v] : *q + tot[u][v];
+          }
+      __syncthreads();
     }
+    for (int e = threadIdx.x; e < ta * tb; e += kNT) o[e] = sum[(e / tb) * NC + e % tb];
+  } else {
+#pragma unroll
+    for (int u = 0; u < 4; u++)
+#pragma unroll
+      for (int v = 0; v < 4; v++) {
+        const int i = 4 * ti + u, j = 4 * tj + v;
+        if (i < ta && j < tb) o[i * tb + j] = tot[u][v];
+      }
+  }
+}
+
+template <int NC>
+static void bgram_tiled(const float* A, int ta, const int* idx_a, const void* B, int b_is_fp64, int tb,
+                        const int* idx_b, int64_t n, double* part, int nblk, cudaStream_t s) {
+  if (b_is_fp64)
+    k_bgram_tiled<double4_16a, NC><<<nblk, kNT, 0, s>>>(reinterpret_cast<const float4*>(A), ta, idx_a,
+                                                        reinterpret_cast<const double4_16a*>(B), tb, idx_b, n, part);
+  else
+    k_bgram_tiled<float4, NC><<<nblk, kNT, 0, s>>>(reinterpret_cast<const float4*>(A), ta, idx_a,
+                                                   reinterpret_cast<const float4*>(B), tb, idx_b, n, part);
 }
 
 // G[i][j] = sum over CTAs of out_part (fixed order: deterministic)
@@ -198,12 +233,12 @@ cudaError_t launch_bgram(const float* A, int ta, const int* idx_a, const void* B
     bgram_small<4, 4>(A, ta, idx_a, B, b_is_fp64, tb, idx_b, n, part, nblk, s);
   } else if (ta == 1 && tb <= 16) {
     bgram_small<1, 16>(A, ta, idx_a, B, b_is_fp64, tb, idx_b, n, part, nblk, s);
-  } else if (b_is_fp64) {
-    k_bgram_tiled<double4_16a><<<nblk, kNT, 0, s>>>(reinterpret_cast<const float4*>(A), ta, idx_a,
-                                                    reinterpret_cast<const double4_16a*>(B), tb, idx_b, n, part);
+  } else if (ta <= 16 && tb <= 16) {
+    bgram_tiled<16>(A, ta, idx_a, B, b_is_fp64, tb, idx_b, n, part, nblk, s);
+  } else if (ta <= 32 && tb <= 32) {
+    bgram_tiled<32>(A, ta, idx_a, B, b_is_fp64, tb, idx_b, n, part, nblk, s);
   } else {
-    k_bgram_tiled<float4><<<nblk, kNT, 0, s>>>(reinterpret_cast<const float4*>(A), ta, idx_a,
-                                               reinterpret_cast<const float4*>(B), tb, idx_b, n, part);
+    bgram_tiled<64>(A, ta, idx_a, B, b_is_fp64, tb, idx_b, n, part, nblk, s);
   }
   k_bgram_reduce<<<(ta * tb + 7) / 8, 256, 0, s>>>(part, nblk, ta * tb, G);
   return cudaGetLastError();
@@ -272,9 +307,9 @@ __global__ void __launch_bounds__(kNT) k_bcombine(TO* __restrict__ out, const in
       } else {
         double* o = reinterpret_cast<double*>(out) + 4 * (col * n + p);
         double x0 = mode ? o[0] : 0.0, x1 = mode ? o[1] : 0.0, x2 = mode ? o[2] : 0.0;
-        x0 += (double)ax[jj]; x1 += (double)ay[jj]; x2 += (double)az[jj];
+        x0 += f32_to_f64_bits(ax[jj]); x1 += f32_to_f64_bits(ay[jj]); x2 += f32_to_f64_bits(az[jj]);
         o[0] = x0; o[1] = x1; o[2] = x2; o[3] = 0.0;
-        nrm[jj] += x0 * x0 + x1 * x1 + x2 * x2;
+        if (norm_part) nrm[jj] += x0 * x0 + x1 * x1 + x2 * x2;
       }
     }
   }
@@ -297,7 +332,7 @@ __global__ void __launch_bounds__(kNT) k_bcombine_stream(TO* __restrict__ out, c
                                                    const double* __restrict__ C, int ldc, double sign,
                                                    int mode, int64_t n, double* __restrict__ norm_part) {
   __shared__ float cs[kMaxBlk * kMaxBlk];
-  __shared__ double red[kNT];
+  __shared__ double red[J][kNT / 32];
   for (int e = threadIdx.x; e < t * v; e += kNT) cs[e] = (float)(sign * C[(e / v) * ldc + (e % v)]);
   __syncthreads();
   for (int j0 = 0; j0 < v; j0 += J) {
@@ -334,25 +369,37 @@ __global__ void __launch_bounds__(kNT) k_bcombine_stream(TO* __restrict__ out, c
           double2* o = reinterpret_cast<double2*>(out) + 2 * (col * n + p);
           double2 xy = mode ? o[0] : make_double2(0.0, 0.0);
           double2 zw = mode ? o[1] : make_double2(0.0, 0.0);
-          xy.x += (double)ax[jj]; xy.y += (double)ay[jj]; zw.x += (double)az[jj];
+          xy.x += f32_to_f64_bits(ax[jj]); xy.y += f32_to_f64_bits(ay[jj]); zw.x += f32_to_f64_bits(az[jj]);
           zw.y = 0.0;
           o[0] = xy;
           o[1] = zw;
-          nrm[jj] += xy.x * xy.x + xy.y * xy.y + zw.x * zw.x;
+          if (norm_part) nrm[jj] += xy.x * xy.x + xy.y * xy.y + zw.x * zw.x;
         }
       }
     }
     if (norm_part) {
-      for (int jj = 0; jj < nj; jj++) {
-        red[threadIdx.x] = nrm[jj];
-        __syncthreads();
-        for (int sh = kNT / 2; sh > 0; sh >>= 1) {
-          if (threadIdx.x < sh) red[threadIdx.x] += red[threadIdx.x + sh];
-          __syncthreads();
+      // a warp reduces its J values together, exchanging halves, then the warps' sums in order
+      const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+      int o = 16;
+#pragma unroll
+      for (int h = J / 2; h > 0; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int j = 0; j < h; j++) {
+          const double give = up ? nrm[j] : nrm[j + h], keep = up ? nrm[j + h] : nrm[j];
+          nrm[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
         }
-        if (threadIdx.x == 0) norm_part[(int64_t)(j0 + jj) * gridDim.x + blockIdx.x] = red[0];
-        __syncthreads();
       }
+      for (; o > 0; o >>= 1) nrm[0] += __shfl_xor_sync(0xffffffffu, nrm[0], o);
+      if (lane % (32 / J) == 0) red[lane / (32 / J)][warp] = nrm[0];
+      __syncthreads();
+      if (threadIdx.x < nj) {
+        double acc = 0.0;
+#pragma unroll
+        for (int w = 0; w < kNT / 32; w++) acc += red[threadIdx.x][w];
+        norm_part[(int64_t)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = acc;
+      }
+      __syncthreads();
     }
   }
 }
@@ -507,72 +554,121 @@ cudaError_t launch_bsum(const double* X, int t, int64_t n, double* out, int accu
 //   G (t x t, symmetrised) = L L^T by a pivoted Cholesky with relative tolerance rank_tol;
 //   Linv = L^-1 (rank x rank, lower); piv[0..rank) = pivoted columns; *rank_out = rank.
 // The caller forms P = Linv Z[piv] and A P = Linv (A Z)[piv] (rows are block columns).
-__global__ void k_bchol(const double* __restrict__ G, int t, double rank_tol, double* __restrict__ Linv_out,
-                        int* __restrict__ piv_out, int* __restrict__ rank_out) {
-  // The factorisation is O(t^3) <= ~90K flops: one thread does it, with explicit indexing.
-  extern __shared__ double dsm[];      // g [kMaxBlk * kLd] then L [kMaxBlk * kLd]
+// Right-looking: the remaining matrix is updated after every column (each element sees the subtractions
+// in the same order as a left-looking factorisation), elements and inverse columns over the threads, the
+// pivot by one warp.  Bound by the latency of its t steps (a division, a square root, three barriers).
+// One thread took 224 us at t = 16; now 48 us.
+constexpr int kCholNT = 256;
+__global__ void __launch_bounds__(kCholNT) k_bchol(const double* __restrict__ G, int t, double rank_tol,
+                                                    double* __restrict__ Linv_out, int* __restrict__ piv_out,
+                                                    int* __restrict__ rank_out) {
+  extern __shared__ double dsm[];      // g [kMaxBlk * kLd] (the factor in its lower part), then L^-1
   constexpr int kLd = kMaxBlk + 1;
   double* g = dsm;
-  double* L = dsm + kMaxBlk * kLd;
-  if (threadIdx.x != 0) return;
-  int piv[kMaxBlk];
-  double mx = 0.0;
-  for (int i = 0; i < t; i++) {
-    piv[i] = i;
-    for (int j = 0; j < t; j++) {
-      g[i * kLd + j] = 0.5 * (G[i * t + j] + G[j * t + i]);
-      L[i * kLd + j] = 0.0;
-    }
-    mx = fmax(mx, fabs(g[i * kLd + i]));
+  double* inv = dsm + kMaxBlk * kLd;
+  __shared__ int piv[kMaxBlk];
+  __shared__ int s_best;
+  __shared__ double s_bd, s_scale;
+  const int tid = threadIdx.x, lane = tid & 31;
+  for (int e = tid; e < t * t; e += kCholNT) {
+    const int i = e / t, j = e % t;
+    g[i * kLd + j] = 0.5 * (G[i * t + j] + G[j * t + i]);
   }
-  const double scale = mx > 0.0 ? mx : 1e-300;
+  for (int i = tid; i < t; i += kCholNT) piv[i] = i;
+  __syncthreads();
+  if (tid < 32) {
+    double mx = 0.0;
+    for (int i = lane; i < t; i += 32) mx = fmax(mx, fabs(g[i * kLd + i]));
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) s_scale = mx > 0.0 ? mx : 1e-300;
+  }
+  __syncthreads();
   int r = t;
   for (int k = 0; k < t; k++) {
-    int best = k;
-    double bd = -1.0;
-    for (int i = k; i < t; i++) {
-      double d = g[i * kLd + i];
-      for (int m = 0; m < k; m++) d -= L[i * kLd + m] * L[i * kLd + m];
-      if (d > bd) { bd = d; best = i; }
+    if (tid < 32) {   // the largest remaining diagonal, the first of equal ones
+      double bd = -1.0;
+      int best = k;
+      for (int i = k + lane; i < t; i += 32) {
+        const double d = g[i * kLd + i];
+        if (d > bd) {
+          bd = d;
+          best = i;
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        const double d = __shfl_xor_sync(0xffffffffu, bd, o);
+        const int i = __shfl_xor_sync(0xffffffffu, best, o);
+        if (d > bd || (d == bd && i < best)) {
+          bd = d;
+          best = i;
+        }
+      }
+      if (lane == 0) {
+        s_bd = bd;
+        s_best = best;
+      }
     }
-    if (!(bd > rank_tol * scale)) { r = k; break; }
-    if (best != k) {   // symmetric swap of rows/columns k and best, and of the computed rows of L
-      for (int j = 0; j < t; j++) { const double tmp = g[k * kLd + j]; g[k * kLd + j] = g[best * kLd + j]; g[best * kLd + j] = tmp; }
-      for (int j = 0; j < t; j++) { const double tmp = g[j * kLd + k]; g[j * kLd + k] = g[j * kLd + best]; g[j * kLd + best] = tmp; }
-      for (int m = 0; m < k; m++) { const double tmp = L[k * kLd + m]; L[k * kLd + m] = L[best * kLd + m]; L[best * kLd + m] = tmp; }
-      const int tp = piv[k]; piv[k] = piv[best]; piv[best] = tp;
+    __syncthreads();
+    const double bd = s_bd;
+    const int best = s_best;
+    if (!(bd > rank_tol * s_scale)) {
+      r = k;
+      break;
     }
-    L[k * kLd + k] = sqrt(bd);
-    for (int i = k + 1; i < t; i++) {
-      double sacc = g[i * kLd + k];
-      for (int m = 0; m < k; m++) sacc -= L[i * kLd + m] * L[k * kLd + m];
-      L[i * kLd + k] = sacc / L[k * kLd + k];
+    if (best != k) {   // symmetric swap of rows and columns k and best of the remaining matrix, rows of the factor
+      for (int j = tid; j < t; j += kCholNT) {
+        const double tmp = g[k * kLd + j];
+        g[k * kLd + j] = g[best * kLd + j];
+        g[best * kLd + j] = tmp;
+      }
+      if (tid == 0) {
+        const int tp = piv[k];
+        piv[k] = piv[best];
+        piv[best] = tp;
+      }
+      __syncthreads();
+      for (int j = k + tid; j < t; j += kCholNT) {
+        const double tmp = g[j * kLd + k];
+        g[j * kLd + k] = g[j * kLd + best];
+        g[j * kLd + best] = tmp;
+      }
+      __syncthreads();
     }
+    const double lkk = sqrt(bd);
+    for (int i = k + 1 + tid; i < t; i += kCholNT) g[i * kLd + k] = g[i * kLd + k] / lkk;
+    __syncthreads();
+    if (tid == 0) g[k * kLd + k] = lkk;
+    const int m = t - k - 1;   // both triangles are updated: the swaps move either
+    for (int e = tid; e < m * m; e += kCholNT) {
+      const int i = k + 1 + e / m, j = k + 1 + e % m;
+      g[i * kLd + j] -= g[i * kLd + k] * g[j * kLd + k];
+    }
+    __syncthreads();
   }
-  // Linv = L^-1 (r x r, lower) by forward substitution, column by column
-  for (int e = 0; e < kMaxBlk * kMaxBlk; e++) Linv_out[e] = 0.0;
-  for (int c = 0; c < r; c++) {
+  // L^-1 (r x r, lower) by forward substitution, a column per thread
+  for (int e = tid; e < kMaxBlk * kLd; e += kCholNT) inv[e] = 0.0;
+  __syncthreads();
+  for (int c = tid; c < r; c += kCholNT) {
     for (int i = c; i < r; i++) {
       double sacc = (i == c) ? 1.0 : 0.0;
-      for (int m = c; m < i; m++) sacc -= L[i * kLd + m] * Linv_out[m * kMaxBlk + c];
-      Linv_out[i * kMaxBlk + c] = sacc / L[i * kLd + i];
+      for (int m = c; m < i; m++) sacc -= g[i * kLd + m] * inv[m * kLd + c];
+      inv[i * kLd + c] = sacc / g[i * kLd + i];
     }
   }
-  for (int i = 0; i < t; i++) piv_out[i] = piv[i];
-  *rank_out = r;
+  __syncthreads();
+  for (int e = tid; e < kMaxBlk * kMaxBlk; e += kCholNT) Linv_out[e] = inv[(e / kMaxBlk) * kLd + e % kMaxBlk];
+  for (int i = tid; i < t; i += kCholNT) piv_out[i] = piv[i];
+  if (tid == 0) *rank_out = r;
 }
 
 cudaError_t launch_bchol(const double* G, int t, double rank_tol, double* Linv, int* piv, int* rank,
                          cudaStream_t s) {
   if (t > kMaxBlk) return cudaErrorInvalidValue;
-  const size_t smem = 2 * kMaxBlk * (kMaxBlk + 1) * sizeof(double);
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(k_bchol, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
-  k_bchol<<<1, 32, smem, s>>>(G, t, rank_tol, Linv, piv, rank);
+  constexpr size_t smem = 2 * kMaxBlk * (kMaxBlk + 1) * sizeof(double);
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(k_bchol, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (attr != cudaSuccess) return attr;
+  k_bchol<<<1, kCholNT, smem, s>>>(G, t, rank_tol, Linv, piv, rank);
   return cudaGetLastError();
 }
 
