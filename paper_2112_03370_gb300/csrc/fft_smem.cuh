@@ -144,13 +144,13 @@ __device__ __forceinline__ void dft_small(C (&a)[R]) {
 // Twiddle factors W_M^k, k in [0, M), from a two-level table in shared memory:
 // W_M^k = hi[k >> 6] * lo[k & 63] with lo[i] = W_M^i (64 entries) and hi[i] = W_M^{64 i}
 // (M / 64 entries); one complex product, accurate to a few ulp.
-// `full` (global memory): W_M^k itself at full[k * fs].
+// `first` (global memory, FP64 and df64 tiles): the twiddles of the first radix-16 pass, W^{j n1} at
+// first[(j - 1) S + n1].
 template <typename C>
 struct TwiddleTab {
   const C* lo;
   const C* hi;
-  const C* full;
-  int fs;
+  const C* first;
   __device__ __forceinline__ C operator()(int k) const { return c_mul(hi[k >> 6], lo[k & 63]); }
 };
 constexpr int twiddle_tab_entries(int m) { return 64 + m / 64; }
@@ -161,24 +161,18 @@ __device__ __forceinline__ C ldg_c(const C* p) { return __ldg(p); }
 
 // Fill the shared table from the global table tw[k * fs] = W_M^k (called by all threads, then sync).
 template <typename C, int MFULL, int NT>
-__device__ __forceinline__ TwiddleTab<C> load_twiddle_tab(C* tab_sm, const C* __restrict__ tw, int fs = 1) {
+__device__ __forceinline__ TwiddleTab<C> load_twiddle_tab(C* tab_sm, const C* __restrict__ tw, int fs = 1,
+                                                          const C* first = nullptr) {
   for (int i = threadIdx.x; i < twiddle_tab_entries(MFULL); i += NT) {
     tab_sm[i] = (i < 64) ? ldg_c(tw + i * fs) : ldg_c(tw + 64 * (i - 64) * fs);
   }
-  return TwiddleTab<C>{tab_sm, tab_sm + 64, tw, fs};
+  return TwiddleTab<C>{tab_sm, tab_sm + 64, first};
 }
 
-// Twiddles w_j = W_C^{n1 j} = W_M^{n1 j (M / C)}, j = 1..R-1: FP32 powers 1, 2, 4, 8 from the table,
-// the rest as products of two of those.  FP64 and double-float products cost as much as a quarter of
-// the butterfly on the pipes that bound those tiles, so their twiddles are read from global memory
-// (L2 holds the table).
+// Twiddles w_j = W_C^{n1 j} = W_M^{n1 j (M / C)}, j = 1..R-1: powers 1, 2, 4, 8 from the table,
+// the rest as products of two of those.
 template <int R, typename C>
 __device__ __forceinline__ void twiddles(const TwiddleTab<C>& tw, int base_idx, C (&w)[R]) {
-  if constexpr (sizeof(C) == 16) {
-#pragma unroll
-    for (int j = 1; j < R; j++) w[j] = ldg_c(tw.full + j * base_idx * tw.fs);
-    return;
-  }
   w[1] = tw(base_idx);
   if constexpr (R > 2) {
     w[2] = tw(2 * base_idx);
@@ -194,6 +188,25 @@ __device__ __forceinline__ void twiddles(const TwiddleTab<C>& tw, int base_idx, 
     w[8] = tw(8 * base_idx);
 #pragma unroll
     for (int j = 1; j < 8; j++) w[8 + j] = c_mul(w[8], w[j]);
+  }
+}
+
+// a[j] *= w_j (CONJ: its conjugate).  FP64 and double-float products of table entries cost as much as a
+// quarter of the butterfly on the pipes that bound those tiles, so their twiddles are read from global
+// memory (L2 holds the table, a warp reads it in whole lines).
+template <int R, bool CONJ, typename C>
+__device__ __forceinline__ void twiddle_all(C (&a)[R], const TwiddleTab<C>& tw, int base_idx, int S, int n1) {
+  if constexpr (sizeof(C) == 16) {
+#pragma unroll
+    for (int j = 1; j < R; j++) {
+      const C w = ldg_c(tw.first + (j - 1) * S + n1);
+      a[j] = CONJ ? c_mulc(a[j], w) : c_mul(a[j], w);
+    }
+  } else {
+    C w[R];
+    twiddles<R>(tw, base_idx, w);
+#pragma unroll
+    for (int j = 1; j < R; j++) a[j] = CONJ ? c_mulc(a[j], w[j]) : c_mul(a[j], w[j]);
   }
 }
 
@@ -257,10 +270,7 @@ __device__ __forceinline__ void fft_pass(C* __restrict__ sm, const TwiddleTab<C>
         if (ptab) {
           ptab_twiddle<R, false>(a, ptab, S, n1);
         } else {
-          C w[R];
-          twiddles<R>(tw, n1 * mfull_over_cs, w);
-#pragma unroll
-          for (int j = 1; j < R; j++) a[j] = c_mul(a[j], w[j]);
+          twiddle_all<R, false>(a, tw, n1 * mfull_over_cs, S, n1);
         }
       }
     } else {
@@ -268,10 +278,7 @@ __device__ __forceinline__ void fft_pass(C* __restrict__ sm, const TwiddleTab<C>
         if (ptab) {
           ptab_twiddle<R, true>(a, ptab, S, n1);
         } else {
-          C w[R];
-          twiddles<R>(tw, n1 * mfull_over_cs, w);
-#pragma unroll
-          for (int j = 1; j < R; j++) a[j] = c_mulc(a[j], w[j]);
+          twiddle_all<R, true>(a, tw, n1 * mfull_over_cs, S, n1);
         }
       }
       dft_small<R, false>(a);

@@ -335,18 +335,6 @@ __device__ const double2 kSinCosPi32[64] = {
     {0.9238795325112867, -0.3826834323650898}, {0.9569403357322088, -0.2902846772544624},
     {0.9807852804032304, -0.19509032201612828}, {0.9951847266721969, -0.0980171403295606}};
 
-// FP64 -> FP32, rounded to nearest even, by moving and rounding the encoding with integer instructions (the
-// conversion instruction runs on the FP64 pipe, 1/64 of the FP32 rate).  |d| below 2^-126 gives a signed zero,
-// magnitudes of 2^128 and more and NaN do not occur here (weights and their remainders).
-__device__ __forceinline__ float f64_to_f32_bits(double d) {
-  const uint64_t u = (uint64_t)__double_as_longlong(d);
-  const uint32_t sign = (uint32_t)(u >> 32) & 0x80000000u;
-  const uint64_t mag = u & 0x7fffffffffffffffull;
-  if (mag < ((uint64_t)(1023 - 126) << 52)) return __uint_as_float(sign);
-  const uint64_t r = mag + 0x0fffffffull + ((mag >> 29) & 1);   // round the 29 dropped bits, ties to even
-  return __uint_as_float(sign | ((uint32_t)(r >> 29) - (896u << 23)));
-}
-
 // (cos x, sin x), x = 2 psi, in FP64 by table lookup and angle addition (the table-driven method of
 // P. T. P. Tang, ACM TOMS 1989-91): x = k pi/32 + r with k = rint(32 x / pi) and r = x - k pi/32 by a
 // two-constant Cody-Waite reduction (pi/32 = H + L, H = fl64(pi/32); k H is taken exactly inside one FMA);

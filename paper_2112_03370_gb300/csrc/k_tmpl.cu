@@ -452,36 +452,27 @@ __device__ __forceinline__ df legendre_q_dot(df x, int n, const df (&c)[NP], df 
 // cos(k phi), sin(k phi), k = 1..n, from cos(phi), sin(phi) by complex multiplication, generated and
 // consumed on the fly
 template <int NH>
-__device__ __forceinline__ void harmonics_df_acc(float4 cs1, int n, df v, df (&ac)[NH], df (&as)[NH]) {
-  const df c1 = df_make(cs1.x, cs1.y), s1 = df_make(cs1.z, cs1.w);
-  df ck = c1, sk = s1;
+__device__ __forceinline__ void harmonics_df_acc(float4 cs1, int n, df v, dfc (&acc)[NH]) {
+  const dfc w1 = dfc_make(df_make(cs1.x, cs1.y), df_make(cs1.z, cs1.w)), w1i = dfc_i(w1), vv = dfc_make(v, v);
+  dfc w = w1;
 #pragma unroll
   for (int k = 0; k < NH; k++) {
     if (k >= n) break;
-    ac[k] = df_fma(ck, v, ac[k]);
-    as[k] = df_fma(sk, v, as[k]);
-    if (k + 1 < n) {
-      const df cn = df_prod_sum(ck, c1, -sk, s1), sn = df_prod_sum(sk, c1, ck, s1);
-      ck = cn;
-      sk = sn;
-    }
+    acc[k] = dfc_fma(w, vv, acc[k]);
+    if (k + 1 < n) w = dfc_prod_sum(dfc_xx(w), w1, dfc_yy(w), w1i);
   }
 }
 template <int NH>
-__device__ __forceinline__ df harmonics_df_dot(float4 cs1, int n, const df (&cc)[NH], const df (&cs)[NH], df s) {
-  const df c1 = df_make(cs1.x, cs1.y), s1 = df_make(cs1.z, cs1.w);
-  df ck = c1, sk = s1;
+__device__ __forceinline__ df harmonics_df_dot(float4 cs1, int n, const dfc (&c)[NH], df s) {
+  const dfc w1 = dfc_make(df_make(cs1.x, cs1.y), df_make(cs1.z, cs1.w)), w1i = dfc_i(w1);
+  dfc w = w1, sum = dfc_make(s, df_make(0.f, 0.f));
 #pragma unroll
   for (int k = 0; k < NH; k++) {
     if (k >= n) break;
-    s = s + df_prod_sum(cc[k], ck, cs[k], sk);
-    if (k + 1 < n) {
-      const df cn = df_prod_sum(ck, c1, -sk, s1), sn = df_prod_sum(sk, c1, ck, s1);
-      ck = cn;
-      sk = sn;
-    }
+    sum = dfc_fma(c[k], w, sum);
+    if (k + 1 < n) w = dfc_prod_sum(dfc_xx(w), w1, dfc_yy(w), w1i);
   }
-  return s;
+  return dfc_x(sum) + dfc_y(sum);
 }
 
 __device__ __forceinline__ df shfl_down_df(df v, int off) {
@@ -592,11 +583,12 @@ __global__ void __cluster_dims__(kTC, 1, 1) __launch_bounds__(kTA)
   };
 
   // ---- pass 1 ----
-  df aq[NP], ahc[NH], ahs[NH];
+  df aq[NP];
+  dfc ah[NH];   // (cos, sin) sums of every harmonic
 #pragma unroll
   for (int q = 0; q < NP; q++) aq[q] = df_make(0.f, 0.f);
 #pragma unroll
-  for (int q = 0; q < NH; q++) ahc[q] = ahs[q] = df_make(0.f, 0.f);
+  for (int q = 0; q < NH; q++) ah[q] = dfc_make(df_make(0.f, 0.f), df_make(0.f, 0.f));
   for (int64_t g0 = s_lo + (int64_t)warp * 32 * kUdf; g0 < s_hi; g0 += (int64_t)kTA * kUdf) {
     Ld L[kUdf];
     load(g0, L, !TOD, true);
@@ -608,7 +600,7 @@ __global__ void __cluster_dims__(kTC, 1, 1) __launch_bounds__(kTA)
       if (L[u].p >= 0) {
         v = wb * unpoint(L[u].tv, L[u].w4, L[u].iq, L[u].u4);
         if (np > 0) legendre_q_acc<NP>(legendre_x(g - lo, nm1, inv), np, v, aq);
-        if (nh > 0) harmonics_df_acc<NH>(L[u].h4, nh, v, ahc, ahs);
+        if (nh > 0) harmonics_df_acc<NH>(L[u].h4, nh, v, ah);
         bin = L[u].bin;
       }
       if (naz > 0) az_run_sums_df(a_sm + c0, bin, v, df_make(L[u].fr.x, L[u].fr.y), d.interp, naz, lane);
@@ -623,7 +615,7 @@ __global__ void __cluster_dims__(kTC, 1, 1) __launch_bounds__(kTA)
 #pragma unroll
   for (int q = 0; q < NH; q++)
     if (q < nh) {
-      const double tc = warp_sum(df_to_double(ahc[q])), ts = warp_sum(df_to_double(ahs[q]));
+      const double tc = warp_sum(df_to_double(dfc_x(ah[q]))), ts = warp_sum(df_to_double(dfc_y(ah[q])));
       if (lane == 0) {
         red[warp][NP + 2 * q] = tc;
         red[warp][NP + 2 * q + 1] = ts;
@@ -655,7 +647,8 @@ __global__ void __cluster_dims__(kTC, 1, 1) __launch_bounds__(kTA)
     c_sm[tid] = t;
   }
   __syncthreads();
-  df cq[NP], chc[NH], chs[NH];
+  df cq[NP];
+  dfc ch[NH];
 #pragma unroll
   for (int q = 0; q < NP; q++) {
     double fact = 1.0;
@@ -664,8 +657,8 @@ __global__ void __cluster_dims__(kTC, 1, 1) __launch_bounds__(kTA)
   }
 #pragma unroll
   for (int q = 0; q < NH; q++) {
-    chc[q] = q < nh ? df(c_sm[h0 + 2 * q]) : df_make(0.f, 0.f);
-    chs[q] = q < nh ? df(c_sm[h0 + 2 * q + 1]) : df_make(0.f, 0.f);
+    ch[q] = q < nh ? dfc_make(df(c_sm[h0 + 2 * q]), df(c_sm[h0 + 2 * q + 1]))
+                   : dfc_make(df_make(0.f, 0.f), df_make(0.f, 0.f));
   }
   for (int j = tid; j <= naz; j += kTA) caz[j] = j < naz ? df(c_sm[c0 + j]) : df_make(0.f, 0.f);
   __syncthreads();
@@ -692,7 +685,7 @@ __global__ void __cluster_dims__(kTC, 1, 1) __launch_bounds__(kTA)
           sv = sv + caz[i];
         }
       }
-      if (nh > 0) sv = harmonics_df_dot<NH>(L[u].h4, nh, chc, chs, sv);
+      if (nh > 0) sv = harmonics_df_dot<NH>(L[u].h4, nh, ch, sv);
       // TOD mode: w_b (t - T c); map mode: -w_b T c (the diagonal part M x is added per pixel)
       df yv;
       if constexpr (TOD) yv = wb * (df_make(L[u].tv.x, L[u].tv.y) - sv);

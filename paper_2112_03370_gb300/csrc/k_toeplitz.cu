@@ -413,6 +413,27 @@ __device__ __forceinline__ C pair_upd(C ab, C z, C zp, T sc) {
   // s (a Z + i b conj(Zp)) = s (a x + b yp, a y + b xp)
   return C{sc * (ab.x * z.x + ab.y * zp.y), sc * (ab.x * z.y + ab.y * zp.x)};
 }
+__device__ __forceinline__ dfc pair_upd(dfc ab, dfc z, dfc zp, df sc) {
+  const dfc u = dfc_prod_sum(dfc_xx(ab), z, dfc_yy(ab), dfc{swap2(zp.hi), swap2(zp.lo)});
+  return dfc_make(sc * dfc_x(u), sc * dfc_y(u));
+}
+
+// complex value of two real ones, and its parts
+template <typename C, typename T>
+__device__ __forceinline__ C c_of(T x, T y) {
+  if constexpr (std::is_same<C, dfc>::value) return dfc_make(x, y);
+  else return C{x, y};
+}
+template <typename C>
+__device__ __forceinline__ auto c_re(C z) {
+  if constexpr (std::is_same<C, dfc>::value) return dfc_x(z);
+  else return z.x;
+}
+template <typename C>
+__device__ __forceinline__ auto c_im(C z) {
+  if constexpr (std::is_same<C, dfc>::value) return dfc_y(z);
+  else return z.y;
+}
 
 // The u-th quad q <= partner_quad(q) (2049 of them): a in 1..7; a = 8 with b < 8; a = 0 with b in
 // 1..7; a = 0, b = 8 with c < 8; a = b = 0 with c in 1..7; then the two quads that pair with
@@ -528,7 +549,8 @@ __global__ void __launch_bounds__(tile_threads(CL, LOGM), kTileThreads / tile_th
   // both CTAs of a cluster read the same flag, so they leave together
   if (a.done != nullptr && a.done[(int64_t)rhs * a.done_stride] != 0) return;
   const C* __restrict__ tw_g = reinterpret_cast<const C*>(a.tw);
-  const TwiddleTab<C> tw = load_twiddle_tab<C, MT, NT>(tw_sm, tw_g, LOGM < kLogM ? kM / MT : 1);
+  const TwiddleTab<C> tw = load_twiddle_tab<C, MT, NT>(tw_sm, tw_g, LOGM < kLogM ? kM / MT : 1,
+                                                              reinterpret_cast<const C*>(a.tw0));
   const C* __restrict__ tab =
       reinterpret_cast<const C*>(a.tab) + ((int64_t)seg.tab * CL + rank) * MS;
   const T sc = (T)seg.scale;
@@ -560,8 +582,8 @@ __global__ void __launch_bounds__(tile_threads(CL, LOGM), kTileThreads / tile_th
         for (int u = 0; u < NQ; u++) {
           const int q = q0 + u * NT;
           if (q < HALF_Q) {
-            sm[smem_pad(2 * q)] = C{v[u][0], v[u][1]};
-            sm[smem_pad(2 * q + 1)] = C{v[u][2], v[u][3]};
+            sm[smem_pad(2 * q)] = c_of<C>(v[u][0], v[u][1]);
+            sm[smem_pad(2 * q + 1)] = c_of<C>(v[u][2], v[u][3]);
           }
         }
       }
@@ -617,8 +639,8 @@ __global__ void __launch_bounds__(tile_threads(CL, LOGM), kTileThreads / tile_th
 #pragma unroll
           for (int h = 0; h < 2; h++) {
             const int n = 2 * q + h;
-            const C z{v[2 * u][2 * h], v[2 * u][2 * h + 1]};
-            const C z2{v[2 * u + 1][2 * h], v[2 * u + 1][2 * h + 1]};
+            const C z = c_of<C>(v[2 * u][2 * h], v[2 * u][2 * h + 1]);
+            const C z2 = c_of<C>(v[2 * u + 1][2 * h], v[2 * u + 1][2 * h + 1]);
             sm[smem_pad(n)] = (rank == 0) ? c_add(z, z2) : c_mul(c_sub(z, z2), tw(n));
           }
         }
@@ -681,16 +703,9 @@ __global__ void __launch_bounds__(tile_threads(CL, LOGM), kTileThreads / tile_th
 #pragma unroll
         for (int b = 0; b < PB; b++) {
           if (!act[b]) continue;
-          if (jj[b] == jp[b]) {
-            sm[smem_pad(jj[b])] = C{sc * (ab[b].x * z[b].x + ab[b].y * z[b].y),
-                                    sc * (ab[b].x * z[b].y + ab[b].y * z[b].x)};
-          } else {
-            // a Z + i b conj(Zp) = (a x + b yp, a y + b xp)
-            sm[smem_pad(jj[b])] = C{sc * (ab[b].x * z[b].x + ab[b].y * zp[b].y),
-                                    sc * (ab[b].x * z[b].y + ab[b].y * zp[b].x)};
-            sm[smem_pad(jp[b])] = C{sc * (abp[b].x * zp[b].x + abp[b].y * z[b].y),
-                                    sc * (abp[b].x * zp[b].y + abp[b].y * z[b].x)};
-          }
+          const C zn = pair_upd(ab[b], z[b], zp[b], sc);   // a frequency that pairs with itself has zp = z
+          if (jj[b] != jp[b]) sm[smem_pad(jp[b])] = pair_upd(abp[b], zp[b], z[b], sc);
+          sm[smem_pad(jj[b])] = zn;
         }
       }
     }
@@ -754,8 +769,8 @@ __global__ void __launch_bounds__(tile_threads(CL, LOGM), kTileThreads / tile_th
                 const C o = other[smem_pad(n)];
                 z = (rank == 0) ? c_add(z, o) : c_sub(o, z);
               }
-              y[u][2 * h] = z.x;
-              y[u][2 * h + 1] = z.y;
+              y[u][2 * h] = c_re(z);
+              y[u][2 * h + 1] = c_im(z);
             }
           } else {
             g[u] = td.out_hi;                          // whole quad outside the output range
@@ -1135,6 +1150,19 @@ __global__ void k_twiddles(double2* tw64, float2* tw32, const double* __restrict
   const double s = costab[(2 * k - l / 4) & (l - 1)];
   if (tw64) tw64[k] = make_double2(c, -s);
   tw32[k] = make_float2((float)c, (float)-s);
+}
+
+// twiddles of the first radix-16 pass of a transform of 2^logms points from tw[k] = W_kM^k: W^{j n1} at
+// [(j - 1) S + n1], S = 2^logms / 16, j = 1..15
+__global__ void k_first_pass(const double2* __restrict__ tw, int logms, double2* __restrict__ out) {
+  const int s = 1 << (logms - 4), i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= 15 * s) return;
+  out[i] = tw[(i / s + 1) * (i % s) * (kM >> logms)];
+}
+cudaError_t launch_first_pass(const double2* tw64, int logms, double2* out, cudaStream_t s) {
+  const int n = 15 << (logms - 4);
+  k_first_pass<<<(n + 255) / 256, 256, 0, s>>>(tw64, logms, out);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_twiddles(double2* tw64, float2* tw32, const double* costab, cudaStream_t s, int logm) {

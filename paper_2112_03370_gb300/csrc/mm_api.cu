@@ -202,7 +202,7 @@ void free_plan(Plan* P) {
   dfree(P->band); dfree(P->block_off_dev); dfree(P->c0_blk); dfree(P->tab32); dfree(P->tab64);
   dfree(P->tw32); dfree(P->tw64); dfree(P->tiles); dfree(P->segs); dfree(P->nsegs); dfree(P->ntab32); dfree(P->ntw32); dfree(P->map32_in); dfree(P->map32_out);
   dfree(P->map64_in); dfree(P->map64_out); dfree(P->td_a); dfree(P->td_b); dfree(P->t32);
-  dfree(P->wdf); dfree(P->tabdf); dfree(P->twdf); dfree(P->tdf); dfree(P->mapdf);
+  dfree(P->wdf); dfree(P->tabdf); dfree(P->twdf); dfree(P->tw64_first); dfree(P->twdf_first); dfree(P->tdf); dfree(P->mapdf);
   dfree(P->ang2); dfree(P->groups); dfree(P->slot); dfree(P->slot_pix); dfree(P->u32);
   dfree(P->seg_ent); dfree(P->seg_ang); dfree(P->seg_kept);
   dfree(P->udf); dfree(P->amax);
@@ -790,6 +790,9 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
   MM_CUDA(launch_spectra(rows_d, P->n_tab, lam, H, costab_d, spec, s));
   MM_CUDA(launch_pair_tables(H, P->n_tab, costab_d, P->logm64, P->tab64, P->tab32, s));
   MM_CUDA(launch_twiddles(P->tw64, P->tw32, costab_d, s));
+  const int logms64 = P->logm64 == kLogM ? kLogM - 1 : P->logm64, n_first = 15 << (logms64 - 4);
+  MM_TRY(dalloc(P, &P->tw64_first, n_first));
+  MM_CUDA(launch_first_pass(P->tw64, logms64, P->tw64_first, s));
   // FP32 N^-1 on 65536-sample tiles (2-CTA clusters) when a 32768-sample tile would keep less than
   // 5/8 of its outputs: tables built here, used when mm_autotune measures them faster
   P->big = P->precision == MM_FP32 && P->algo == MM_TPLZ_FFT && !P->tc && !P->no_windows && !P->no_big &&
@@ -838,6 +841,8 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
     MM_TRY(dalloc(P, &P->twdf, kM));
     MM_CUDA(launch_c64_to_df(P->tab64, (int64_t)P->n_tab << P->logm64, P->tabdf, s));
     MM_CUDA(launch_c64_to_df(P->tw64, kM, P->twdf, s));
+    MM_TRY(dalloc(P, &P->twdf_first, n_first));
+    MM_CUDA(launch_c64_to_df(P->tw64_first, n_first, P->twdf_first, s));
   }
   std::vector<double> Hh((size_t)P->n_tab * (kM + 1));
   MM_CUDA(cudaMemcpyAsync(Hh.data(), H, Hh.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -909,6 +914,7 @@ TileArgs base_args(const Plan* P, bool fp32) {
   a.w64 = P->w64;
   a.tab = fp32 ? (const void*)P->tab32 : (const void*)P->tab64;
   a.tw = fp32 ? (const void*)P->tw32 : (const void*)P->tw64;
+  a.tw0 = P->tw64_first;
   a.done = nullptr;
   a.done_stride = 0;
   return a;
@@ -986,6 +992,7 @@ TileArgs df_args(const Plan* P) {
   a.wdf = P->wdf;
   a.tab = P->tabdf;
   a.tw = P->twdf;
+  a.tw0 = P->twdf_first;
   a.x_stride = df_stride(P);
   a.y_stride = P->n_obs * 4;
   return a;

@@ -182,6 +182,7 @@ struct TileArgs {
   const float4* wdf;        // [N] (cos hi, cos lo, sin hi, sin lo) (df64 path)
   const void* tab;          // [n_tab][cl][M/cl] (a, b) of float2 / double2
   const void* tw;           // [M] twiddles W_M^k (float2 / double2)
+  const void* tw0;          // FP64 / df64 tiles: twiddles of the first radix-16 pass (launch_first_pass)
   const void* x;            // APPLY: map in, [nrhs][n_obs][4]; RHS: d [nrhs][N]; NINV: t [N]
   int32_t x_is_fp32;        // RHS only: d in float32
   int64_t x_stride;         // elements between right-hand sides of x
@@ -224,6 +225,8 @@ struct Plan {
   double2* tab64 = nullptr;            // [n_tab][2^logm64]
   float2* tw32 = nullptr;              // [M]
   double2* tw64 = nullptr;             // [M]
+  double2* tw64_first = nullptr;       // first-pass twiddles of the FP64 and of the df64 tiles
+  float4* twdf_first = nullptr;
   float4* tabdf = nullptr;             // [n_tab][2^logm64] df64 pair tables (df64 plans)
   float4* twdf = nullptr;              // [M] df64 twiddles
   float2* tdf = nullptr;               // [nrhs][N4] un-pointed df64 input, N4 = N rounded up to 4
@@ -393,6 +396,8 @@ cudaError_t launch_pair_table32_big(const double* H, int32_t n_tab, const double
 // W_M^k, k < M = 2^logm (tw64 may be null)
 cudaError_t launch_twiddles(double2* tw64, float2* tw32, const double* costab, cudaStream_t s,
                             int logm = kLogM);
+// first-pass twiddles of transforms of 2^logms points: out [15 2^logms / 16]
+cudaError_t launch_first_pass(const double2* tw64, int logms, double2* out, cudaStream_t s);
 // FP32 u = N^-1 t over 65536-sample 2-CTA tiles
 cudaError_t launch_ninv32_big(const TileArgs& a, cudaStream_t s);
 

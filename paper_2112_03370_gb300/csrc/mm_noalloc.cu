@@ -147,6 +147,7 @@ extern "C" int mm_apply_A_noalloc(mm_plan_t plan, const double* x, double* y, in
     a.n_tiles = P->n_tiles;
     a.tab = P->tab64;
     a.tw = P->tw64;
+    a.tw0 = P->tw64_first;
     MM_CUDA(launch_tiles_fp64(P->logm64, MODE_APPLY, a, s));
   }
   k_na_unpack<<<grid_of((int64_t)tot), 256, 0, s>>>(out4, (int64_t)tot, fp32 ? 1 : 0, y);
