@@ -204,6 +204,7 @@ void free_plan(Plan* P) {
   dfree(P->map64_in); dfree(P->map64_out); dfree(P->td_a); dfree(P->td_b); dfree(P->t32);
   dfree(P->wdf); dfree(P->tabdf); dfree(P->twdf); dfree(P->tw64_first); dfree(P->twdf_first); dfree(P->tdf); dfree(P->mapdf);
   dfree(P->ang2); dfree(P->groups); dfree(P->slot); dfree(P->slot_pix); dfree(P->u32);
+  dfree(P->srt_ent); dfree(P->srt_ang); dfree(P->srt_slot);
   dfree(P->seg_ent); dfree(P->seg_ang); dfree(P->seg_kept);
   dfree(P->udf); dfree(P->amax);
   dfree(P->tc_tiles); dfree(P->tc_tab); dfree(P->tc_scale); dfree(P->tc_err);
