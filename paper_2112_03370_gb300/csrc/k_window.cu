@@ -435,17 +435,19 @@ __device__ __forceinline__ void fill_window(float4* win, const float4* __restric
 // memory, then one coalesced pass over the group's samples, each lane's next slots and angles loaded
 // while it works on the current ones (and the first before the window is filled).  Bound by HBM:
 // 10 B per sample (slot 2, angle 4, t 4); 256 detectors x 4 x 65,536 samples: 144 us, 4.7 TB/s (175 us
-// before the window was filled by asynchronous copies, 4 x 65,536 samples: 55 -> 5 us).  MULTI: the group's problem (one column) comes from
-// probs[G.prob].
+// before the window was filled by asynchronous copies, 4 x 65,536 samples: 55 -> 5 us).  Several columns are
+// bound by instruction issue (slots, angles and cos / sin again for each), so NC = 2 of them go through the
+// samples together while two windows leave four CTAs on an SM: 8.4M samples x 16 columns, 205 -> 156 us.
+// MULTI: the group's problem (one column) comes from probs[G.prob].
 constexpr int kUnpointThreads = 256;
-template <bool MULTI>
-__global__ void __launch_bounds__(kUnpointThreads, 6) k_unpoint_win32(
+template <bool MULTI, int NC>
+__global__ void __launch_bounds__(kUnpointThreads, NC == 1 ? 6 : 4) k_unpoint_win32(
     const PGroup* __restrict__ groups, const int64_t* __restrict__ block_off,
     const uint16_t* __restrict__ slot, const int32_t* __restrict__ slot_pix, const float* __restrict__ ang2,
     const float4* __restrict__ x4, int64_t x_stride4, int nrhs, const int32_t* __restrict__ done,
     int done_stride, float* __restrict__ t, int64_t t_stride, const WinProb* __restrict__ probs, WinSize size) {
-  extern __shared__ float4 win[];   // [size.slots], then the row table
-  RowTab rt(win + size.slots, size.dets);
+  extern __shared__ float4 win[];   // [NC][size.slots], then the row table
+  RowTab rt(win + NC * size.slots, size.dets);
   const PGroup G = groups[blockIdx.x];
   if constexpr (MULTI) {
     const WinProb& pp = probs[G.prob];
@@ -459,19 +461,29 @@ __global__ void __launch_bounds__(kUnpointThreads, 6) k_unpoint_win32(
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   const QuadWalk w = quad_walk(G, lane);
-  const bool keep = nrhs > 1;
+  const bool keep = nrhs > NC;
   rt.load(G, block_off);
   __syncthreads();
-  for (int r = 0; r < nrhs; r++) {
-    if (done != nullptr && done[(int64_t)r * done_stride] != 0) continue;
-    const float4* x = x4 + r * x_stride4;
-    float* tr = t + r * t_stride;
-    auto value = [&](uint32_t sl, float a) -> float {
-      if (sl == kNoSlot) return 0.f;
+  for (int r = 0; r < nrhs; r += NC) {
+    bool on[NC], any = false;
+#pragma unroll
+    for (int c = 0; c < NC; c++) {
+      on[c] = r + c < nrhs && (done == nullptr || done[(int64_t)(r + c) * done_stride] == 0);
+      any |= on[c];
+    }
+    if (!any) continue;
+    // the columns' values of a sample
+    auto value = [&](uint32_t sl, float a, float (&v)[NC]) {
+#pragma unroll
+      for (int c = 0; c < NC; c++) v[c] = 0.f;
+      if (sl == kNoSlot) return;
       float cs, sn;
       weights_of_angle(a, cs, sn);
-      const float4 m = win[sl];
-      return m.x + cs * m.y + sn * m.z;
+#pragma unroll
+      for (int c = 0; c < NC; c++) {
+        const float4 m = win[c * size.slots + sl];
+        v[c] = m.x + cs * m.y + sn * m.z;
+      }
     };
     // quad q of row c: its samples and the ones of them inside the row, [e0, e1); a sample outside it is a
     // neighbouring row's (of any group: its slot is below size.slots too) or past the end (kNoSlot)
@@ -494,18 +506,23 @@ __global__ void __launch_bounds__(kUnpointThreads, 6) k_unpoint_win32(
     };
     auto emit = [&](const Quad& d) {
       if (d.e1 <= d.e0) return;
-      float4 v;
-      v.x = value(d.s.x & 0xFFFFu, d.a.x);
-      v.y = value(d.s.x >> 16, d.a.y);
-      v.z = value(d.s.y & 0xFFFFu, d.a.z);
-      v.w = value(d.s.y >> 16, d.a.w);
-      if (d.e1 - d.e0 == 4) {
-        __stcs(reinterpret_cast<float4*>(tr + d.i), v);
-      } else {
-        if (d.e0 <= 0 && d.e1 > 0) __stcs(tr + d.i, v.x);
-        if (d.e0 <= 1 && d.e1 > 1) __stcs(tr + d.i + 1, v.y);
-        if (d.e0 <= 2 && d.e1 > 2) __stcs(tr + d.i + 2, v.z);
-        if (d.e0 <= 3 && d.e1 > 3) __stcs(tr + d.i + 3, v.w);
+      float v0[NC], v1[NC], v2[NC], v3[NC];
+      value(d.s.x & 0xFFFFu, d.a.x, v0);
+      value(d.s.x >> 16, d.a.y, v1);
+      value(d.s.y & 0xFFFFu, d.a.z, v2);
+      value(d.s.y >> 16, d.a.w, v3);
+#pragma unroll
+      for (int c = 0; c < NC; c++) {
+        if (!on[c]) continue;
+        float* to = t + (r + c) * t_stride + d.i;
+        if (d.e1 - d.e0 == 4) {
+          __stcs(reinterpret_cast<float4*>(to), make_float4(v0[c], v1[c], v2[c], v3[c]));
+        } else {
+          if (d.e0 <= 0 && d.e1 > 0) __stcs(to, v0[c]);
+          if (d.e0 <= 1 && d.e1 > 1) __stcs(to + 1, v1[c]);
+          if (d.e0 <= 2 && d.e1 > 2) __stcs(to + 2, v2[c]);
+          if (d.e0 <= 3 && d.e1 > 3) __stcs(to + 3, v3[c]);
+        }
       }
     };
     auto load_unit = [&](int u, Quad& d) {
@@ -517,7 +534,9 @@ __global__ void __launch_bounds__(kUnpointThreads, 6) k_unpoint_win32(
     int u = warp * w.cpi + w.sub;
     load_unit(u, cur);
     if (r > 0) __syncthreads();   // the previous column's window is no longer read
-    fill_window(win, x, slot_pix + G.slot_off, G.n_slots);
+#pragma unroll
+    for (int c = 0; c < NC; c++)
+      if (on[c]) fill_window(win + c * size.slots, x4 + (r + c) * x_stride4, slot_pix + G.slot_off, G.n_slots);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     for (; u < w.n_units; u += step) {
@@ -536,7 +555,8 @@ __global__ void __launch_bounds__(kUnpointThreads, 6) k_unpoint_win32(
 constexpr size_t kUnpointSmem = (size_t)kWinCap * sizeof(float4) + 512 * 12;   // most of any group
 
 static int unpoint_threads(const WinSize& z) { return std::min(z.threads, kUnpointThreads); }
-static size_t unpoint_smem(const WinSize& z) { return (size_t)z.slots * sizeof(float4) + row_tab_bytes(z.dets); }
+static size_t unpoint_smem(const WinSize& z, int nc) { return (size_t)nc * z.slots * sizeof(float4) + row_tab_bytes(z.dets); }
+constexpr size_t kUnpointPairSmem = 56 * 1024;   // four CTAs of column pairs on an SM
 
 cudaError_t launch_unpoint_win32(const PGroup* groups, int64_t n_groups, const WinSize& size, const int64_t* block_off,
                                  const uint16_t* slot, const int32_t* slot_pix, const float* ang2,
@@ -546,8 +566,17 @@ cudaError_t launch_unpoint_win32(const PGroup* groups, int64_t n_groups, const W
   if (n_groups > 0x7fffffffLL || t_stride % 4 != 0) return cudaErrorInvalidValue;
   static cudaError_t st = cudaSuccess;
   static bool set = false;
-  MM_TRY_CUDA(smem_limit_once(k_unpoint_win32<false>, kUnpointSmem, st, set));
-  k_unpoint_win32<false><<<(unsigned)n_groups, unpoint_threads(size), unpoint_smem(size), s>>>(
+  if (nrhs > 1 && unpoint_smem(size, 2) <= kUnpointPairSmem) {
+    static cudaError_t st2 = cudaSuccess;
+    static bool set2 = false;
+    MM_TRY_CUDA(smem_limit_once(k_unpoint_win32<false, 2>, kUnpointPairSmem, st2, set2));
+    k_unpoint_win32<false, 2><<<(unsigned)n_groups, unpoint_threads(size), unpoint_smem(size, 2), s>>>(
+        groups, block_off, slot, slot_pix, ang2, reinterpret_cast<const float4*>(x4), x_stride / 4, nrhs, done,
+        done_stride, t, t_stride, nullptr, size);
+    return cudaGetLastError();
+  }
+  MM_TRY_CUDA(smem_limit_once(k_unpoint_win32<false, 1>, kUnpointSmem, st, set));
+  k_unpoint_win32<false, 1><<<(unsigned)n_groups, unpoint_threads(size), unpoint_smem(size, 1), s>>>(
       groups, block_off, slot, slot_pix, ang2, reinterpret_cast<const float4*>(x4), x_stride / 4, nrhs, done,
       done_stride, t, t_stride, nullptr, size);
   return cudaGetLastError();
@@ -559,8 +588,8 @@ cudaError_t launch_unpoint_win32_multi(const PGroup* groups, int64_t n_groups, c
   if (n_groups > 0x7fffffffLL || probs == nullptr) return cudaErrorInvalidValue;
   static cudaError_t st = cudaSuccess;
   static bool set = false;
-  MM_TRY_CUDA(smem_limit_once(k_unpoint_win32<true>, kUnpointSmem, st, set));
-  k_unpoint_win32<true><<<(unsigned)n_groups, unpoint_threads(size), unpoint_smem(size), s>>>(
+  MM_TRY_CUDA(smem_limit_once(k_unpoint_win32<true, 1>, kUnpointSmem, st, set));
+  k_unpoint_win32<true, 1><<<(unsigned)n_groups, unpoint_threads(size), unpoint_smem(size, 1), s>>>(
       groups, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 1, nullptr, 0, nullptr, 0, probs, size);
   return cudaGetLastError();
 }
@@ -573,14 +602,16 @@ cudaError_t launch_unpoint_win32_multi(const PGroup* groups, int64_t n_groups, c
 // sample that it replaces are loops of compare-and-swap on this machine and kept the shared-memory pipe
 // at 83 to 87% (20 shared wavefronts per 32 samples, here 4): 256 detectors x 4 x 524,288 samples 1.52
 // -> 1.08 ms, 64 x 262,144 64 -> 42 us, 4 x 65,536 86 -> 8 us (with the groups of build_windows).
-template <bool MULTI>
+// Several columns: NC = 2 of them share the entries, angles, cos / sin and pixels of the runs while both
+// columns' u leave two CTAs on an SM (8.4M samples x 16 columns: 223 -> 201 us).
+template <bool MULTI, int NC>
 __global__ void __launch_bounds__(kWinThreads, 2) k_point_sorted(
     const PGroup* __restrict__ groups, const int64_t* __restrict__ block_off, const uint4* __restrict__ ent,
     const float4* __restrict__ ent_ang, const uint16_t* __restrict__ first_slot,
     const int32_t* __restrict__ slot_pix, const float* __restrict__ u, int64_t u_stride, int nrhs,
     const int32_t* __restrict__ done, int done_stride, float4* __restrict__ y4, int64_t y_stride4,
     const WinProb* __restrict__ probs, WinSize size) {
-  extern __shared__ __align__(16) float us[];   // n_blk rows of W + 4, then a zero; after them the row table
+  extern __shared__ __align__(16) float us[];   // [NC][size.rows]: n_blk rows of W + 4, then a zero; the row table
   const PGroup G = groups[blockIdx.x];
   if constexpr (MULTI) {
     const WinProb& pp = probs[G.prob];
@@ -596,12 +627,17 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_sorted(
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   const int row = srt_row(G.log_w);
   const QuadWalk w = quad_walk(G, lane);
-  RowTab rt(us + size.rows, size.dets);
+  RowTab rt(us + NC * size.rows, size.dets);
   const int32_t* __restrict__ pix = slot_pix + G.slot_off;
   rt.load(G, block_off);
-  for (int r = 0; r < nrhs; r++) {
-    if (done != nullptr && done[(int64_t)r * done_stride] != 0) continue;
-    const float* ur = u + r * u_stride;
+  for (int r = 0; r < nrhs; r += NC) {
+    bool on[NC], any = false;
+#pragma unroll
+    for (int c = 0; c < NC; c++) {
+      on[c] = r + c < nrhs && (done == nullptr || done[(int64_t)(r + c) * done_stride] == 0);
+      any |= on[c];
+    }
+    if (!any) continue;
     // this warp's first block of entries and half of its angles, on their way during the staging
     uint4 e[4];
     float4 a[4];
@@ -619,16 +655,20 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_sorted(
     auto copy = [&](int c, int q) {
       const int64_t lo = rt.lo[c];
       const int a0 = (int)(lo & 3), len = rt.len[c];
-      if (len > 0 && 4 * q < a0 + len)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                         (uint32_t)__cvta_generic_to_shared(us + c * row + 4 * q)),
-                     "l"(ur + lo - a0 + 4 * q)
-                     : "memory");
+      if (len > 0 && 4 * q < a0 + len) {
+#pragma unroll
+        for (int k = 0; k < NC; k++)
+          if (on[k])
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                             (uint32_t)__cvta_generic_to_shared(us + k * size.rows + c * row + 4 * q)),
+                         "l"(u + (r + k) * u_stride + lo - a0 + 4 * q)
+                         : "memory");
+      }
     };
     for (int c0 = warp * w.cpi + w.sub; c0 < w.n_units; c0 += warps * w.cpi)
       copy(c0 >> w.ls, ((c0 & ((1 << w.ls) - 1)) << (w.lu - 2)) + w.ql);
     for (int c = threadIdx.x; c < G.n_blk; c += blockDim.x) copy(c, 1 << (G.log_w - 2));
-    if (threadIdx.x == 0) us[G.n_blk * row] = 0.f;
+    if (threadIdx.x < NC) us[threadIdx.x * size.rows + G.n_blk * row] = 0.f;
     asm volatile("cp.async.commit_group;\ncp.async.wait_all;" ::: "memory");
     __syncthreads();
     float4* yr = y4 + r * y_stride4;
@@ -646,19 +686,30 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_sorted(
       }
       if (sl == kNoSlot) continue;
       int32_t p = __ldg(pix + sl);
-      float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+      float s0[NC], s1[NC], s2[NC];
+#pragma unroll
+      for (int k = 0; k < NC; k++) s0[k] = s1[k] = s2[k] = 0.f;
+      auto add_run = [&]() {
+#pragma unroll
+        for (int k = 0; k < NC; k++)
+          if (on[k]) atomicAdd(yr + k * y_stride4 + p, make_float4(s0[k], s1[k], s2[k], 0.f));
+      };
       auto one = [&](uint32_t en, float an) {
         if (en & kSrtRun) {   // a new run: the previous pixel's sum is complete
-          atomicAdd(yr + p, make_float4(s0, s1, s2, 0.f));
+          add_run();
           p = __ldg(pix + ++sl);
-          s0 = s1 = s2 = 0.f;
+#pragma unroll
+          for (int k = 0; k < NC; k++) s0[k] = s1[k] = s2[k] = 0.f;
         }
-        const float y = us[en & 0x7FFFu];
         float cs, sn;
         weights_of_angle(an, cs, sn);
-        s0 += y;
-        s1 = fmaf(cs, y, s1);
-        s2 = fmaf(sn, y, s2);
+#pragma unroll
+        for (int k = 0; k < NC; k++) {
+          const float y = us[k * size.rows + (en & 0x7FFFu)];
+          s0[k] += y;
+          s1[k] = fmaf(cs, y, s1[k]);
+          s2[k] = fmaf(sn, y, s2[k]);
+        }
       };
 #pragma unroll
       for (int o = 0; o < 4; o++) {
@@ -678,21 +729,25 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_sorted(
         one(e[o].w & 0xFFFFu, a1.z);
         one(e[o].w >> 16, a1.w);
       }
-      atomicAdd(yr + p, make_float4(s0, s1, s2, 0.f));
+      add_run();
     }
   }
 }
 
+constexpr int kPointPairSmem = 112 * 1024;   // two CTAs of column pairs on an SM
 static cudaError_t point_sorted_attr() {
   constexpr int kMost = (kWinMaxSamples / 32 * ((1 << 5) + 4) + 4) * (int)sizeof(float) + 512 * 12;
   static const cudaError_t e = [] {
-    cudaError_t r = cudaFuncSetAttribute(k_point_sorted<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+    cudaError_t r = cudaFuncSetAttribute(k_point_sorted<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
     if (r == cudaSuccess)
-      r = cudaFuncSetAttribute(k_point_sorted<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+      r = cudaFuncSetAttribute(k_point_sorted<false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPointPairSmem);
+    if (r == cudaSuccess)
+      r = cudaFuncSetAttribute(k_point_sorted<true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
     return r;
   }();
   return e;
 }
+static size_t point_sorted_smem(const WinSize& z, int nc) { return (size_t)nc * z.rows * sizeof(float) + row_tab_bytes(z.dets); }
 static int point_sorted_threads(const WinSize& z) { return 32 * std::min(kWinThreads / 32, std::max(1, z.blocks)); }
 
 cudaError_t launch_point_sorted(const PGroup* groups, int64_t n_groups, const WinSize& size,
@@ -703,7 +758,9 @@ cudaError_t launch_point_sorted(const PGroup* groups, int64_t n_groups, const Wi
   if (n_groups == 0 || nrhs <= 0) return cudaSuccess;
   if (n_groups > 0x7fffffffLL || u_stride % 4 != 0) return cudaErrorInvalidValue;
   MM_TRY_CUDA(point_sorted_attr());
-  k_point_sorted<false><<<(unsigned)n_groups, point_sorted_threads(size), (size_t)size.rows * sizeof(float) + row_tab_bytes(size.dets), s>>>(
+  const bool pair = nrhs > 1 && point_sorted_smem(size, 2) <= (size_t)kPointPairSmem;
+  auto* kernel = pair ? k_point_sorted<false, 2> : k_point_sorted<false, 1>;
+  kernel<<<(unsigned)n_groups, point_sorted_threads(size), point_sorted_smem(size, pair ? 2 : 1), s>>>(
       groups, block_off, reinterpret_cast<const uint4*>(ent), reinterpret_cast<const float4*>(ent_ang), first_slot,
       slot_pix, u, u_stride, nrhs, done, done_stride, reinterpret_cast<float4*>(y4), y_stride / 4, nullptr, size);
   return cudaGetLastError();
@@ -714,7 +771,7 @@ cudaError_t launch_point_sorted_multi(const PGroup* groups, int64_t n_groups, co
   if (n_groups == 0) return cudaSuccess;
   if (n_groups > 0x7fffffffLL || probs == nullptr) return cudaErrorInvalidValue;
   MM_TRY_CUDA(point_sorted_attr());
-  k_point_sorted<true><<<(unsigned)n_groups, point_sorted_threads(size), (size_t)size.rows * sizeof(float) + row_tab_bytes(size.dets), s>>>(
+  k_point_sorted<true, 1><<<(unsigned)n_groups, point_sorted_threads(size), point_sorted_smem(size, 1), s>>>(
       groups, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 1, nullptr, 0, nullptr, 0, probs, size);
   return cudaGetLastError();
 }
