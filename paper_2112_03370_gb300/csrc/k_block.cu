@@ -326,6 +326,22 @@ __global__ void __launch_bounds__(kNT) k_bcombine(TO* __restrict__ out, const in
 // Narrow blocks (v, t <= kCombJ): each thread streams pixels (grid-stride) and forms all v outputs
 // of its pixel in registers; no staging, so a column or two costs one pass over A.
 constexpr int kCombJ = 16;
+// columns whose loads are in flight together: FP32 outputs 4 (65,536 pixels, 16 x 16: 18.8 -> 11.5 us: one column's
+// load at a time, and each output read after the last one's store, waited for memory); FP64 outputs 1 (30 us, with
+// 4 columns' 32-byte pixels in registers 35)
+template <typename TO>
+constexpr int kCombU = sizeof(TO) == sizeof(float4) ? 4 : 1;
+__device__ __forceinline__ float4 load_pixel(const float4* o) { return *o; }
+__device__ __forceinline__ void store_pixel(float4* o, float4 v) { *o = v; }
+// 16-byte accesses to the pixel's 32 bytes
+__device__ __forceinline__ double4_16a load_pixel(const double4_16a* o) {
+  const double2 a = reinterpret_cast<const double2*>(o)[0], b = reinterpret_cast<const double2*>(o)[1];
+  return double4_16a{a.x, a.y, b.x, b.y};
+}
+__device__ __forceinline__ void store_pixel(double4_16a* o, double4_16a v) {
+  reinterpret_cast<double2*>(o)[0] = make_double2(v.x, v.y);
+  reinterpret_cast<double2*>(o)[1] = make_double2(v.z, v.w);
+}
 template <typename TO, int J>
 __global__ void __launch_bounds__(kNT) k_bcombine_stream(TO* __restrict__ out, const int* __restrict__ idx_out,
                                                    int v, const float4* __restrict__ A, int t,
@@ -333,6 +349,7 @@ __global__ void __launch_bounds__(kNT) k_bcombine_stream(TO* __restrict__ out, c
                                                    int mode, int64_t n, double* __restrict__ norm_part) {
   __shared__ float cs[kMaxBlk * kMaxBlk];
   __shared__ double red[J][kNT / 32];
+  constexpr int kU = kCombU<TO>;
   for (int e = threadIdx.x; e < t * v; e += kNT) cs[e] = (float)(sign * C[(e / v) * ldc + (e % v)]);
   __syncthreads();
   for (int j0 = 0; j0 < v; j0 += J) {
@@ -344,36 +361,47 @@ __global__ void __launch_bounds__(kNT) k_bcombine_stream(TO* __restrict__ out, c
       float ax[J], ay[J], az[J];
 #pragma unroll
       for (int jj = 0; jj < J; jj++) ax[jj] = ay[jj] = az[jj] = 0.f;
-      for (int i = 0; i < t; i++) {
-        const float4 a = __ldg(A + (int64_t)i * n + p);
+      for (int i0 = 0; i0 < t; i0 += kU) {
+        float4 a[kU];
 #pragma unroll
-        for (int jj = 0; jj < J; jj++) {
-          const float c = (jj < nj) ? cs[i * v + j0 + jj] : 0.f;
-          ax[jj] = fmaf(a.x, c, ax[jj]);
-          ay[jj] = fmaf(a.y, c, ay[jj]);
-          az[jj] = fmaf(a.z, c, az[jj]);
+        for (int u = 0; u < kU; u++)
+          a[u] = i0 + u < t ? __ldg(A + (int64_t)(i0 + u) * n + p) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < kU; u++) {
+          if (i0 + u >= t) break;
+#pragma unroll
+          for (int jj = 0; jj < J; jj++) {
+            const float c = (jj < nj) ? cs[(i0 + u) * v + j0 + jj] : 0.f;
+            ax[jj] = fmaf(a[u].x, c, ax[jj]);
+            ay[jj] = fmaf(a[u].y, c, ay[jj]);
+            az[jj] = fmaf(a[u].z, c, az[jj]);
+          }
         }
       }
 #pragma unroll
-      for (int jj = 0; jj < J; jj++) {
-        if (jj >= nj) break;
-        const int64_t col = idx_out ? idx_out[j0 + jj] : (j0 + jj);
-        if constexpr (sizeof(TO) == sizeof(float4)) {
-          float4* o = reinterpret_cast<float4*>(out) + col * n + p;
-          float4 cur = mode ? *o : make_float4(0.f, 0.f, 0.f, 0.f);
-          cur.x += ax[jj]; cur.y += ay[jj]; cur.z += az[jj];
-          cur.w = 0.f;
-          *o = cur;
-        } else {
-          // 16-byte accesses to the pixel's 32 bytes
-          double2* o = reinterpret_cast<double2*>(out) + 2 * (col * n + p);
-          double2 xy = mode ? o[0] : make_double2(0.0, 0.0);
-          double2 zw = mode ? o[1] : make_double2(0.0, 0.0);
-          xy.x += f32_to_f64_bits(ax[jj]); xy.y += f32_to_f64_bits(ay[jj]); zw.x += f32_to_f64_bits(az[jj]);
-          zw.y = 0.0;
-          o[0] = xy;
-          o[1] = zw;
-          if (norm_part) nrm[jj] += xy.x * xy.x + xy.y * xy.y + zw.x * zw.x;
+      for (int j1 = 0; j1 < J; j1 += kU) {
+        TO cur[kU];   // kU columns' pixels before the first of them is stored
+        int64_t at[kU];
+#pragma unroll
+        for (int u = 0; u < kU; u++) {
+          if (j1 + u < nj) {
+            at[u] = (idx_out ? idx_out[j0 + j1 + u] : (j0 + j1 + u)) * n + p;
+            if (mode) cur[u] = load_pixel(out + at[u]);
+            else cur[u] = TO{};
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kU; u++) {
+          const int jj = j1 + u;
+          if (jj >= nj) break;
+          if constexpr (sizeof(TO) == sizeof(float4)) {
+            cur[u].x += ax[jj]; cur[u].y += ay[jj]; cur[u].z += az[jj];
+          } else {
+            cur[u].x += f32_to_f64_bits(ax[jj]); cur[u].y += f32_to_f64_bits(ay[jj]); cur[u].z += f32_to_f64_bits(az[jj]);
+            if (norm_part) nrm[jj] += cur[u].x * cur[u].x + cur[u].y * cur[u].y + cur[u].z * cur[u].z;
+          }
+          cur[u].w = 0;
+          store_pixel(out + at[u], cur[u]);
         }
       }
     }
