@@ -92,12 +92,12 @@ def fft_flops_per_sample(L: int, lam: int) -> float:
 
 
 def kernel_source_hash() -> str:
-    """Hash of the FP32 N^-1 tile kernel's own source (k_toeplitz.cu, fft_smem.cuh, df64.cuh and
-    the TileArgs definition it is compiled against)."""
+    """Hash of the FP32 N^-1 tile kernel's own source (k_ninv32.cu, fft_reg.cuh and the TileArgs
+    definition it is compiled against)."""
     import hashlib
     h = hashlib.sha256()
     d = os.path.join(ROOT, "paper_2112_03370_gb300", "csrc")
-    for f in ("df64.cuh", "fft_smem.cuh", "k_toeplitz.cu"):
+    for f in ("fft_reg.cuh", "k_ninv32.cu"):
         h.update(open(os.path.join(d, f), "rb").read())
     internal = open(os.path.join(d, "mm_internal.cuh")).read()
     a = internal.index("struct TileArgs")
@@ -458,7 +458,7 @@ def run_ours(a):
     apply_alg_bytes = 8.0 * N + 6.0 * n_obs * 4   # the fused floor of the A-application (8 B/sample)
     roof = {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
             "frac": achieved / fp32_peak, "traffic": measured_traffic(N),
-            "kernel": "k_tile<float,1,MODE_NINV_T> (overlap-save FFT N^-1, L = 32768: "
+            "kernel": "k_ninv32 (overlap-save FFT N^-1, transform in registers, L = 32768: "
                       f"{fft_flops_per_sample(L, cfg.lam):.0f} flops per output sample)",
             "peak_kind": f"derived: {n_sm} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 x "
                          f"{sm_max:.0f} MHz ({pk_kind} sm_max_mhz)",
@@ -469,7 +469,7 @@ def run_ours(a):
             "unpoint_kernel": {"name": "k_unpoint_win32 (t = P x over pixel windows)",
                                "ms_per_launch": t_up * 1e3, "achieved_gbs": win_bytes / t_up / 1e9,
                                "hbm_frac": win_bytes / t_up / 1e9 / hbm_peak, "bound": "hbm"},
-            "point_kernel": {"name": "k_point_win32 (y += P^T u over pixel windows)",
+            "point_kernel": {"name": "k_point_sorted (y += P^T u over pixel windows)",
                              "ms_per_launch": t_pt * 1e3, "achieved_gbs": win_bytes / t_pt / 1e9,
                              "hbm_frac": win_bytes / t_pt / 1e9 / hbm_peak, "bound": "hbm"},
             "a_apply_ms": t_apply * 1e3,
@@ -1011,7 +1011,7 @@ def run_serving(a, n_requests=None, compare_fp64=0):
         "iters_mean": float(np.mean([i.iters for i in infos])),
         "arrivals": "absolute Poisson schedule", "submit_ms_mean": sub[0], "submit_ms_max": sub[1],
         "mode": "FP32 iterations batched per launch across requests (P, N^-1 and P^T over pixel windows "
-                "and segments, three launches per step), double-float rhs and replacement"}
+                "and segments, CG steps in one more launch), double-float rhs and replacement"}
     if compare_fp64:
         k = min(compare_fp64, n_requests)
         lat64, inf64, dt64, _ = _serve(mm, pool, order[:k], gaps[:k], fp64=True)

@@ -276,7 +276,7 @@ typedef struct {
   int32_t n_rejected;        /* candidates not chosen because their A x differed */
   int32_t seg_sub;           /* chosen P^T: sub-window samples of the segment reduction, 0 = windows */
   int32_t n_seg;
-  int32_t seg_cand[4];       /* 0 = per-sample sums over the windows, else sub-window samples */
+  int32_t seg_cand[4];       /* 0 = run sums over the sorted groups, else sub-window samples */
   double seg_ms[4];
 } mm_tune_info;
 int mm_autotune(mm_plan_t plan, int max_width, mm_tune_info* out, void* stream);
@@ -429,7 +429,7 @@ int mm_deflation_apply(mm_plan_t plan, const double* r, double* z, int nrhs, voi
  * per step; requests join between steps once planned and leave when they finish.  Their state
  * stays resident until then.
  *   FP32 requests (opts->precision MM_FP32): FP32 operators over pixel windows, P, N^-1 and P^T of
- *     all such requests in three shared launches per step (all their window groups, all their
+ *     all such requests in shared launches per step (all their window groups, all their
  *     tile segments); right-hand side and residual replacement per request with the double-float
  *     FP64-class operators, as mm_pcg_solve on an MM_FP32_DF64 plan (the request's
  *     desc->precision is ignored).  A failed launch or copy ends the running requests with

@@ -17,10 +17,12 @@
 // instead of the 16 of in-place passes in shared memory, which were bound by the shared-memory pipe
 // and instruction issue (89k warp instructions and 22.8k shared wavefronts in 40k cycles per
 // 32768-sample tile; here 54k and 11.2k in 25k cycles).  What bounds it now: latency at 16 warps per
-// SM between the arithmetic (FMA pipe 51% busy) and the shared-memory pipe (54%).
+// SM between the arithmetic (FMA pipe 53% busy, its throttle the first of the stalls) and the shared-memory
+// pipe (50%).
 // Measured (GB300, t and u in HBM, kernel alone, before -> now): 512 blocks x 524,288 samples, lambda
 // 8192: 2.18 -> 1.34 ms; 256 x 524,288, lambda 1024: 0.69 -> 0.35 ms; 64 x 262,144, lambda 2048:
-// 120 -> 64 us; 4 x 65,536, lambda 1024: 28 -> 10 us.
+// 120 -> 64 us; 4 x 65,536, lambda 1024: 28 -> 10 us (plus 4% since the rotation constants carry their low
+// parts, fft_reg.cuh).
 //
 // Geometry by tile size: 32768 samples R1 = R2 = 32 (512 threads, one CTA per SM), 16384 samples
 // 32 x 16 (256 threads, two), 8192 samples 16 x 16 (128 threads, four).

@@ -1561,7 +1561,7 @@ struct Server {
   mm_req_t next_id = 1;
   std::thread th;
   // one server step's launches: requests with pixel windows run P, N^-1 and P^T over all their
-  // groups and segments in three launches (wgroups / wprobs, ntiles / nprobs); requests whose plan
+  // groups and segments (N^-1 in one launch per tile size; wgroups / wprobs, ntiles / nprobs); requests whose plan
   // has no windows run the fused tiles (un-pointing in the gather, per-sample scatter) in one
   TileDesc* tiles_dev = nullptr;
   size_t tiles_cap = 0;
@@ -1866,7 +1866,7 @@ void server_loop(Server* S) {
     const int nb = (int)S->running.size();
     for (Request* r : S->running) r->batch = std::max(r->batch, nb);
     // one PCG iteration of every running request: the FP32 requests' A-applications in shared
-    // launches (three over the pixel windows and segments, one of fused tiles for plans without
+    // launches (over the pixel windows and segments, one of fused tiles for plans without
     // windows), the FP64-class requests' own operator launches after them
     cudaStream_t s = S->stream;
     bool ok = true;
@@ -2579,7 +2579,7 @@ int mm_autotune(mm_plan_t plan, int max_width, mm_tune_info* out, void* stream) 
     }
   }
   P->win_samples = best_win;
-  // 2b. the FP32 P^T: per-sample sums over the windows, or segment reduction over pixel-sorted
+  // 2b. the FP32 P^T: run sums over the sorted groups, or segment reduction over pixel-sorted
   // sub-windows of a few sizes (each size rebuilds the windows)
   int best_seg = 0;
   if (P->precision == MM_FP32) {
