@@ -372,7 +372,9 @@ __global__ void k_cg_init(CgWork w) {
 __global__ void k_cg_pupdate(CgWork w) {
   const int col = blockIdx.y;
   const CgScalars& s = w.scal[col];
-  if (s.halt) return;
+  // fused works: k_cg_step forms p, this kernel the first one after the start or a replacement only; a
+  // column that iterates beside a replaced one has its next p already
+  if (s.halt || (w.fused && s.since_rep != 0)) return;
   const double beta = s.beta;
   const double* z = col4(w.z, w, col);
   double* p = col4(w.p, w, col);
