@@ -407,7 +407,7 @@ int choose_ninv_logm(const std::vector<int64_t>& off, int lam, bool shared) {
   const double us[3] = {10.6, 11.5, 13.5};
   for (int logm = kNinvLogMax; logm >= kNinvLogMin; logm--) {
     const int64_t vmax = ((int64_t)2 << logm) - 2 * (int64_t)lam - 4;
-    if (vmax <= 0) break;
+    if (vmax < 4) break;   // make_tiles would be left without an output for some block starts
     int64_t n = 0;
     for (size_t b = 0; b + 1 < off.size(); b++) n += (off[b + 1] - off[b] + vmax - 1) / vmax;
     const int64_t slots = (int64_t)sm_count() << (kNinvLogMax - logm);
@@ -431,7 +431,7 @@ int choose_logm64(const std::vector<int64_t>& off, int lam) {
   double best_t = 1e300;
   for (int logm = kLogM; logm >= 11; logm--) {
     const int64_t vmax = ((int64_t)2 << logm) - 2 * (int64_t)lam - 4;
-    if (vmax <= 0) break;
+    if (vmax < 4) break;   // as in choose_ninv_logm
     int64_t n = 0;
     for (size_t b = 0; b + 1 < off.size(); b++) n += (off[b + 1] - off[b] + vmax - 1) / vmax;
     const int64_t sms = logm == kLogM ? sm_count() / 2 : sm_count();
