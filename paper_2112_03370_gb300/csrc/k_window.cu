@@ -594,6 +594,36 @@ cudaError_t launch_unpoint_win32_multi(const PGroup* groups, int64_t n_groups, c
   return cudaGetLastError();
 }
 
+// The map that this CTA's group adds to (PtMaps), y4 or one of the extra ones of `stride4` pixels.
+__device__ __forceinline__ float4* group_map(float4* y4, int64_t stride4, const PtMaps& maps) {
+  const int k = blockIdx.x & (maps.n - 1);
+  return k == 0 ? y4 : reinterpret_cast<float4*>(maps.extra) + (k - 1) * stride4;
+}
+
+__global__ void k_sum_maps(PtMaps maps, int64_t stride4, const int32_t* __restrict__ done, int done_stride,
+                           float4* __restrict__ y4, int64_t n) {
+  if (done != nullptr && done[(int64_t)blockIdx.y * done_stride] != 0) return;
+  const int64_t col = blockIdx.y * n;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    float4 v = y4[col + i];
+    for (int k = 1; k < maps.n; k++) {
+      const float4 e = __ldcs(reinterpret_cast<const float4*>(maps.extra) + (k - 1) * stride4 + col + i);
+      v.x += e.x;
+      v.y += e.y;
+      v.z += e.z;
+    }
+    y4[col + i] = v;
+  }
+}
+cudaError_t launch_sum_maps(const PtMaps& maps, int nrhs, const int32_t* done, int done_stride, float* y4,
+                            int64_t y_stride, cudaStream_t s) {
+  const int64_t n = y_stride / 4;
+  if (maps.n <= 1 || n == 0 || nrhs <= 0) return cudaSuccess;
+  const dim3 grid((unsigned)std::min<int64_t>((n + 255) / 256, 8 * (int64_t)sm_count()), nrhs);
+  k_sum_maps<<<grid, 256, 0, s>>>(maps, nrhs * n, done, done_stride, reinterpret_cast<float4*>(y4), n);
+  return cudaGetLastError();
+}
+
 // y += P^T u by run sums: one CTA per group.  The group's u goes to shared memory by 16-byte
 // asynchronous copies; then every lane walks 32 consecutive pixel-sorted entries (position, angle),
 // sums u, u cos 2psi, u sin 2psi of a run of equal pixels in registers and adds each run to the map
@@ -610,7 +640,7 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_sorted(
     const float4* __restrict__ ent_ang, const uint16_t* __restrict__ first_slot,
     const int32_t* __restrict__ slot_pix, const float* __restrict__ u, int64_t u_stride, int nrhs,
     const int32_t* __restrict__ done, int done_stride, float4* __restrict__ y4, int64_t y_stride4,
-    const WinProb* __restrict__ probs, WinSize size) {
+    const WinProb* __restrict__ probs, WinSize size, PtMaps maps) {
   extern __shared__ __align__(16) float us[];   // [NC][size.rows]: n_blk rows of W + 4, then a zero; the row table
   const PGroup G = groups[blockIdx.x];
   if constexpr (MULTI) {
@@ -621,8 +651,10 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_sorted(
     first_slot = pp.srt_slot;
     slot_pix = pp.slot_pix;
     u = pp.u;
-    y4 = reinterpret_cast<float4*>(pp.y);
+    y4 = group_map(reinterpret_cast<float4*>(pp.y), pp.n_obs, pp.maps);
     done = pp.done;
+  } else {
+    y4 = group_map(y4, nrhs * y_stride4, maps);
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   const int row = srt_row(G.log_w);
@@ -754,7 +786,7 @@ cudaError_t launch_point_sorted(const PGroup* groups, int64_t n_groups, const Wi
                                 const int64_t* block_off, const uint16_t* ent, const float* ent_ang,
                                 const uint16_t* first_slot, const int32_t* slot_pix, const float* u,
                                 int64_t u_stride, int nrhs, const int32_t* done, int done_stride, float* y4,
-                                int64_t y_stride, cudaStream_t s) {
+                                int64_t y_stride, const PtMaps& maps, cudaStream_t s) {
   if (n_groups == 0 || nrhs <= 0) return cudaSuccess;
   if (n_groups > 0x7fffffffLL || u_stride % 4 != 0) return cudaErrorInvalidValue;
   MM_TRY_CUDA(point_sorted_attr());
@@ -762,7 +794,8 @@ cudaError_t launch_point_sorted(const PGroup* groups, int64_t n_groups, const Wi
   auto* kernel = pair ? k_point_sorted<false, 2> : k_point_sorted<false, 1>;
   kernel<<<(unsigned)n_groups, point_sorted_threads(size), point_sorted_smem(size, pair ? 2 : 1), s>>>(
       groups, block_off, reinterpret_cast<const uint4*>(ent), reinterpret_cast<const float4*>(ent_ang), first_slot,
-      slot_pix, u, u_stride, nrhs, done, done_stride, reinterpret_cast<float4*>(y4), y_stride / 4, nullptr, size);
+      slot_pix, u, u_stride, nrhs, done, done_stride, reinterpret_cast<float4*>(y4), y_stride / 4, nullptr, size,
+      maps);
   return cudaGetLastError();
 }
 
@@ -772,7 +805,7 @@ cudaError_t launch_point_sorted_multi(const PGroup* groups, int64_t n_groups, co
   if (n_groups > 0x7fffffffLL || probs == nullptr) return cudaErrorInvalidValue;
   MM_TRY_CUDA(point_sorted_attr());
   k_point_sorted<true, 1><<<(unsigned)n_groups, point_sorted_threads(size), point_sorted_smem(size, 1), s>>>(
-      groups, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 1, nullptr, 0, nullptr, 0, probs, size);
+      groups, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 1, nullptr, 0, nullptr, 0, probs, size, PtMaps{});
   return cudaGetLastError();
 }
 
@@ -892,7 +925,7 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_seg32(
     const PGroup* __restrict__ groups, const int64_t* __restrict__ block_off, const uint32_t* __restrict__ ent,
     const float* __restrict__ ent_ang, const int32_t* __restrict__ kept, const int32_t* __restrict__ slot_pix,
     int sub_cap, const float* __restrict__ u, int64_t u_stride, int nrhs, const int32_t* __restrict__ done,
-    int done_stride, float4* __restrict__ y4, int64_t y_stride4) {
+    int done_stride, float4* __restrict__ y4, int64_t y_stride4, PtMaps maps) {
   extern __shared__ __align__(16) float smem_f[];
   float* acc = smem_f;                   // [3][kAccStride]
   float* us = smem_f + 3 * kAccStride;   // [sub_cap] u of the sub-window, sample l at us[l]
@@ -905,6 +938,7 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_point_seg32(
   S.log_w = ls;
   const ChunkWalk cw = chunk_walk(S.log_w, lane);
   const int n_pad = acc_index(G.n_slots);
+  y4 = group_map(y4, nrhs * y_stride4, maps);
   for (int r = 0; r < nrhs; r++) {
     if (done != nullptr && done[(int64_t)r * done_stride] != 0) continue;
     const float* ur = u + r * u_stride;
@@ -1018,7 +1052,7 @@ cudaError_t launch_point_seg32(const PGroup* groups, int64_t n_groups, const int
                                const uint32_t* ent, const float* ent_ang, const int32_t* kept,
                                const int32_t* slot_pix, int sub_cap, const float* u, int64_t u_stride,
                                int nrhs, const int32_t* done, int done_stride, float* y4, int64_t y_stride,
-                               cudaStream_t s) {
+                               const PtMaps& maps, cudaStream_t s) {
   if (n_groups == 0 || nrhs <= 0) return cudaSuccess;
   if (n_groups > 0x7fffffffLL || u_stride % 4 != 0 || sub_cap < 32 || sub_cap > kSegSubMax)
     return cudaErrorInvalidValue;
@@ -1028,7 +1062,7 @@ cudaError_t launch_point_seg32(const PGroup* groups, int64_t n_groups, const int
   MM_TRY_CUDA(smem_limit_once(k_point_seg32, kPointSegSmemMax, st, set));
   k_point_seg32<<<(unsigned)n_groups, kWinThreads, smem, s>>>(groups, block_off, ent, ent_ang, kept, slot_pix,
                                                                sub_cap, u, u_stride, nrhs, done, done_stride,
-                                                               reinterpret_cast<float4*>(y4), y_stride / 4);
+                                                               reinterpret_cast<float4*>(y4), y_stride / 4, maps);
   return cudaGetLastError();
 }
 

@@ -204,7 +204,7 @@ void free_plan(Plan* P) {
   dfree(P->map64_in); dfree(P->map64_out); dfree(P->td_a); dfree(P->td_b); dfree(P->t32);
   dfree(P->wdf); dfree(P->tabdf); dfree(P->twdf); dfree(P->tw64_first); dfree(P->twdf_first); dfree(P->tdf); dfree(P->mapdf);
   dfree(P->ang2); dfree(P->groups); dfree(P->slot); dfree(P->slot_pix); dfree(P->u32);
-  dfree(P->srt_ent); dfree(P->srt_ang); dfree(P->srt_slot);
+  dfree(P->srt_ent); dfree(P->srt_ang); dfree(P->srt_slot); dfree(P->ptmap);
   dfree(P->seg_ent); dfree(P->seg_ang); dfree(P->seg_kept);
   dfree(P->udf); dfree(P->amax);
   dfree(P->tc_tiles); dfree(P->tc_tab); dfree(P->tc_scale); dfree(P->tc_err);
@@ -596,7 +596,7 @@ int build_windows(Plan* P, cudaStream_t s) {
   });
   int64_t total = 0;
   const bool seg = P->precision == MM_FP32 && P->use_seg;   // pixel-sorted sub-windows (FP32 P^T)
-  int64_t n_ent = 0, n_sub = 0, n_srt = 0;
+  int64_t n_ent = 0, n_sub = 0, n_srt = 0, adds = 0;
   for (PGroup& g : done) {
     g.slot_off = total;
     total += g.n_slots;
@@ -608,6 +608,7 @@ int build_windows(Plan* P, cudaStream_t s) {
     g.srt_off = n_srt;
     g.n_srt = (int32_t)((samples + kSrtBlock - 1) / kSrtBlock);
     n_srt += g.n_srt;
+    adds += g.n_slots + (samples + 31) / 32;   // one per run of equal slots, and where a lane's range cuts one
     P->win_size.cover(WinSize{0, g.n_slots, g.n_blk, g.n_blk * srt_row(g.log_w) + 4, g.n_srt});
     const int ls = seg_log_s(g.n_blk, g.log_w, P->seg_sub);
     g.sub0 = (int32_t)n_sub;
@@ -618,6 +619,8 @@ int build_windows(Plan* P, cudaStream_t s) {
   if (seg && n_sub > 0x7fffffffLL) return fail(MM_EINVAL, "pixel windows: too many sub-windows");
   P->n_groups = (int64_t)done.size();
   P->n_slots_total = total;
+  P->pt_maps = 1;
+  while (P->pt_maps < kPtMaps && adds > (int64_t)kPtAdds * P->pt_maps * P->n_obs) P->pt_maps *= 2;
   P->win_repeat = total > 0 ? (double)P->N / (double)total : 0.0;
   MM_TRY(dalloc(P, &P->groups, done.size()));
   // the un-point kernel reads whole quads: up to 3 slots past the end, which must be valid ones
@@ -1142,6 +1145,9 @@ int split32_cols(const Plan* P, int nrhs) {
   return (int)std::min<size_t>((size_t)nrhs, kSplitTBytes / per);
 }
 
+// floats of the extra maps of P^T (PtMaps) for `cols` columns
+size_t ptmap_elems(const Plan* P, int cols) { return P->groups ? (size_t)(P->pt_maps - 1) * cols * P->n_obs * 4 : 0; }
+
 int ensure_t32(Plan* P, int nrhs) {
   const int k = split32_cols(P, nrhs);
   if (k == 0) return MM_OK;
@@ -1160,19 +1166,36 @@ int ensure_t32(Plan* P, int nrhs) {
     MM_TRY(dalloc(P, &P->u32, t_elems));
     P->u32_cap = t_elems;
   }
+  if (P->ptmap_cap < ptmap_elems(P, k)) {
+    dfree(P->ptmap);
+    P->bytes -= P->ptmap_cap * sizeof(float);
+    P->ptmap_cap = 0;
+    P->buf_gen++;
+    MM_TRY(dalloc(P, &P->ptmap, ptmap_elems(P, k)));
+    P->ptmap_cap = ptmap_elems(P, k);
+  }
   return MM_OK;
 }
 
 // y4 += P^T u (FP32) of a plan with pixel windows: segment reduction over the pixel-sorted
-// sub-windows, or run sums over the pixel-sorted groups
+// sub-windows, or run sums over the pixel-sorted groups.  Plans whose pixels get many additions spread
+// them over several maps.  Full ground workload (1.07e9 samples, 153 additions per pixel), one map -> four:
+// FP32 A x against double-float 1.89e-7 -> 1.00e-7 of its norm, mixed map against the double-float map 6.7 to
+// 10.1e-6 -> 2.4 to 3.8e-6 (six solves each), A x 10.35 ms either way.
 cudaError_t point32(Plan* P, const float* u, int64_t u_stride, int nrhs, const int32_t* done, int done_stride,
                     float* y4, int64_t y_stride, cudaStream_t s) {
+  const PtMaps maps{P->ptmap, P->pt_maps};
+  cudaError_t e = cudaSuccess;
+  if (maps.n > 1)
+    e = cudaMemsetAsync(P->ptmap, 0, (size_t)(maps.n - 1) * nrhs * y_stride * sizeof(float), s);
+  if (e != cudaSuccess) return e;
   if (P->use_seg && P->seg_ent)
-    return launch_point_seg32(P->groups, P->n_groups, P->block_off_dev, P->seg_ent, P->seg_ang, P->seg_kept,
-                              P->slot_pix, P->seg_sub, u, u_stride, nrhs, done, done_stride, y4, y_stride, s);
-  return launch_point_sorted(P->groups, P->n_groups, P->win_size, P->block_off_dev, P->srt_ent,
-                             P->srt_ang, P->srt_slot, P->slot_pix, u, u_stride, nrhs, done, done_stride, y4,
-                             y_stride, s);
+    e = launch_point_seg32(P->groups, P->n_groups, P->block_off_dev, P->seg_ent, P->seg_ang, P->seg_kept,
+                           P->slot_pix, P->seg_sub, u, u_stride, nrhs, done, done_stride, y4, y_stride, maps, s);
+  else
+    e = launch_point_sorted(P->groups, P->n_groups, P->win_size, P->block_off_dev, P->srt_ent, P->srt_ang,
+                            P->srt_slot, P->slot_pix, u, u_stride, nrhs, done, done_stride, y4, y_stride, maps, s);
+  return e == cudaSuccess ? launch_sum_maps(maps, nrhs, done, done_stride, y4, y_stride, s) : e;
 }
 
 // y32 (accumulated, pre-zeroed) += A x32 in FP32, [nrhs][n_obs][4] float.  Profiling events: mid
@@ -1199,7 +1222,7 @@ int apply32_internal(Plan* P, const float* x32, float* y32, int nrhs, cudaStream
   }
   const int kc = split32_cols(P, nrhs);
   if (kc > 0 && P->groups) {
-    if (capturing(s) && P->u32_cap < (size_t)kc * t32_stride(P))
+    if (capturing(s) && (P->u32_cap < (size_t)kc * t32_stride(P) || P->ptmap_cap < ptmap_elems(P, kc)))
       return fail(MM_EINVAL, "FP32 buffers must be allocated before graph capture");
     MM_TRY(ensure_t32(P, nrhs));
     const int64_t ts = t32_stride(P);
@@ -1747,7 +1770,8 @@ int rebuild_launch(Server* S) {
       }
       wprobs.push_back(WinProb{P->block_off_dev, P->slot, P->slot_pix, P->ang2,
                                reinterpret_cast<const uint4*>(P->srt_ent), reinterpret_cast<const float4*>(P->srt_ang),
-                               P->srt_slot, r->cg->p32, P->t32, P->u32, r->cg->q32, halt});
+                               P->srt_slot, r->cg->p32, P->t32, P->u32, r->cg->q32, halt,
+                               PtMaps{P->ptmap, P->pt_maps}, P->n_obs});
       wsize.cover(P->win_size);
       const int sz = P->ninv_logm - kNinvLogMin;
       S->ntw32[sz] = P->ntw32;
@@ -1803,7 +1827,15 @@ int enqueue_multi_apply(Server* S, cudaStream_t s) {
       a.probs = S->nprobs_dev;
       MM_CUDA(launch_ninv32(kNinvLogMin + k, a, s));
     }
+    for (Request* r : S->running)
+      if (r->fp32 && r->plan->pt_maps > 1)
+        MM_CUDA(cudaMemsetAsync(r->plan->ptmap, 0, ptmap_elems(r->plan, 1) * sizeof(float), s));
     MM_CUDA(launch_point_sorted_multi(S->wgroups_dev, S->n_wgroups, S->wsize, S->wprobs_dev, s));
+    for (Request* r : S->running)
+      if (r->fp32 && r->plan->pt_maps > 1)
+        MM_CUDA(launch_sum_maps(PtMaps{r->plan->ptmap, r->plan->pt_maps}, 1,
+                                reinterpret_cast<const int32_t*>(r->cg->scal) + kHaltOffsetInts, kScalStrideInts,
+                                r->cg->q32, r->plan->n_obs * 4, s));
   }
   if (S->n_tiles > 0) {
     TileArgs a{};

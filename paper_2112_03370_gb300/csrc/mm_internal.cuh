@@ -116,6 +116,16 @@ struct WinSize {
   }
 };
 
+// Maps that P^T of the FP32 operators adds to: group g of a plan adds to map g mod n, the output map itself
+// (0) or one of the n - 1 maps at extra, which launch_sum_maps then adds to the output.  Each addition to
+// the map rounds to the ulp of the pixel's sum so far, and a pixel gets one per run of its samples, so the
+// error grows with the square root of their number; n keeps it near kPtAdds per map.
+constexpr int kPtAdds = 40, kPtMaps = 4;   // n: the least power of two, at most kPtMaps, that does
+struct PtMaps {
+  float* extra = nullptr;   // [n - 1][columns][n_obs][4]
+  int32_t n = 1;
+};
+
 // Per-problem pointers of the multi-problem window launches of a server step (every running
 // FP32 request's groups in one launch; group g belongs to problem groups[g].prob): its plan's
 // block offsets, slots, slot tables and reduced angles, the map x read by P, the un-pointed t it
@@ -133,6 +143,8 @@ struct WinProb {
   const float* u;    // [N]
   float* y;          // [n_obs][4]
   const int32_t* done;
+  PtMaps maps;
+  int64_t n_obs;
 };
 
 // Pixel-sorted sub-windows (P^T by segment reduction).  Sub-window s of a group is the window
@@ -257,6 +269,9 @@ struct Plan {
   float* srt_ang = nullptr;            // [n_srt][kSrtBlock] their angles
   uint16_t* srt_slot = nullptr;        // [n_srt][32] slot of each lane's first entry (kNoSlot: none)
   int64_t n_srt = 0;
+  int32_t pt_maps = 1;                 // maps that the groups add to (PtMaps)
+  float* ptmap = nullptr;              // [pt_maps - 1][columns][n_obs][4]: the maps after the first
+  size_t ptmap_cap = 0;
   int32_t tuned_width = 0;             // block width chosen by mm_autotune (0: not tuned)
 
   // tensor-core Toeplitz product (MM_TPLZ_GEMM plans)
@@ -455,14 +470,17 @@ cudaError_t launch_point_seg32(const PGroup* groups, int64_t n_groups, const int
                                const uint32_t* ent, const float* ent_ang, const int32_t* kept,
                                const int32_t* slot_pix, int sub_cap, const float* u, int64_t u_stride,
                                int nrhs, const int32_t* done, int done_stride, float* y4, int64_t y_stride,
-                               cudaStream_t s);
+                               const PtMaps& maps, cudaStream_t s);
 // y4 [nrhs][y_stride] += P^T u (FP32) by run sums over the sorted entries, u [nrhs][u_stride] (a
 // multiple of 4)
 cudaError_t launch_point_sorted(const PGroup* groups, int64_t n_groups, const WinSize& size,
                                 const int64_t* block_off, const uint16_t* ent, const float* ent_ang,
                                 const uint16_t* first_slot, const int32_t* slot_pix, const float* u,
                                 int64_t u_stride, int nrhs, const int32_t* done, int done_stride, float* y4,
-                                int64_t y_stride, cudaStream_t s);
+                                int64_t y_stride, const PtMaps& maps, cudaStream_t s);
+// y4 [nrhs][y_stride] += the n - 1 extra maps
+cudaError_t launch_sum_maps(const PtMaps& maps, int nrhs, const int32_t* done, int done_stride, float* y4,
+                            int64_t y_stride, cudaStream_t s);
 // the same two operators for several problems in one launch (continuous batching): groups from
 // every problem's plan, each with its prob index into probs (one column per problem)
 cudaError_t launch_unpoint_win32_multi(const PGroup* groups, int64_t n_groups, const WinSize& size, const WinProb* probs,
