@@ -1317,6 +1317,12 @@ int ensure_cg(Plan* P, int nrhs, bool fp32, CgState** out, cudaStream_t s) {
   return MM_OK;
 }
 
+// reliable_every rounded up to the iterations between two looks at the scalars, on which the replacements
+// fall.  Values near INT32_MAX (the natural way to ask for none) stay there.
+int32_t round_replacement(int32_t rel_every, int chunk) {
+  return (int32_t)std::min<int64_t>(((int64_t)rel_every + chunk - 1) / chunk * chunk, INT32_MAX);
+}
+
 CgWork make_work(Plan* P, CgState* c, int nrhs, bool fp32, double tol, int max_iter) {
   CgWork w{};
   w.n = P->n_obs;
@@ -1672,7 +1678,7 @@ int start_request(Server* S, Request* r, cudaStream_t ps) {
   r->w = make_work(P, r->cg, 1, r->fp32, r->opts.tol, r->opts.max_iter);
   const int rel_every = r->opts.reliable_every > 0 ? r->opts.reliable_every : 50;
   r->w.fused = 1;
-  r->w.rel_every = (rel_every + kServerCheck - 1) / kServerCheck * kServerCheck;
+  r->w.rel_every = round_replacement(rel_every, kServerCheck);
   MM_CUDA(cudaMallocHost((void**)&r->scal_host, sizeof(CgScalars)));
   MM_CUDA(launch_pack3to4(r->b_dev, P->n_obs, 1, r->cg->b, ps));
   MM_CUDA(launch_cg(CG_INIT, r->w, ps));
@@ -2255,7 +2261,7 @@ static int pcg_solve_impl(Plan* P, const double* b, const TodSrc* tod, double* x
   }
   // replacements fall on the host checks: rel_every rounded up to the iterations between them
   w.fused = !dwp && cg_step_fits(nrhs);
-  w.rel_every = (rel_every + chunk - 1) / chunk * chunk;
+  w.rel_every = round_replacement(rel_every, chunk);
 
   cudaEvent_t ev;
   MM_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
