@@ -1030,8 +1030,8 @@ def run_crossover(a):
     """N^-1 on the tensor cores (MM_TPLZ_GEMM: banded Toeplitz-block GEMMs, tcgen05, 3xTF32)
     against the overlap-save FFT tiles (MM_TPLZ_FFT), per half-bandwidth, on the ground geometry
     cut to --dets detectors: a profiled FP32 PCG of --iters iterations per algorithm, and the
-    N^-1 time per A-application from its per-launch events.  MM_TPLZ_AUTO takes the FFT at
-    every lambda.  Also the two maps after the same iterations (the algorithms
+    N^-1 time per A-application from its per-launch events.  On blocks this long MM_TPLZ_AUTO
+    takes the FFT at every lambda.  Also the two maps after the same iterations (the algorithms
     differ only by FP32 rounding)."""
     import numpy as np
     import torch
@@ -1081,7 +1081,7 @@ def run_crossover(a):
         "config": {"workload": f"ground geometry: {a.dets} det x 4 int x 524288 samples, FP32 operators, "
                                f"{a.iters} PCG iterations per algorithm", "n_samples": n_total},
         "rows": rows, "gemm_wins_up_to_lambda": max(wins) if wins else None,
-        "auto_rule": "MM_TPLZ_AUTO takes the FFT tiles at every lambda",
+        "auto_rule": "MM_TPLZ_AUTO takes the FFT tiles but for short blocks with lambda <= 64",
         "roofline": {"bound": "tensor", "kernel": "k_tplz_tc", "lambda": best["lambda"],
                      "achieved": best["gemm_tensor_tflops"], "peak": tf32_peak, "unit": "TFLOP/s",
                      "frac": best["gemm_tensor_frac"], "traffic": None,

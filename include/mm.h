@@ -66,7 +66,9 @@ enum { MM_FP64 = 0, MM_FP32 = 1, MM_DF64 = 2, MM_FP32_DF64 = 3 };
  *                   (tcgen05, 3xTF32, lambda <= 128, plans with FP32 operators); the FP64-class
  *                   operators keep the FFT tiles.
  *   MM_TPLZ_DIRECT  band sum by the definition (checks, tiny lambda).
- *   MM_TPLZ_AUTO    the algorithm that measured fastest: MM_TPLZ_FFT at every lambda. */
+ *   MM_TPLZ_AUTO    the FP32 operators' N^-1 by the form that is estimated faster from the block lengths:
+ *                   MM_TPLZ_GEMM for blocks of at most a few thousand samples with lambda <= 64,
+ *                   MM_TPLZ_FFT otherwise (and always in served requests). */
 enum { MM_TPLZ_AUTO = 0, MM_TPLZ_FFT = 1, MM_TPLZ_GEMM = 2, MM_TPLZ_DIRECT = 3 };
 /* Preconditioner: block-Jacobi, or the two-level a-posteriori A-DEF1 preconditioner built by
  * mm_deflation_build (Sect. 3.2, Eq. 2lvlDef). */

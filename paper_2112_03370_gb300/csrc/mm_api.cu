@@ -401,7 +401,7 @@ struct Scratch {
 // 8192 for lambda 1024, N 262144: 10 us, 32768: 18), so few tiles ask for small ones (one wave) and
 // many for the ones that keep the most outputs per unit of work.  shared: the tiles run in launches
 // together with other plans' (server), so the waves are not counted, only the work.
-int choose_ninv_logm(const std::vector<int64_t>& off, int lam, bool shared) {
+int choose_ninv_logm(const std::vector<int64_t>& off, int lam, bool shared, double* us_out = nullptr) {
   int best = kNinvLogMax;
   double best_t = 1e300;
   const double us[3] = {10.6, 11.5, 13.5};
@@ -418,7 +418,30 @@ int choose_ninv_logm(const std::vector<int64_t>& off, int lam, bool shared) {
       best = logm;
     }
   }
+  if (us_out) *us_out = best_t;
   return best;
+}
+
+// MM_TPLZ_AUTO: the tensor-core product where it is estimated to take less than the FFT tiles.  Its tiles
+// hold 4096 samples of one block, four CTAs per SM; a tile takes 5.7, 7.7 and 9.5 us for lambda 0, up to 32 and
+// up to 64, and 1.6 us more when it is full.  An FFT tile takes the same time for a short block as for a
+// full one, so short blocks go to the tensor cores.  A x, FFT and tensor cores, us: 4 x 2000 blocks of 100
+// samples, lambda 0, 16, 48: 192 and 124, 152, 176; 8 x 4096 of 256: 747 and 494, 591, 690; 16 x 512 of 1000: 222
+// and 167, 187, 218; 16 x 256 of 4096: 176 and 152, 165, 179; 8 x 128 of 8000: 89 and 93, 101, 116; 128 of 262,144:
+// 262 and 278, 310 (lambda 32), 338 (64).  Nearer than 9% the estimates do not tell the two apart (512 blocks of
+// 16,384, lambda 0: 89 and 94.5), and the FFT is kept, as above lambda 64, where it was never slower.
+bool auto_takes_tc(const std::vector<int64_t>& off, int lam) {
+  constexpr int64_t kSamples = 4096;
+  constexpr double kUs[3] = {5.7, 7.7, 9.5};
+  if (lam > 64) return false;
+  int64_t tiles = 0;
+  for (size_t b = 0; b + 1 < off.size(); b++) tiles += (off[b + 1] - off[b] + kSamples - 1) / kSamples;
+  if (tiles == 0) return false;
+  const int64_t slots = 4 * (int64_t)sm_count();
+  const double fill = (double)off.back() / (double)(tiles * kSamples);
+  double fft = 0.0;
+  choose_ninv_logm(off, lam, false, &fft);
+  return (double)((tiles + slots - 1) / slots) * (kUs[(lam + 31) / 32] + 1.6 * fill) < 0.91 * fft;
 }
 
 // Tile size of the FP64 and df64 tiles: the least estimated time over 4096- to 32768-sample tiles.  Their
@@ -668,10 +691,6 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
   // P->precision: arithmetic of the CG-iteration operators; P->df64: FP64-class ones in df64
   P->precision = (d->precision == MM_FP32 || d->precision == MM_FP32_DF64) ? MM_FP32 : MM_FP64;
   P->algo = (d->toeplitz_algo == MM_TPLZ_DIRECT) ? MM_TPLZ_DIRECT : MM_TPLZ_FFT;
-  // MM_TPLZ_AUTO takes the FFT tiles at every lambda: A x on 33.5M samples, FFT against GEMM: lambda 0
-  // 262 and 278 us, 32: 266 and 310, 64: 267 and 338, 128: 268 and 498; on 262,144 samples 40 to 42 us both
-  P->tc = P->precision == MM_FP32 && P->algo == MM_TPLZ_FFT && d->lambda <= kTcMaxJ0 * 32 &&
-          d->toeplitz_algo == MM_TPLZ_GEMM;
   P->df64 = (d->precision == MM_DF64 || d->precision == MM_FP32_DF64) && P->algo == MM_TPLZ_FFT;
   P->cond_max = d->cond_max > 0 ? d->cond_max : 1e3;
   P->use_seg = d->pt_sub > 0;
@@ -684,6 +703,9 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
   }
   P->N = P->block_off[nb];
   if (P->N <= 0) return fail(MM_EINVAL, "no samples");
+  P->tc = P->precision == MM_FP32 && P->algo == MM_TPLZ_FFT &&
+          (d->toeplitz_algo == MM_TPLZ_GEMM ||
+           (d->toeplitz_algo == MM_TPLZ_AUTO && auto_takes_tc(P->block_off, lam)));
   MM_CUDA(cudaStreamCreateWithFlags(&P->stream, cudaStreamNonBlocking));
   cudaStream_t s = P->stream;
   // order after the caller's stream (inputs may be produced there)
