@@ -560,7 +560,8 @@ int build_windows(Plan* P, cudaStream_t s) {
         maxlen = std::max(maxlen, off[b + 1] - off[b]);
       }
       int log_w = kMinLogW;
-      while (log_w < 30 && ((int64_t)nd << (log_w + 1)) <= kWinSamples) log_w++;
+      // no longer than the blocks: the rows that k_point_sorted stages take 2^log_w samples of shared memory
+      while (log_w < 30 && ((int64_t)1 << log_w) < maxlen && ((int64_t)nd << (log_w + 1)) <= kWinSamples) log_w++;
       for (int64_t w0 = 0; w0 < maxlen; w0 += (int64_t)1 << log_w) {
         PGroup g{};
         g.b0 = d0 * P->n_int + i;
