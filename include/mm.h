@@ -244,12 +244,12 @@ int mm_solve_tod(mm_plan_t plan, const void* d, int d_is_fp32, double* x, int nr
 
 /* Autotuner of the FP32 A-application (an interface of this library; the paper has none).  Times
  * the plan's own FP32 A x (CUDA events on the plan's stream, median of a few runs, inputs of the
- * plan's size) over candidate configurations and keeps the fastest:
- *   1. FP32 overlap-save tiles walked per segment (1, 2, 4, ..., 32; a CTA keeps the overlap of
- *      consecutive tiles in shared memory, more segments keep more SMs busy); for lambda > 6144,
+ * plan's size) over candidate configurations, the plan's own choice first, and keeps the fastest:
+ *   1. FP32 overlap-save tiles walked per segment (1, 2, 4, ..., 32; more tiles share a CTA's tables,
+ *      more segments keep more SMs busy); for lambda > 6144,
  *      also 65536-sample tiles split over 2-CTA clusters (more of each tile kept, but every CTA
  *      reads the whole tile);
- *   2. target samples per pixel-window group of P and P^T (2048 ... 16384);
+ *   2. target samples per pixel-window group of P and P^T (1024 ... 16384);
  *   2b. the P^T reduction: run sums over the sorted groups, or segment reduction
  *      over pixel-sorted sub-windows of at most 4096, 8192 or 16384 samples;
  *   3. block width for mm_block_cg_solve with block_width = 0: the widest of 1, 2, 4, ..., max_width

@@ -490,8 +490,10 @@ int build_segments(Plan* P, int steps, cudaStream_t s) {
     const int64_t len = (int64_t)2 << P->ninv_logm;
     const int64_t slots = (int64_t)sm_count() << (kNinvLogMax - P->ninv_logm);
     const int64_t n1 = (int64_t)make_tiles(P->block_off, bt, P->lambda, 1, 0, nullptr, len).size();
-    const int walk = P->steps_given ? std::max(1, steps) : (int)std::max<int64_t>(1, std::min<int64_t>(4, n1 / (8 * slots)));
-    P->nsegs_host = make_tiles(P->block_off, bt, P->lambda, walk, kL, nullptr, len);
+    P->n_ninv_tiles = n1;
+    P->ninv_walk_used =
+        P->ninv_walk > 0 ? P->ninv_walk : (int)std::max<int64_t>(1, std::min<int64_t>(4, n1 / (8 * slots)));
+    P->nsegs_host = make_tiles(P->block_off, bt, P->lambda, P->ninv_walk_used, kL, nullptr, len);
     if (P->nsegs) {
       P->bytes -= (size_t)P->n_nsegs * sizeof(TileDesc);
       dfree(P->nsegs);
@@ -519,6 +521,7 @@ int build_windows(Plan* P, cudaStream_t s) {
     kWinSamples = kWinMaxSamples;
     while (kWinSamples > 1024 && P->N / kWinSamples < 6 * sm_count()) kWinSamples /= 2;
   }
+  P->win_used = (int32_t)kWinSamples;
   P->win_size = WinSize{};
   P->win_size.threads = (int)std::min<int64_t>(kWinThreads, std::max<int64_t>(64, kWinSamples / 4));
   constexpr int kMinLogW = 5;
@@ -888,7 +891,7 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
     MM_CUDA(launch_pair_table_reg(P->ninv_logm, H, P->n_tab, costab_d, P->ntab32, s));
     MM_CUDA(launch_twiddle_image(P->ninv_logm, P->tw32, P->ntw32, s));
   }
-  P->steps_given = d->tile_steps > 0;
+  P->ninv_walk = d->tile_steps;
   // FP32 segments: enough of them to keep every SM busy (about 8 per SM), at most 16 tiles each
   const int64_t steps = d->tile_steps > 0 ? d->tile_steps
                                            : std::max<int64_t>(1, std::min<int64_t>(16, P->n_tiles32 / (8 * sm_count())));
@@ -2588,14 +2591,28 @@ int mm_autotune(mm_plan_t plan, int max_width, mm_tune_info* out, void* stream) 
     if (!*pass) out->n_rejected++;
     return MM_OK;
   };
-  // 1. tiles per segment: more tiles per CTA re-read less of the overlap, fewer leave SMs idle
-  const int steps_c[] = {1, 2, 4, 8, 16, 32};
+  // the plan's own choice is the first candidate of each step: what replaces it was faster
+  auto with_own = [](int own, std::initializer_list<int> others) {
+    std::vector<int> c{own};
+    for (int v : others)
+      if (v != own) c.push_back(v);
+    return c;
+  };
+  // 1. tiles per segment of the tiles that the plan runs (k_ninv32, or the fused ones): more tiles per CTA
+  // re-read less, fewer leave SMs idle
+  const bool reg = P->ninv_logm > 0;
+  const int64_t n_tiles = reg ? P->n_ninv_tiles : P->n_tiles32;
+  const int64_t slots = reg ? (int64_t)sm_count() << (kNinvLogMax - P->ninv_logm) : sm_count();
+  const int own_steps = reg ? P->ninv_walk_used : P->tile_steps;
+  auto segments_of = [&](int v) {
+    if (reg) P->ninv_walk = v;
+    return build_segments(P, reg ? P->tile_steps : v, P->stream);
+  };
   double best = 1e300;
-  int best_steps = P->tile_steps;
-  P->steps_given = true;
-  for (int v : steps_c) {
-    if (v > 1 && P->n_tiles32 / v < sm_count()) continue;   // fewer segments than SMs
-    MM_TRY(build_segments(P, v, P->stream));
+  int best_steps = own_steps;
+  for (int v : with_own(own_steps, {1, 2, 4, 8, 16, 32})) {
+    if (v > 1 && v != own_steps && n_tiles / v < slots) continue;   // fewer segments than run at once
+    MM_TRY(segments_of(v));
     double ms = 0.0;
     bool pass = false;
     MM_TRY(time_apply32(P, 1, kReps, &ms));
@@ -2607,7 +2624,7 @@ int mm_autotune(mm_plan_t plan, int max_width, mm_tune_info* out, void* stream) 
       best_steps = v;
     }
   }
-  MM_TRY(build_segments(P, best_steps, P->stream));
+  MM_TRY(segments_of(best_steps));
   // 1b. 65536-sample tiles over 2-CTA clusters (large lambda): kept when faster
   out->big_tiles = -1;
   if (P->big) {
@@ -2622,10 +2639,9 @@ int mm_autotune(mm_plan_t plan, int max_width, mm_tune_info* out, void* stream) 
     out->big_tiles = P->use_big ? 1 : 0;
   }
   // 2. samples per pixel-window group: larger groups repeat more pixels but stream shorter chunks
-  const int win_c[] = {2048, 4096, 8192, kWinMaxSamples};
   best = 1e300;
-  int best_win = P->win_samples;
-  for (int v : win_c) {
+  int best_win = P->win_used;
+  for (int v : with_own(P->win_used, {1024, 2048, 4096, 8192, kWinMaxSamples})) {
     P->win_samples = v;
     MM_TRY(build_windows(P, P->stream));
     double ms = 0.0;

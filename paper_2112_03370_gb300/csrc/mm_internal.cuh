@@ -261,9 +261,13 @@ struct Plan {
   std::vector<TileDesc> nsegs_host;    // host copy (multi-problem launches)
   float* ntab32 = nullptr;             // pair tables of every band table
   float2* ntw32 = nullptr;             // twiddle image
-  bool steps_given = false;            // the caller or the autotuner chose tile_steps
+  int32_t ninv_walk = 0;               // tiles that a CTA of k_ninv32 walks: the caller's or the autotuner's (0: from
+                                       // the plan's size), and the one in use
+  int32_t ninv_walk_used = 1;
+  int64_t n_ninv_tiles = 0;            // its tiles
   int32_t tile_steps = 0;              // FP32 tiles walked per segment
-  int32_t win_samples = 0;             // target samples per pixel-window group (0: from the plan's size)
+  int32_t win_samples = 0;             // target samples per pixel-window group (0: from the plan's size), and the
+  int32_t win_used = 0;                // one in use
   WinSize win_size;                    // largest group, for the launches of the window kernels
   uint16_t* srt_ent = nullptr;         // [n_srt][kSrtBlock] sorted entries (FP32 plans, interleaved)
   float* srt_ang = nullptr;            // [n_srt][kSrtBlock] their angles
