@@ -1028,7 +1028,10 @@ cudaError_t launch_tiles_fp64(int logm, int mode, const TileArgs& a, cudaStream_
 // c' = c with c_0 halved and W_n = exp(-2 pi i / n); A[t1][Q - m] = conj A[t1][m].  About 8M FP64
 // multiply-adds instead of lambda L / 2 (FP64 runs at 1/64 of the FP32 rate): lambda 3001 387 ->
 // 82 us, one table.
-constexpr int kSpecT1 = 128;
+// A frequency takes 256 of them at any lambda, so half-bandwidths below kSpecDirect sum by the definition
+// (whole plans of 1024 tables, definition and factorised: lambda 48 93.3 and 99.7 ms, 192 98.2 and 100.5, 256
+// 103.5 and 100.6), and the tables go kSpecBatch at a time through a scratch of 264 KB each.
+constexpr int kSpecT1 = 128, kSpecDirect = 224, kSpecBatch = 256;
 __device__ __forceinline__ double cos_of(const double* __restrict__ costab, int64_t i, int l) {
   return __ldg(costab + (i & (l - 1)));
 }
@@ -1071,20 +1074,41 @@ __global__ void k_spectra_h(const double2* __restrict__ A, const double* __restr
   H[(int64_t)blockIdx.y * (m_all + 1) + j] = 2.0 * acc;
 }
 
-size_t spectra_scratch(int32_t n_tab, int logm) {   // double2 values
-  return (size_t)n_tab * kSpecT1 * ((2 << logm) / kSpecT1 / 2 + 1);
+// the sum by its definition: lambda multiply-adds per frequency
+__global__ void k_spectra(const double* __restrict__ band_rows, int32_t lambda, const double* __restrict__ costab,
+                          double* __restrict__ H, int logm) {
+  __shared__ double c_s[kSpecDirect];
+  const int m_all = 1 << logm, l = 2 * m_all;
+  const double* c = band_rows + (int64_t)blockIdx.y * (lambda + 1);
+  for (int i = threadIdx.x; i <= lambda; i += blockDim.x) c_s[i] = c[i];
+  __syncthreads();
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j > m_all) return;
+  double acc = 0.0;
+  for (int tau = 1; tau <= lambda; tau++) acc = fma(c_s[tau], cos_of(costab, (int64_t)tau * j, l), acc);
+  H[(int64_t)blockIdx.y * (m_all + 1) + j] = c_s[0] + 2.0 * acc;
+}
+
+size_t spectra_scratch(int32_t n_tab, int32_t lambda, int logm) {   // double2 values
+  if (lambda < kSpecDirect) return 0;
+  return (size_t)std::min<int32_t>(n_tab, kSpecBatch) * kSpecT1 * ((2 << logm) / kSpecT1 / 2 + 1);
 }
 cudaError_t launch_spectra(const double* band_rows, int32_t n_tab, int32_t lambda, double* H,
                            const double* costab, double2* scratch, cudaStream_t s, int logm) {
   if (n_tab == 0) return cudaSuccess;
   const int m = 1 << logm;
-  const size_t per = spectra_scratch(1, logm);
-  for (int32_t t0 = 0; t0 < n_tab; t0 += 65535) {   // gridDim.y limit
-    const int32_t nt_y = (n_tab - t0) < 65535 ? (n_tab - t0) : 65535;
-    k_spectra_a<<<dim3(kSpecT1, nt_y), 128, 0, s>>>(band_rows + (int64_t)t0 * (lambda + 1), lambda, costab,
-                                                    scratch + (size_t)t0 * per, logm);
-    k_spectra_h<<<dim3((m + 128) / 128, nt_y), 128, 0, s>>>(scratch + (size_t)t0 * per, costab,
-                                                            H + (int64_t)t0 * (m + 1), logm);
+  const bool direct = lambda < kSpecDirect;
+  const int32_t step = direct ? 65535 : kSpecBatch;   // gridDim.y limit; tables in the scratch
+  for (int32_t t0 = 0; t0 < n_tab; t0 += step) {
+    const int32_t nt_y = std::min(n_tab - t0, step);
+    const double* rows = band_rows + (int64_t)t0 * (lambda + 1);
+    double* out = H + (int64_t)t0 * (m + 1);
+    if (direct) {
+      k_spectra<<<dim3((m + 256) / 256, nt_y), 256, 0, s>>>(rows, lambda, costab, out, logm);
+    } else {
+      k_spectra_a<<<dim3(kSpecT1, nt_y), 128, 0, s>>>(rows, lambda, costab, scratch, logm);
+      k_spectra_h<<<dim3((m + 128) / 128, nt_y), 128, 0, s>>>(scratch, costab, out, logm);
+    }
   }
   return cudaGetLastError();
 }

@@ -816,7 +816,7 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
   MM_CUDA(cudaMemcpyAsync(rows_d, rows.data(), rows.size() * sizeof(double), cudaMemcpyHostToDevice, s));
   MM_CUDA(cudaMemcpyAsync(costab_d, costab.data(), kL * sizeof(double), cudaMemcpyHostToDevice, s));
   double2* spec = nullptr;
-  MM_TRY(scr.alloc(&spec, spectra_scratch(P->n_tab)));
+  MM_TRY(scr.alloc(&spec, spectra_scratch(P->n_tab, lam)));
   MM_CUDA(launch_spectra(rows_d, P->n_tab, lam, H, costab_d, spec, s));
   MM_CUDA(launch_pair_tables(H, P->n_tab, costab_d, P->logm64, P->tab64, P->tab32, s));
   MM_CUDA(launch_twiddles(P->tw64, P->tw32, costab_d, s));
@@ -838,7 +838,7 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
     MM_TRY(dalloc(P, &P->tw32_big, mb));
     MM_CUDA(cudaMemcpyAsync(cb_d, cb.data(), lb * sizeof(double), cudaMemcpyHostToDevice, s));
     double2* spec_b = nullptr;
-    MM_TRY(scr.alloc(&spec_b, spectra_scratch(P->n_tab, kLogM + 1)));
+    MM_TRY(scr.alloc(&spec_b, spectra_scratch(P->n_tab, lam, kLogM + 1)));
     MM_CUDA(launch_spectra(rows_d, P->n_tab, lam, Hb, cb_d, spec_b, s, kLogM + 1));
     MM_CUDA(launch_pair_table32_big(Hb, P->n_tab, cb_d, P->tab32_big, s));
     MM_CUDA(launch_twiddles(nullptr, P->tw32_big, cb_d, s, kLogM + 1));

@@ -401,8 +401,8 @@ cudaError_t launch_weights(const float* psi, int64_t N, double2* w64, float2* w3
 cudaError_t launch_validate(const int32_t* pix, const float* psi, int64_t N, int64_t n_pix,
                             int32_t* bad, cudaStream_t s);
 // spectra of the L-point circulants, L = 2^(logm + 1): H [n_tab][M + 1], costab [L], scratch
-// [spectra_scratch(n_tab, logm)]
-size_t spectra_scratch(int32_t n_tab, int logm = kLogM);
+// [spectra_scratch(n_tab, lambda, logm)]
+size_t spectra_scratch(int32_t n_tab, int32_t lambda, int logm = kLogM);
 cudaError_t launch_spectra(const double* band_rows, int32_t n_tab, int32_t lambda,
                            double* H /* [n_tab][M+1] */, const double* costab /* [L] */,
                            double2* scratch, cudaStream_t s, int logm = kLogM);
