@@ -338,13 +338,16 @@ __device__ const double2 kSinCosPi32[64] = {
 // (cos x, sin x), x = 2 psi, in FP64 by table lookup and angle addition (the table-driven method of
 // P. T. P. Tang, ACM TOMS 1989-91): x = k pi/32 + r with k = rint(32 x / pi) and r = x - k pi/32 by a
 // two-constant Cody-Waite reduction (pi/32 = H + L, H = fl64(pi/32); k H is taken exactly inside one FMA);
-//   cos x = C_k cos r - S_k sin r,  sin x = S_k cos r + C_k sin r,  (C_k, S_k) = table[k mod 64].
+//   cos x = C_k + (C_k (cos r - 1) - S_k sin r),  sin x = S_k + (S_k (cos r - 1) + C_k sin r),
+// (C_k, S_k) = table[k mod 64]: what is added to the table's value is below 0.05, so only its rounding and the
+// last addition's are of the result's size.
 // GB300 runs FP64, and conversions to and from it, at 1/64 of the FP32 rate.  FP64 is kept where the result's
-// 53 bits are formed (the reduction, r + (sin r - r), 1 + (cos r - 1) and the four products); the small parts
+// 53 bits are formed (the reduction, r + (sin r - r), the products and sums above); the small parts
 // sin r - r and cos r - 1 (below 2e-5 and 1.3e-3 for |r| <= pi/64 and a little) come from double-float
-// Taylor series on the FP32 pipes, 48 bits of them being below 2^-57 absolute.  Within 1.6e-16 of the exact
-// values, 5.7e-17 rms, in a CPU check against 113-bit arithmetic over |psi| < 16384 (with the series in FP64:
-// 1.5e-16, 5.7e-17 rms).  16.8M samples, all outputs: 1.06 ms with the series in FP64 -> 0.42 ms.
+// Taylor series on the FP32 pipes, 48 bits of them being below 2^-57 absolute.  Within 1.2e-16 of the exact
+// values, 3.8e-17 rms, in a CPU check against 113-bit arithmetic over |psi| < 16384 (C_k cos r - S_k sin r with the
+// series in FP64: 1.54e-16, 4.4e-17 rms; with these series 1.63e-16).  16.8M samples, all outputs: 1.06 ms with
+// the series in FP64 -> 0.42 ms.
 __device__ __forceinline__ void sincos_x2(float psi, double& sn, double& cs) {
   const float x = 2.f * psi;   // exact
   if (!(fabsf(x) < 32768.f)) {   // outside any angle a scan produces: the general routine
@@ -366,10 +369,10 @@ __device__ __forceinline__ void sincos_x2(float psi, double& sn, double& cs) {
   // cos r - 1 = z (-1/2 + z (1/24 + z (-1/720 + z / 40320)))
   const df cp = df(1.0 / 24.0) + df_make(zh * __fmaf_rn(zh, 2.4801587e-5f, -1.3888889e-3f), 0.f);
   const df dcs = z * (df(-0.5) + z * cp);
-  const double sr = r + df_to_double(dsn), cr = 1.0 + df_to_double(dcs);
+  const double sr = r + df_to_double(dsn), dc = df_to_double(dcs);
   const double2 t = kSinCosPi32[(int)kf & 63];
-  cs = fma(t.x, cr, -t.y * sr);
-  sn = fma(t.y, cr, t.x * sr);
+  cs = t.x + fma(t.x, dc, -t.y * sr);
+  sn = t.y + fma(t.y, dc, t.x * sr);
 }
 
 // One evaluation of (cos 2 psi, sin 2 psi) per sample: the FP64 weights, their FP32 roundings, (wdf non-null)
