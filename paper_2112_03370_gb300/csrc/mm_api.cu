@@ -1288,6 +1288,24 @@ int apply32_internal(Plan* P, const float* x32, float* y32, int nrhs, cudaStream
   return MM_OK;
 }
 
+// kernels that apply32_internal and apply64_internal launch for nrhs columns (n_kernels of a solve)
+int kernels_point32(const Plan* P) { return P->pt_maps > 1 ? 2 : 1; }
+int kernels_apply32(const Plan* P, int nrhs) {
+  if (P->tmpl) return 2;
+  const int kc = split32_cols(P, nrhs);
+  if (kc > 0 && P->groups) return (nrhs + kc - 1) / kc * (2 + kernels_point32(P));
+  return kc >= nrhs ? 2 : 1;
+}
+int kernels_apply64(const Plan* P, int nrhs) {
+  if (P->tmpl) return 3;
+  if (P->df64) return (nrhs + df_cols(P, nrhs) - 1) / df_cols(P, nrhs) * (P->groups ? 4 : 3);
+  return P->algo == MM_TPLZ_DIRECT ? 3 * nrhs : 1;
+}
+int kernels_rhs32(const Plan* P, int nrhs) {
+  const int kc = split32_cols(P, nrhs);
+  return kc > 0 ? (nrhs + kc - 1) / kc * (2 + kernels_point32(P)) + 1 : 0;
+}
+
 // b4 [nrhs][n_obs][4] (FP64) = P^T N^-1 G d with the FP32 operators over the pixel windows (the
 // start of a solve whose true residuals come from the TOD); needs an FP32 plan with windows
 int rhs32_internal(Plan* P, const void* d, int d_is_fp32, int nrhs, double* b4, cudaStream_t s) {
@@ -1471,6 +1489,7 @@ int blk_apply(Plan* P, BlkState* b, int t, bool fp32, cudaStream_t s) {
   MM_CUDA(launch_to32(b->T64, (int64_t)(n4 / 4), b->AZ, s));
   return MM_OK;
 }
+int kernels_blk_apply(const Plan* P, int t, bool fp32) { return fp32 ? kernels_apply32(P, t) : 2 + kernels_apply64(P, t); }
 
 
 // ---------------------------------------------------------------------------------------------
@@ -2333,12 +2352,12 @@ static int pcg_solve_impl(Plan* P, const double* b, const TodSrc* tod, double* x
     c->g_buf_gen = P->buf_gen;
   }
 
-  // kernels of an iteration: its A-application counted as one (three per column on the direct path),
-  // and p, <p, q> and the updates in three launches or one
-  const int apply_kernels = (fp32 || P->algo != MM_TPLZ_DIRECT) ? 1 : 3 * nrhs, cg_kernels = w.fused ? 1 : 3;
+  // kernels of an iteration: its A-application, and p, <p, q> and the updates in three launches or one
+  const int apply_kernels = fp32 ? kernels_apply32(P, nrhs) : kernels_apply64(P, nrhs), cg_kernels = w.fused ? 1 : 3;
   std::vector<int> timed_out(nrhs, 0);
   const bool profile = opts->profile != 0;
-  int64_t n_kernels = w.fused ? 3 : 2;   // pack + init (+ the first p)
+  // the packed or formed right-hand side, init, the first p or the deflation
+  int64_t n_kernels = (tod ? kernels_rhs32(P, nrhs) : 1) + 1 + (w.fused ? 1 : 0) + (dwp ? 2 : 0);
   // profile mode: event pairs around every tile launch, summed at each host sync
   struct EvPair { cudaEvent_t a, b, m, m2; int is64; };
   std::vector<EvPair> pool, pending;
@@ -2396,7 +2415,7 @@ static int pcg_solve_impl(Plan* P, const double* b, const TodSrc* tod, double* x
     } else {
       n64++;
     }
-    n_kernels += (P->algo == MM_TPLZ_DIRECT) ? 3 * nrhs : 1;
+    n_kernels += kernels_apply64(P, nrhs);
     return MM_OK;
   };
   const int32_t* halt = reinterpret_cast<const int32_t*>(c->scal) + kHaltOffsetInts;
@@ -2798,7 +2817,7 @@ int mm_block_cg_solve(mm_plan_t plan, const double* b, double* x, int nrhs, int 
       MM_CUDA(cudaMemsetAsync(B->AX, 0, n4 * sizeof(double), s));
       MM_TRY(apply64_internal(P, B->X, B->AX, sg, s));
       MM_CUDA(launch_bresid(B->B, B->AX, sg, n, B->R, B->norm_part, blk_ctas(), B->norms, s));
-      n_kernels += 3;
+      n_kernels += 2 + kernels_apply64(P, sg);
       n_apply64 += 1;
       MM_TRY(read_norms(sg));
       active.clear();
@@ -2849,7 +2868,7 @@ int mm_block_cg_solve(mm_plan_t plan, const double* b, double* x, int nrhs, int 
       fresh = false;
       MM_CUDA(cudaStreamSynchronize(s));
       r = B->host_i[0];
-      n_kernels += 1 + (ortho ? 3 : 0) + (fp32 ? 1 : 3) + 3;
+      n_kernels += 1 + (ortho ? 3 : 0) + kernels_blk_apply(P, t, fp32) + 3;
       n_apply += 1;
       if (r == 0) {
         // every direction dropped: on the FP32 path away from a restart this is operator noise
@@ -3011,7 +3030,7 @@ int mm_ecg_solve(mm_plan_t plan, const double* b, double* x, int t, int variant,
       }
       MM_CUDA(cudaStreamSynchronize(s));
       const int r = B->host_i[0];
-      n_kernels += (fp32 ? 2 : 3) + 3;
+      n_kernels += kernels_blk_apply(P, tz, fp32) + 3;
       n_apply += 1;
       if (r == 0) {
         // every direction dropped: on the FP32 path after the first step of a recurrence this is
@@ -3097,7 +3116,7 @@ int mm_ecg_solve(mm_plan_t plan, const double* b, double* x, int t, int variant,
     MM_CUDA(cudaMemsetAsync(B->ax, 0, (size_t)n * 4 * sizeof(double), s));
     MM_TRY(apply64_internal(P, B->xe, B->ax, 1, s));
     MM_CUDA(launch_bresid(B->B, B->ax, 1, n, B->re, B->norm_part, blk_ctas(), B->norms, s));
-    n_kernels += 5;
+    n_kernels += 4 + kernels_apply64(P, 1);
     n_apply64 += 1;
     MM_TRY(read_host(B->norms, 1));
     tn2 = B->host[0];
