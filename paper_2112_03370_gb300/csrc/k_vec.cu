@@ -2,6 +2,8 @@
 // its definition, block-Jacobi apply, layout conversions and the fused CG kernels of Algorithm 1.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "df64.cuh"
 #include "mm_internal.cuh"
 #include "mm_cg.cuh"
@@ -838,7 +840,8 @@ static int step_capacity() {
   }();
   return per_sm * sm_count();
 }
-bool cg_step_fits(int columns) { return columns > 0 && columns <= step_capacity<512>() && columns <= step_capacity<128>(); }
+int cg_step_columns() { return std::min(step_capacity<512>(), step_capacity<128>()); }
+bool cg_step_fits(int columns) { return columns > 0 && columns <= cg_step_columns(); }
 
 template <int NT>
 static cudaError_t launch_step(const CgWork* w, const CgWork* list, int cols, int64_t n_max, cudaStream_t s) {

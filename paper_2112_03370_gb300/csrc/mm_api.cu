@@ -1611,11 +1611,12 @@ struct Request {
 };
 
 constexpr int kServerCheck = 4;    // iterations between the server's looks at the requests' scalars
-constexpr int kStepBatch = 64;     // requests whose CG steps share a launch
+constexpr int kStepBatch = 64;     // most requests whose CG steps share a launch
 
 struct Server {
   size_t budget = 0;
   int max_slots = 1;
+  int step_batch = 1;              // kStepBatch, or what the device holds of k_cg_step at once
   int device = 0;
   cudaStream_t stream = nullptr;
   std::mutex mu;
@@ -1954,9 +1955,9 @@ void server_loop(Server* S) {
     cudaStream_t s = S->stream;
     bool ok = true;
     ok = ok && enqueue_multi_apply(S, s) == MM_OK;
-    // the rest of every FP32 request's iteration in one launch per kStepBatch requests
-    for (int k = 0; k < S->n_works; k += kStepBatch)
-      ok = ok && launch_cg_step(nullptr, S->works_dev + k, std::min(kStepBatch, S->n_works - k), S->works_n_max, s) ==
+    // the rest of every FP32 request's iteration in one launch per step_batch requests
+    for (int k = 0; k < S->n_works; k += S->step_batch)
+      ok = ok && launch_cg_step(nullptr, S->works_dev + k, std::min(S->step_batch, S->n_works - k), S->works_n_max, s) ==
                      cudaSuccess;
     for (Request* r : S->running) {
       if (!r->fp32) ok = ok && enqueue_iteration(r->plan, r->w, 1, false, s) == MM_OK;
@@ -3460,6 +3461,11 @@ int mm_server_create(size_t hbm_budget, int max_slots, mm_server_t* out) {
   }
   S->budget = hbm_budget;
   S->max_slots = max_slots;
+  S->step_batch = std::min(kStepBatch, cg_step_columns());
+  if (S->step_batch < 1) {
+    delete S;
+    return fail(MM_ECUDA, "the device cannot hold the iteration step of one request at once");
+  }
   const cudaError_t e = cudaStreamCreateWithFlags(&S->stream, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
     delete S;

@@ -63,6 +63,7 @@ cudaError_t launch_cg(CgKernel k, const CgWork& w, cudaStream_t s);
 // Refused (cudaErrorInvalidValue) when the columns do not fit the device at once; see cg_step_fits.
 cudaError_t launch_cg_step(const CgWork* w, const CgWork* list, int count, int64_t n_max, cudaStream_t s);
 bool cg_step_fits(int columns);
+int cg_step_columns();   // most columns of one launch on this device (0 when it cannot hold any)
 int cg_blocks_for(int64_t n);
 
 }  // namespace mm
