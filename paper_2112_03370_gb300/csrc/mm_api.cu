@@ -4,6 +4,7 @@
 #include <condition_variable>
 #include <deque>
 #include <memory>
+#include <new>
 #include <mutex>
 #include <thread>
 #include <cmath>
@@ -1530,7 +1531,8 @@ class HostPool {
     std::unique_ptr<unsigned char[]> p;
     size_t cap = 0;
   };
-  // the smallest kept buffer of at least n bytes that n fills by half or more, else a new one
+  // the smallest kept buffer of at least n bytes that n fills by half or more, else a new one (empty when
+  // the host has no memory for it)
   Buf take(size_t n) {
     {
       std::lock_guard<std::mutex> lock(mu_);
@@ -1545,8 +1547,8 @@ class HostPool {
       }
     }
     Buf b;
-    b.p.reset(new unsigned char[n]);
-    b.cap = n;
+    b.p.reset(new (std::nothrow) unsigned char[n]);
+    b.cap = b.p ? n : 0;
     return b;
   }
   // kept if it fits beside the others; the oldest make room
@@ -1576,9 +1578,11 @@ class HostPool {
 template <typename T>
 struct HostArray {
   HostPool::Buf b;
-  void copy_from(HostPool& pool, const T* src, size_t count) {
+  bool copy_from(HostPool& pool, const T* src, size_t count) {
     if (count) b = pool.take(count * sizeof(T));
+    if (count && !b.p) return false;
     par_copy(b.p.get(), src, count * sizeof(T));
+    return true;
   }
   T* data() { return reinterpret_cast<T*>(b.p.get()); }
   void release(HostPool& pool) { pool.give(std::move(b)); }
@@ -3498,12 +3502,16 @@ int mm_submit(mm_server_t server, const mm_problem_desc* desc, const void* d, in
     if (v < 0) { delete r; return fail(MM_EINVAL, "negative block length"); }
     N += v;
   }
-  r->pix.copy_from(S->host_pool, desc->pix, (size_t)N);
-  r->psi.copy_from(S->host_pool, desc->psi, (size_t)N);
-  r->band.assign(desc->band, desc->band + (size_t)nb * (desc->lambda + 1));
   r->d_is_fp32 = d_is_fp32 ? 1 : 0;
   const unsigned char* db = reinterpret_cast<const unsigned char*>(d);
-  r->d.copy_from(S->host_pool, db, (size_t)N * (d_is_fp32 ? sizeof(float) : sizeof(double)));
+  if (!r->pix.copy_from(S->host_pool, desc->pix, (size_t)N) || !r->psi.copy_from(S->host_pool, desc->psi, (size_t)N) ||
+      !r->d.copy_from(S->host_pool, db, (size_t)N * (d_is_fp32 ? sizeof(float) : sizeof(double)))) {
+    r->pix.release(S->host_pool);
+    r->psi.release(S->host_pool);
+    delete r;
+    return fail(MM_ENOMEM, "no host memory for the request's arrays");
+  }
+  r->band.assign(desc->band, desc->band + (size_t)nb * (desc->lambda + 1));
   r->fp32 = opts->precision == MM_FP32;
   r->opts = *opts;
   r->footprint = estimate_footprint(*r);
