@@ -849,13 +849,7 @@ static size_t smem64(int logm) {
   return logm == 13 ? smem64_of<13>() : logm == 12 ? smem64_of<12>() : smem64_of<11>();
 }
 
-int tile_kernels_init() {
-  static int done = 0;
-  static int status = MM_OK;
-  if (done) return status;
-  done = 1;
-  status = ninv32_init();
-  if (status != MM_OK) return status;
+static cudaError_t tile_attributes() {
   cudaError_t e = cudaSuccess;
 #define MM_SET(K, B)                                                                       \
   if (e == cudaSuccess) e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(B));
@@ -890,8 +884,13 @@ int tile_kernels_init() {
     // CTA count terms; allow it explicitly.
     e = cudaFuncSetAttribute((k_tile<double, 2, MODE_APPLY>), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   }
-  if (e != cudaSuccess) status = cuda_fail(e, "tile kernel attributes");
-  return status;
+  return e;
+}
+// Set once per process; threads that come meanwhile wait (their launches need the shared-memory limits).
+int tile_kernels_init() {
+  static const cudaError_t e = tile_attributes();
+  if (e != cudaSuccess) return cuda_fail(e, "tile kernel attributes");
+  return ninv32_init();
 }
 
 template <typename T, int CL, int MODE, bool MULTI = false, int LOGM = kLogM>
