@@ -92,8 +92,9 @@ enum { MM_PREC_BD = 0, MM_PREC_2LVL_POST = 1 };
  *   toeplitz_algo  MM_TPLZ_AUTO, MM_TPLZ_FFT, MM_TPLZ_GEMM or MM_TPLZ_DIRECT (above); MM_TPLZ_GEMM
  *                  needs lambda <= 128 and FP32 operators (MM_FP32 or MM_FP32_DF64), else MM_EINVAL.
  *   inputs_on_device  non-zero: pix, psi and band are device pointers; zero: host pointers.
- *   tile_steps     FP32 operators: overlap-save tiles walked by one CTA, which keeps the overlap
- *                  of consecutive tiles in shared memory (0 = chosen from the problem size).
+ *   tile_steps     FP32 operators: overlap-save tiles walked by one CTA (0 = chosen from the problem
+ *                  size): the tiles share its twiddle tables, and the fused tiles of plans without
+ *                  pixel windows also keep the overlap of consecutive tiles in shared memory.
  *   pt_sub         FP32 operators, the reduction of P^T: 0 = run sums over the pixel-sorted window
  *                  groups, added to the map run by run; 4096, 8192 or 16384 = segment reduction over
  *                  pixel-sorted sub-windows of at most that many samples into per-group sums in
@@ -446,7 +447,9 @@ int mm_server_create(size_t hbm_budget, int max_slots, mm_server_t* out);
  * copied (by up to 8 threads) before the call returns; d is the TOD [N], float64 (d_is_fp32 = 0) or float32
  * (d_is_fp32 = 1).  opts->precision is MM_FP32 or MM_FP64 (above); opts->precond must be MM_PREC_BD;
  * MM_TPLZ_DIRECT plans are refused.  Non-blocking; *id identifies the request.  MM_EINVAL on bad
- * input (validated again at admission: a request that fails there finishes with that status). */
+ * input (validated again at admission: a request that fails there finishes with that status), MM_ENOMEM
+ * when the host has no memory for the copies.  The buffers of finished requests serve the next ones:
+ * the server keeps at most 1 GiB of them until it is destroyed. */
 int mm_submit(mm_server_t server, const mm_problem_desc* desc, const void* d, int d_is_fp32,
               const mm_solve_opts* opts, mm_req_t* id);
 /* MM_EBUSY while the request is queued or running; MM_OK (info filled) once it has finished. */

@@ -515,8 +515,10 @@ int build_segments(Plan* P, int steps, cudaStream_t s) {
 // detectors halved, until every group fits; then each group's pixel-sorted slot table and every
 // sample's slot are written.
 int build_windows(Plan* P, cudaStream_t s) {
-  // samples per group: 16384 when that leaves every SM its three CTAs twice over, down to 1024 for
-  // small plans (262,144 samples: 256 groups instead of 8 of 32768, P 55 -> 5 us and P^T 86 -> 8 us)
+  // samples per group: 16384 while that makes six groups per SM (one wave of P's CTAs, six per SM, three of
+  // P^T's, two per SM), down to 1024 for smaller plans, where a group more per SM is worth more than the
+  // pixels that smaller groups repeat (A x of 262,144 samples by group size: 1024 to 4096 22 us, 8192 24, 16384 28;
+  // 1.05M samples: 1024 27, 2048 to 4096 25, 16384 31; P 55 -> 5 us and P^T 86 -> 8 us against 8 groups of 32768)
   int64_t kWinSamples = P->win_samples;
   if (kWinSamples <= 0) {
     kWinSamples = kWinMaxSamples;
