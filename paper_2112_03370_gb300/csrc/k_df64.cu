@@ -36,12 +36,11 @@ __device__ __forceinline__ float4 split4(double a, double b) {
   return make_float4(x.hi, x.lo, y.hi, y.lo);
 }
 
-// (cos 2psi, sin 2psi) in FP64, split into df64
-__global__ void k_weights_df(const float* __restrict__ psi, int64_t N, float4* __restrict__ w) {
+// the FP64 weights (cos 2psi, sin 2psi) split into df64
+__global__ void k_weights_df(const double2* __restrict__ w64, int64_t N, float4* __restrict__ w) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    double s, c;
-    sincos(2.0 * (double)psi[i], &s, &c);
-    w[i] = split4(c, s);
+    const double2 v = w64[i];
+    w[i] = split4(v.x, v.y);
   }
 }
 
@@ -151,9 +150,9 @@ unsigned grid_for(int64_t n, int per_block) {
 
 }  // namespace
 
-cudaError_t launch_weights_df(const float* psi, int64_t N, float4* wdf, cudaStream_t s) {
+cudaError_t launch_weights_df(const double2* w64, int64_t N, float4* wdf, cudaStream_t s) {
   if (N == 0) return cudaSuccess;
-  k_weights_df<<<8 * sm_count(), 256, 0, s>>>(psi, N, wdf);
+  k_weights_df<<<8 * sm_count(), 256, 0, s>>>(w64, N, wdf);
   return cudaGetLastError();
 }
 

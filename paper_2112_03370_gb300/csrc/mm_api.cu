@@ -199,7 +199,7 @@ void free_plan(Plan* P) {
   cudaGetDevice(&cur);
   cudaSetDevice(P->device);
   if (P->stream) cudaStreamSynchronize(P->stream);
-  dfree(P->lpix); dfree(P->psi); dfree(P->w32); dfree(P->w64); dfree(P->obs_to_global); dfree(P->minv);
+  dfree(P->lpix); dfree(P->w32); dfree(P->w64); dfree(P->obs_to_global); dfree(P->minv);
   dfree(P->band); dfree(P->block_off_dev); dfree(P->c0_blk); dfree(P->tab32); dfree(P->tab64);
   dfree(P->tw32); dfree(P->tw64); dfree(P->tiles); dfree(P->segs); dfree(P->nsegs); dfree(P->ntab32); dfree(P->ntw32); dfree(P->map32_in); dfree(P->map32_out);
   dfree(P->map64_in); dfree(P->map64_out); dfree(P->td_a); dfree(P->td_b); dfree(P->t32);
@@ -743,9 +743,10 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
   // inputs
   int32_t* pix = nullptr;
   MM_TRY(scr.alloc(&pix, P->N));
-  MM_TRY(dalloc(P, &P->psi, P->N));
+  float* psi = nullptr;   // only the weights are kept
+  MM_TRY(scr.alloc(&psi, P->N));
   MM_CUDA(cudaMemcpyAsync(pix, d->pix, P->N * sizeof(int32_t), kind, s));
-  MM_CUDA(cudaMemcpyAsync(P->psi, d->psi, P->N * sizeof(float), kind, s));
+  MM_CUDA(cudaMemcpyAsync(psi, d->psi, P->N * sizeof(float), kind, s));
   MM_TRY(dalloc(P, &P->block_off_dev, nb + 1));
   MM_TRY(dalloc(P, &P->c0_blk, nb));
   MM_TRY(dalloc(P, &P->band, (size_t)nb * (lam + 1)));
@@ -757,7 +758,7 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
   int32_t* flag = nullptr;
   MM_TRY(scr.alloc(&flag, 4));
   MM_CUDA(cudaMemsetAsync(flag, 0, 4 * sizeof(int32_t), s));
-  MM_CUDA(launch_validate(pix, P->psi, P->N, P->n_pix, flag, s));
+  MM_CUDA(launch_validate(pix, psi, P->N, P->n_pix, flag, s));
   int32_t hflag[4] = {0, 0, 0, 0};
   MM_CUDA(cudaMemcpyAsync(hflag, flag, sizeof(hflag), cudaMemcpyDeviceToHost, s));
   MM_CUDA(cudaStreamSynchronize(s));
@@ -783,7 +784,7 @@ int build_plan(const mm_problem_desc* d, cudaStream_t us, Plan* P) {
   if (P->df64) MM_TRY(dalloc(P, &P->wdf, P->N));
   const bool windows = (P->precision == MM_FP32 || P->df64) && P->algo == MM_TPLZ_FFT && !P->no_windows;
   if (windows && P->precision == MM_FP32) MM_TRY(dalloc(P, &P->ang2, P->N + 3));   // quads read past the end
-  MM_CUDA(launch_weights(P->psi, P->N, P->w64, P->w32, P->df64 ? P->wdf : nullptr, P->ang2, s));
+  MM_CUDA(launch_weights(psi, P->N, P->w64, P->w32, P->df64 ? P->wdf : nullptr, P->ang2, s));
   MM_CUDA(launch_bd_accum(pix, P->w64, P->block_off_dev, P->c0_blk, nb, P->N, B6, hits, s));
   MM_CUDA(launch_bd_finalize(B6, hits, P->n_pix, P->cond_max, keep, inv6, s));
   MM_CUDA(launch_scan_keep(keep, P->n_pix, lid, flag + 1, scan_scratch, (int64_t)sl, s));
@@ -3371,7 +3372,7 @@ int mm_templates_set(mm_plan_t plan, const mm_templates_desc* t, void* stream) {
   }
   if (!P->wdf) {   // df64 pointing weights of the FP64-class template operator
     MM_TRY(dalloc(P, &P->wdf, P->N));
-    MM_CUDA(launch_weights_df(P->psi, P->N, P->wdf, s));
+    MM_CUDA(launch_weights_df(P->w64, P->N, P->wdf, s));
   }
   // Legendre abscissa scale 2 / (n - 1) and the orthonormal rescaling sqrt((2k + 1) / n) per block
   std::vector<double> xs(nb), xo(nb), ps((size_t)nb * std::max(t->n_poly, 1));

@@ -219,7 +219,6 @@ struct Plan {
 
   // device state
   int32_t* lpix = nullptr;             // [N]
-  float* psi = nullptr;                // [N]
   float2* w32 = nullptr;               // [N] cos 2psi, sin 2psi in FP32 (FP32 operators)
   double2* w64 = nullptr;              // [N] cos 2psi, sin 2psi in FP64 (FP64 operators)
   bool df64 = false;                   // FP64-class operators run in df64 arithmetic
@@ -497,7 +496,7 @@ int sm_count();
 cudaError_t launch_tiles_df(int logm, const TileArgs& a, cudaStream_t s);
 // df64 u = N^-1 t (pairs in, pairs out), per-column max |u| into a.amax
 cudaError_t launch_ninv_df(int logm, const TileArgs& a, cudaStream_t s);
-cudaError_t launch_weights_df(const float* psi, int64_t N, float4* wdf, cudaStream_t s);
+cudaError_t launch_weights_df(const double2* w64, int64_t N, float4* wdf, cudaStream_t s);
 cudaError_t launch_c64_to_df(const double2* in, int64_t n, float4* out, cudaStream_t s);
 cudaError_t launch_map_to_df(const double* m4, int64_t n_pix4, float4* out, cudaStream_t s);
 cudaError_t launch_unpoint_df(const int32_t* lpix, const float4* wdf, int64_t N, const float4* mapdf,
