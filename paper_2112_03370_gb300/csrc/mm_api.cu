@@ -1674,7 +1674,7 @@ struct Server {
 size_t estimate_footprint(const Request& r) {
   int64_t N = 0;
   for (int64_t v : r.block_len) N += v;
-  // pointing (pixel, angle, reduced angle, window slot, sorted entries), FP32, FP64 and df64 weights, un-pointed
+  // pointing (pixel, reduced angle, window slot, sorted entries), FP32, FP64 and df64 weights, un-pointed
   // FP32 and df64 buffers, N^-1 t in FP32 and df64 and the TOD: 100 bytes per sample
   return (size_t)N * 100 + (size_t)r.desc.n_pix * 480 + ((size_t)64 << 20);
 }
